@@ -328,6 +328,10 @@ int vcsgc_profile_steps(void* ctx, int64_t n, double* ms_propose, double* ms_com
  *           the period-q sublattice schedule, the five-shell BCC table, one
  *           density function and no surrogate; vcsgc_cluster_sizes lists
  *           the sizes these lattices allow.
+ * Until a shape is set, calls of 8 steps or more run a resident form chosen by
+ * size where one applies (form 1, or for the BLOCKS and OVERLAP schedules one
+ * block per replica with the whole lattice in shared memory); vcsgc_get_launch
+ * then reports the shape of the per-step launch that shorter calls use.
  * vcsgc_autotune picks a shape by timing; this call sets one explicitly.
  * Errors: INVALID_ARG (unknown form or shape), STATE (not the fused form,
  * or a form-1 size these lattices or this GPU do not allow). */

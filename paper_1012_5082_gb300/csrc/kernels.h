@@ -169,38 +169,59 @@ struct LatArgs {
   int da;
   MlpW mlp;
   int bcc5;                     // rows and masks equal the compile-time 5-shell BCC table
+  int bcc2;                     // the neighbourhood is the first two BCC shells (14 sites)
   int unpack4;                  // every replica's nx is even and its bytes 4-aligned: unpack 4 sites per thread
 };
 
 void launch_lattice_step(const LatArgs& a, int j, bool propose, cudaStream_t st);
 
-// ---- cluster-resident form of the fused step (kernels_cluster.cu)
+// ---- resident forms of the fused step (kernels_cluster.cu)
 // Tiling of one replica's rows over the CTAs of its cluster: TY x TZ tiles
 // (rank = tz TY + ty) of Ty rows by Tz planes (ny = TY Ty, nz = TZ Tz,
-// Ty, Tz >= 2); lcap: accepted-trial list capacity per step (>= the trials
-// of a CTA in a step).
+// Ty, Tz >= 2); lcap: most trials of one CTA in one step.
 struct ClTile {
   int TY, TZ, Ty, Tz, lcap;
 };
 constexpr int CL_TRIALS_PER_THREAD = 8;
-// dynamic shared memory of a tile: rows with halo, one pad word (a trial's
-// second window word may lie one past its row; its bits are never used),
-// the uniforms of a step's trials, two accept lists
+// dynamic shared memory of a tile: rows with halo, two pad words (a window's
+// second word may lie one past the last row; its bits are never used), two
+// bytes per trial group (lcap rounded to 16 each)
 inline size_t cluster_smem_bytes(const ClTile& t, int W) {
-  return sizeof(unsigned long long) * ((size_t)(t.Ty + 4) * (t.Tz + 4) * W + 1 + t.lcap) +
-         sizeof(int) * 2 * (size_t)t.lcap;
+  return sizeof(uint32_t) * ((size_t)(t.Ty + 4) * (t.Tz + 4) * W + 2) + 2 * (((size_t)t.lcap + 15) / 16 * 16);
+}
+// Draws of a chunk of steps (k_chain_draws): P entries per step, replica r's
+// from off[r] (pmax: most of one replica).
+struct ChainDraws {
+  float* lu;       // SUBLATTICE: -ln u per trial (rows padded to groups)
+  int2* su;        // else: site, -ln u
+  int2* cg;        // [step][R] colour or domains of the colour, -ln of the global uniform
+  const int* off;  // [R]
+  int P, pmax;
+};
+cudaError_t launch_chain_draws(const LatArgs& a, const ChainDraws& cd, long long base, int m, cudaStream_t st);
+// the footprint by which a size is offered as launch form 1: 64-bit words (32
+// species and 32 pending bits) and 16 bytes per trial
+inline size_t cluster_offer_bytes(const ClTile& t, int W) {
+  return 8 * ((size_t)(t.Ty + 4) * (t.Tz + 4) * W + 1 + t.lcap) + 8 * (size_t)t.lcap;
 }
 // largest dynamic shared memory a tile may use
 constexpr size_t CL_SMEM_MAX = 200 * 1024;
 // n colour steps from step `base` of every replica (R clusters of `csize`
-// CTAs of `block` threads, block 256 or 512); needs the five-shell table, the
-// sublattice schedule, a uniform dF and no pending commit.  Returns the
-// launch status.
-cudaError_t launch_cluster_steps(const LatArgs& a, const ClTile* d_tiles, size_t smem, int csize, int block,
-                                 long long base, int n, cudaStream_t st);
+// CTAs of `block` trial threads, block 256 or 512); needs the five-shell or
+// (period 4 along x) two-shell table, the sublattice schedule, a uniform dF
+// and no pending commit.  Returns the launch status.
+cudaError_t launch_cluster_steps(const LatArgs& a, const ClTile* d_tiles, const ChainDraws& cd, size_t smem, int csize,
+                                 int block, long long base, int n, cudaStream_t st);
 // clusters of csize CTAs with `smem` bytes each that can be resident at once
 // (0: the shape cannot launch)
-int cluster_capacity(int csize, int block, size_t smem);
+int cluster_capacity(const LatArgs& a, int csize, int block, size_t smem);
+// n colour steps from step `base` of a BLOCKS or OVERLAP schedule, one CTA of
+// `block` threads (a multiple of 32, at most 512) per replica, at most 8
+// trials per thread.  Needs a uniform dF and no pending commit.
+inline size_t pick_smem_bytes(long long words) { return sizeof(uint32_t) * ((size_t)words + 2); }
+constexpr size_t PICK_SMEM_MAX = 220 * 1024;
+cudaError_t launch_pick_steps(const LatArgs& a, const ChainDraws& cd, size_t smem, int block, long long base, int n,
+                              cudaStream_t st);
 // true when the rows and masks of a equal the compile-time five-shell table
 bool lattice_rows_bcc5(const LatArgs& a);
 // B count and energy of replicas r0 .. r0 + nrep - 1 from their packed

@@ -110,9 +110,11 @@ __device__ __forceinline__ bool lattice_accept(const LatArgs& a, const LatRep& l
 // (Eq. trans_vcsgc_par2), identical to the FP64 decision: Y is formed in FP32
 // with a bound on its rounding (beta kappa_p and n0 rounded to float, n <
 // 2^24 exact, two products and two sums), FP64 only when the screen cannot
-// settle it or |Y| is tiny.
-__device__ __forceinline__ bool global_accept(const LatRep& lr, const RepParams& p, int dn, long long n,
-                                              uint64_t ug53, int* tie) {
+// settle it or |Y| is tiny.  n: long long or (where it is known to fit) int,
+// whose conversion to float is not a 64-bit one.
+template <typename Int>
+__device__ __forceinline__ bool global_accept(const LatRep& lr, const RepParams& p, int dn, Int n, uint64_t ug53,
+                                              int* tie) {
   if (dn == 0) {
     if (ug53 >= U53_NEAR_ONE) *tie = 1;
     return true;

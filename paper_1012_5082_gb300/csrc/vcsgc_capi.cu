@@ -153,7 +153,16 @@ struct Ctx {
   ClTile* cl_tiles[5] = {};
   size_t cl_smem[5] = {};
   int cl_lcap[5] = {};             // most trials of one CTA in one step
-  long long base_lag = 0;          // steps run in form 1 not yet added to lat.ctl->base_step
+  long long base_lag = 0;          // steps run in a resident form not yet added to lat.ctl->base_step
+  // until a launch shape is set (vcsgc_set_launch, vcsgc_autotune): the
+  // resident form chosen by size (resident_shape)
+  bool shape_set = false;
+  int res_size = 0, res_block = 0;  // CTAs per cluster (0: none), trial threads
+  bool cl_offer[5] = {};            // sizes vcsgc_cluster_sizes lists (of cl_tiles)
+  int pick_block = 0;               // BLOCKS, OVERLAP: trial threads of the one-CTA form (0: none)
+  size_t pick_smem = 0;
+  ChainDraws draws{};               // draws of a chunk of steps of a resident form
+  long long draw_steps = 0;         // steps the buffers hold
   // SPATIAL schedule rebuilt on the device between MD phases: box -> domain
   // rank, and scratch of the counting sort
   int* sp_dom_of_block = nullptr;
@@ -346,6 +355,20 @@ void fill_args(Ctx* c) {
   l.rp = c->rp;
   l.rs = c->rs;
   l.err = c->derr;
+}
+
+// release the draw buffers (all: and the slices, for a new schedule)
+int drop_draws(Ctx* c, bool all) {
+  ChainDraws& d = c->draws;
+  if (d.cg) CK(cudaStreamSynchronize(c->st));
+  if (d.lu) cudaFree(d.lu);
+  if (d.su) cudaFree(d.su);
+  if (d.cg) cudaFree(d.cg);
+  d.lu = nullptr;
+  d.su = d.cg = nullptr;
+  c->draw_steps = 0;
+  if (all) d.P = 0;
+  return VCSGC_OK;
 }
 
 void drop_graph(Ctx* c) {
@@ -764,18 +787,73 @@ int sync_base(Ctx* c) {
 
 bool cluster_form_usable(const Ctx* c) {
   const int q = cl_index(c->cl_size);
-  return c->form == 1 && q >= 0 && c->cl_tiles[q] && !c->lat.da;
+  return c->form == 1 && q >= 0 && c->cl_offer[q] && !c->lat.da;
 }
 
-// n colour steps in the cluster-resident form: any pending commit of the
-// per-step form first, then one persistent launch per chunk of steps
-int run_steps_cluster(Ctx* c, long long n) {
+// Buffers of the resident forms' draws: 4 bytes per trial (8 with the picked
+// site) for as many steps as DRAW_BYTES hold, at most DRAW_STEPS (blockIdx.y,
+// and the kernels' integer sums), grown to what the longest call so far
+// uses.  One chunk of steps is one launch of draws and one of the chain.
+constexpr long long DRAW_BYTES = 64LL << 20, DRAW_STEPS = 4096;
+
+int draw_buffers(Ctx* c, long long n) {
+  LatArgs& l = c->lat;
+  ChainDraws& d = c->draws;
+  if (d.P == 0) {
+    // per-replica slices: rows of the colour padded to whole groups of four
+    std::vector<int> off(c->R);
+    long long P = 0;
+    int pmax = 0;
+    for (int r = 0; r < c->R; ++r) {
+      const LatGeom& g = c->h_geom[r];
+      const int gs = l.qx == 4 ? 4 : 1;
+      const int e = l.sublattice ? g.d / g.nxq * ((g.nxq + gs - 1) / gs * gs) : (g.dmax + 3) / 4 * 4;
+      off[r] = (int)P;
+      P += (e + 3) / 4 * 4;
+      pmax = std::max(pmax, e);
+    }
+    if (P > (1LL << 30)) return fail(c, VCSGC_ERR_NOMEM, "too many trials per colour step");
+    int* doff = nullptr;
+    TRY(dalloc(c, &doff, c->R));
+    CK(cudaMemcpyAsync(doff, off.data(), sizeof(int) * c->R, cudaMemcpyHostToDevice, c->st));
+    CK(cudaStreamSynchronize(c->st));
+    d.off = doff;
+    d.P = (int)P;
+    d.pmax = pmax;
+    c->draw_steps = 0;
+  }
+  const long long per = (long long)d.P * (l.sublattice ? 4 : 8);
+  const long long want = std::min({n, DRAW_STEPS, std::max(1LL, DRAW_BYTES / per)});
+  if (want <= c->draw_steps) return VCSGC_OK;
+  TRY(drop_draws(c, false));
+  void *q = nullptr, *g = nullptr;
+  if (cudaMalloc(&q, (size_t)(want * per)) != cudaSuccess ||
+      cudaMalloc(&g, sizeof(int2) * (size_t)(want * c->R)) != cudaSuccess) {
+    cudaGetLastError();
+    if (q) cudaFree(q);
+    return fail(c, VCSGC_ERR_NOMEM, "cudaMalloc: draws of the colour steps");
+  }
+  d.lu = l.sublattice ? static_cast<float*>(q) : nullptr;
+  d.su = l.sublattice ? nullptr : static_cast<int2*>(q);
+  d.cg = static_cast<int2*>(g);
+  c->draw_steps = want;
+  return VCSGC_OK;
+}
+
+// n colour steps in a resident form (csize 0: one CTA per replica with site
+// picks): any pending commit of the per-step form first, then one persistent
+// launch per chunk of steps
+int run_steps_resident(Ctx* c, long long n, int csize, int block) {
   TRY(flush(c));
-  const int q = cl_index(c->cl_size);
-  const long long chunk = 1LL << 20;
+  const int q = cl_index(csize);
+  TRY(draw_buffers(c, n));
   while (n > 0) {
-    const int m = (int)std::min(n, chunk);
-    CK(launch_cluster_steps(c->lat, c->cl_tiles[q], c->cl_smem[q], c->cl_size, c->cl_block, c->h_base, m, c->st));
+    const int m = (int)std::min(n, c->draw_steps);
+    CK(launch_chain_draws(c->lat, c->draws, c->h_base, m, c->st));
+    if (csize > 0)
+      CK(launch_cluster_steps(c->lat, c->cl_tiles[q], c->draws, c->cl_smem[q], csize, block, c->h_base, m, c->st));
+    else
+      CK(launch_pick_steps(c->lat, c->draws, c->pick_smem, block, c->h_base, m, c->st));
     c->h_base += m;
     c->base_lag += m;
     n -= m;
@@ -784,8 +862,15 @@ int run_steps_cluster(Ctx* c, long long n) {
   return VCSGC_OK;
 }
 
+// fewest steps of one call that pay for loading the lattice into shared memory
+constexpr long long RESIDENT_MIN_STEPS = 8;
+
 int run_steps_fast(Ctx* c, long long n) {
-  if (cluster_form_usable(c)) return run_steps_cluster(c, n);
+  if (cluster_form_usable(c)) return run_steps_resident(c, n, c->cl_size, c->cl_block);
+  if (!c->shape_set && !c->lat.da && n >= RESIDENT_MIN_STEPS) {
+    if (c->res_size) return run_steps_resident(c, n, c->res_size, c->res_block);
+    if (c->pick_block) return run_steps_resident(c, n, 0, c->pick_block);
+  }
   TRY(sync_base(c));
   const int G = 64;
   if (n >= G && !c->graph) {
@@ -1557,6 +1642,7 @@ static int lattice_shared(Ctx* c, int& unsupported) {
   l.bcc5 = lattice_rows_bcc5(l) ? 1 : 0;
   std::vector<int> zs(S, 0);
   for (int sh : c->offset_shell) zs[sh]++;
+  l.bcc2 = S == 2 && zs[0] == 8 && zs[1] == 6 ? 1 : 0;  // (+-1,+-1,+-1) and (+-2,0,0), ... by distance
   c->sum_absG = 0.0;
   for (int s = 0; s < S; ++s) c->sum_absG += zs[s] * std::fabs(l.G[s]);
   if (uni) {
@@ -1702,6 +1788,42 @@ static int lattice_state(Ctx* c, const std::vector<long long>& n0, const std::ve
   return check_device_error(c);
 }
 
+// The resident form a context runs until a launch shape is set, by size.
+// SUBLATTICE: the largest cluster size that gives every CTA an SM of its own
+// with all R clusters resident, down to 32 groups of trials per CTA.  A step
+// costs about 1.3 us of fixed work (two barriers, the decision, the chain of
+// one group) and 3.3 ns per group of four trials of a CTA; 80^3 x 8 replicas:
+// 8 CTAs 2.3, 4 CTAs 3.2, 2 CTAs 4.9 us per step, 16 CTAs 4.1 (7 clusters
+// resident, the eighth after them), the per-step launch 4.2.  64 replicas of
+// 24^3-48^3: 2 CTAs 3.9 us, 1 CTA 5.3, 8 CTAs 8.3, per-step 4.8.
+// BLOCKS and OVERLAP: one CTA per replica while its step holds at most 1024
+// trials and the lattice fits in shared memory (10^3 cells, 1 trial per step:
+// 0.9 us against 2.8 per launch; 40^3, 64 trials: 1.4 against 6.5).
+static void resident_shape(Ctx* c, const int* capacity) {
+  const LatArgs& l = c->lat;
+  c->res_size = c->res_block = c->pick_block = 0;
+  if (!l.df_uniform) return;
+  if (l.sublattice) {
+    int n_sm = 0;
+    if (cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, c->device) != cudaSuccess) cudaGetLastError();
+    const int gs = l.qx == 4 ? 4 : 1;
+    for (int qi = 0; qi < 5; ++qi) {
+      if (!c->cl_tiles[qi]) continue;
+      const int s = 1 << qi, groups = c->cl_lcap[qi] / gs;
+      if (s > 1 && (capacity[qi] < c->R || (long long)c->R * s > n_sm || groups < 32)) continue;
+      c->res_size = s;
+      c->res_block = groups > 256 ? 512 : 256;
+    }
+    return;
+  }
+  // site picks: the whole replica in one CTA
+  const size_t smem = pick_smem_bytes(c->max_words);
+  if (c->R >= 1 && c->subs.empty() && l.dmax <= 1024 && smem <= PICK_SMEM_MAX) {
+    c->pick_smem = smem;
+    c->pick_block = std::min(512, (l.dmax + 31) / 32 * 32);
+  }
+}
+
 // Tilings of the cluster-resident form.  For each cluster size s in 1, 2,
 // 4, 8, 16 every replica needs a TY x TZ = s grid of tiles dividing its
 // ny x nz rows with Ty, Tz >= 2, whose rows with halo, (Ty + 4)(Tz + 4) W
@@ -1712,12 +1834,16 @@ static int lattice_state(Ctx* c, const std::vector<long long>& n0, const std::ve
 // dropped.
 static int cluster_setup(Ctx* c) {
   const LatArgs& l = c->lat;
-  if (!l.sublattice || !l.bcc5 || !l.df_uniform || l.n_shells != 5) return VCSGC_OK;
+  int capacity[5] = {0, 0, 0, 0, 0};
+  if (!l.sublattice || !(l.bcc5 || (l.bcc2 && l.qx == 4)) || !l.df_uniform) {
+    resident_shape(c, capacity);
+    return VCSGC_OK;
+  }
   const int sizes[5] = {1, 2, 4, 8, 16};
   for (int qi = 0; qi < 5; ++qi) {
     const int s = sizes[qi];
     std::vector<ClTile> tiles;
-    size_t smem = 0;
+    size_t smem = 0, offer = 0;
     bool ok = true;
     for (int r = 0; r < c->R && ok; ++r) {
       const LatGeom& g = c->h_geom[r];
@@ -1745,13 +1871,17 @@ static int cluster_setup(Ctx* c) {
       if (!found) ok = false;
       tiles.push_back(best);
       smem = std::max(smem, cluster_smem_bytes(best, g.W));
+      offer = std::max(offer, cluster_offer_bytes(best, g.W));
       c->cl_lcap[qi] = std::max(c->cl_lcap[qi], best.lcap);
     }
-    if (!ok || cluster_capacity(s, 512, smem) < 1) continue;
+    if (!ok || cluster_capacity(l, s, 512, smem) < 1) continue;
+    capacity[qi] = cluster_capacity(l, s, 256, smem);
     TRY(dalloc(c, &c->cl_tiles[qi], tiles.size()));
     CK(cudaMemcpyAsync(c->cl_tiles[qi], tiles.data(), sizeof(ClTile) * tiles.size(), cudaMemcpyHostToDevice, c->st));
     c->cl_smem[qi] = smem;
+    c->cl_offer[qi] = l.bcc5 && offer <= CL_SMEM_MAX;
   }
+  resident_shape(c, capacity);
   return VCSGC_OK;
 }
 
@@ -1793,6 +1923,7 @@ static void destroy(Ctx* c) {
   c->subs.clear();
   drop_graph(c);
   if (c->st) cudaStreamSynchronize(c->st);
+  drop_draws(c, true);
   if (c->h_pin) cudaFreeHost(c->h_pin);
   for (void* p : c->allocs) cudaFree(p);
   if (c->own_stream && c->st) cudaStreamDestroy(c->st);
@@ -1977,7 +2108,7 @@ int vcsgc_autotune(void* ctx, int64_t steps, int32_t* best_block) {
   std::vector<std::array<int, 3>> cand = {{0, 64, 1}, {0, 128, 1}, {0, 256, 1}, {0, 64, 0}, {0, 128, 0}, {0, 256, 0}};
   if (!c->lat.da)
     for (int s : {1, 2, 4, 8, 16})
-      if (c->cl_tiles[cl_index(s)])
+      if (c->cl_offer[cl_index(s)])
         for (int b : {256, 512}) cand.push_back({1, b, s});
   float best = 0.0f;
   std::array<int, 3> bc = {0, 128, 1};
@@ -2077,9 +2208,11 @@ static int reschedule(Ctx* c, int kind, const int32_t sched[6]) {
   TRY(sync_base(c));
   launch_colour_table(l, c->st);
   CK(cudaGetLastError());
+  TRY(drop_draws(c, true));
   // cluster tilings exist for the sublattice schedule only
   for (int k = 0; k < 5; ++k) {
     c->cl_tiles[k] = nullptr;
+    c->cl_offer[k] = false;
     c->cl_smem[k] = 0;
     c->cl_lcap[k] = 0;
   }
@@ -2195,16 +2328,18 @@ int vcsgc_set_launch(void* ctx, int32_t form, int32_t block, int32_t variant) {
   if (!c->fast) return fail(c, VCSGC_ERR_STATE, "launch shape: the context is not in the fused form");
   if (f1) {
     const int q = cl_index(variant);
-    if (!c->cl_tiles[q] || c->cl_lcap[q] > block * CL_TRIALS_PER_THREAD ||
-        (block == 256 && cluster_capacity(variant, 256, c->cl_smem[q]) < 1))
+    if (!c->cl_offer[q] || c->cl_lcap[q] > block * CL_TRIALS_PER_THREAD ||
+        (block == 256 && cluster_capacity(c->lat, variant, 256, c->cl_smem[q]) < 1))
       return fail(c, VCSGC_ERR_STATE, "launch shape: no cluster-resident form of this size for these lattices");
     if (c->lat.da) return fail(c, VCSGC_ERR_STATE, "launch shape: the cluster-resident form has no delayed acceptance");
     c->form = 1;
     c->cl_size = variant;
     c->cl_block = block;
+    c->shape_set = true;
     return VCSGC_OK;
   }
   c->form = 0;
+  c->shape_set = true;
   c->lat.block = block;
   c->lat.prefetch = variant;
   select_blk(c);
@@ -2227,7 +2362,7 @@ int vcsgc_cluster_sizes(void* ctx, int32_t* mask) {
   if (!c || !mask) return VCSGC_ERR_INVALID_ARG;
   int m = 0;
   for (int q = 0; q < 5; ++q)
-    if (c->cl_tiles[q]) m |= 1 << q;
+    if (c->cl_offer[q]) m |= 1 << q;
   *mask = m;
   return VCSGC_OK;
 }
@@ -2983,7 +3118,7 @@ int vcsgc_profile_steps(void* ctx, int64_t n, double* ms_propose, double* ms_com
     CK(cudaEventCreate(&e1));
     TRY(flush(c));
     CK(cudaEventRecord(e0, c->st));
-    TRY(c->multi ? run_steps(c, n) : run_steps_cluster(c, n));
+    TRY(c->multi ? run_steps(c, n) : run_steps_resident(c, n, c->cl_size, c->cl_block));
     CK(cudaEventRecord(e1, c->st));
     CK(cudaEventSynchronize(e1));
     float ms = 0.f;
