@@ -82,6 +82,14 @@ void launch_fill_rf(const McArgs& a, int r, cudaStream_t st);
 // Block partial sums of the energy of replica r into part[0..nblocks).
 int energy_blocks(long long N);
 void launch_energy(const McArgs& a, bool shell, int r, double* part, cudaStream_t st);
+// five-shell BCC lattice: densities (rho null: not written) of replicas r0 ..
+// r0 + nrep - 1 from their species, and what their energies need (part[nrep][
+// shell_state_blocks], tot[nrep][6]; see k_shell_state); shell: 25 doubles of
+// launch_shell_values
+void launch_shell_values(const McArgs& a, double* out, cudaStream_t st);
+int shell_state_blocks(long long N);
+void launch_shell_state(const McArgs& a, const int n3[3], const double* shell, int r0, int nrep, double* rho,
+                        double* part, unsigned long long* tot, cudaStream_t st);
 
 // ---- fused colour step of the rigid lattice (kernels_lattice.cu)
 constexpr int LAT_BLOCK = 128;

@@ -307,6 +307,157 @@ __host__ __device__ constexpr int mk_shell0(int s) {
   return s == 0 ? 0 : (s == 1 ? 8 : (s == 2 ? 14 : (s == 3 ? 26 : (s == 4 ? 50 : MK_BCC5_N))));
 }
 
+// ------------------------------------------- re-embedding table (K = 2)
+// A neighbour's re-embedding change F_t(rho + f_b(r_s) - f_a(r_s)) - F_t(rho)
+// depends on the neighbour alone, and its density and species change only
+// with an accepted step (0.5 % of the trials flip on the re-embedding
+// workload).  So it is kept per site for both directions and every shell
+// (dtab), and a trial sums 58 floats it reads in order instead of looking up
+// 116 table cubics; the commit refreshes the entries of the sites a flip
+// touches, 12 evaluations each.
+//   An accepted step of 80^3 flips 900 sites, 640,000 evaluations, so they
+// avoid FP64 (55 us of an accepted step's commit) and still give the FP64
+// difference to about 10^-9 eV: the argument x / h is a 64-bit fixed-point
+// number (32 fraction bits; adding f_b - f_a is an integer addition), the
+// interval's value c0 is split in two floats whose high parts subtract
+// exactly, and the rest of the cubic is small (h F').  The screen's bound
+// falls from 1.3e-4 eV (FP32 cubics) to about 2e-6 eV, and with it the trials
+// that need FP64, each a chain of 3 us in its warp, from twenty a step to
+// less than one.
+struct EmbPoint {  // F_t at one argument: high part of c0, the rest
+  float hi, lo;
+};
+__device__ __forceinline__ long long emb_fix(const MultiArgs& a, double x) { return (long long)(x * a.embed[0].inv_h * 4294967296.0); }
+__device__ __forceinline__ bool emb_fix_in(const MultiArgs& a, long long u) { return u >= a.fix_lo && u <= a.fix_hi; }
+__device__ __forceinline__ EmbPoint emb_point(const MultiArgs& a, int t, long long u) {
+  int j = (int)(u >> 32);
+  j = j < 0 ? 0 : (j > a.emb_n - 1 ? a.emb_n - 1 : j);
+  const float x = __uint2float_rn((uint32_t)u) * 2.3283064365386963e-10f;
+  const float4 c = __ldg(a.emb_s + t * a.emb_n + j);
+  return EmbPoint{c.x, fmaf(x, fmaf(x, fmaf(x, c.w, c.z), c.y), __ldg(a.emb_lo0 + t * a.emb_n + j))};
+}
+__device__ __forceinline__ float emb_diff(const EmbPoint& p, const EmbPoint& q) { return (p.hi - q.hi) + (p.lo - q.lo); }
+// F_t(u1) - F_t(u0), NaN when an argument leaves the bounded range
+__device__ __forceinline__ float dtab_value(const MultiArgs& a, int t, long long u1, long long u0, const EmbPoint& p0) {
+  if (!emb_fix_in(a, u0) || !emb_fix_in(a, u1)) return __int_as_float(0x7FFFFFFF);
+  return emb_diff(emb_point(a, t, u1), p0);
+}
+
+// table entries of every site of replicas r0 ...
+__global__ void k_multi_table(MultiArgs a, int r0) {
+  const int r = r0 + blockIdx.y;
+  __shared__ long long s_df[5];
+  if (threadIdx.x < 5) s_df[threadIdx.x] = emb_fix(a, a.Fd[2 * threadIdx.x + 1] - a.Fd[2 * threadIdx.x]);
+  __syncthreads();
+  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= a.N) return;
+  const int3 h = multi_half(a, (int)i);
+  const int b = (int)(i & 1);
+  const long long q = multi_rfi(a, (h.x - b) >> 1, (h.y - b) >> 1, (h.z - b) >> 1, b);
+  const int t = a.types[(long long)r * a.N + i];
+  const long long u = emb_fix(a, a.rho[(long long)r * a.N + i]);
+  const EmbPoint p = emb_point(a, t, u);
+  float* D = a.dtab + (long long)r * DTAB_PLANES * a.rf_n + q;
+  for (int s = 0; s < 5; ++s) {
+    D[s * a.rf_n] = dtab_value(a, t, u + s_df[s], u, p);
+    D[(5 + s) * a.rf_n] = dtab_value(a, t, u - s_df[s], u, p);
+  }
+  D[10 * a.rf_n] = dtab_value(a, 1 - t, u, u, p);
+}
+
+void launch_multi_table(const MultiArgs& a, int r0, int nrep, cudaStream_t st) {
+  k_multi_table<<<dim3((unsigned)((a.N + 255) / 256), (unsigned)nrep), 256, 0, st>>>(a, r0);
+}
+
+// exact pair part (K = 2) of a trial from the B counts of its shells: with all
+// neighbours of species 0, and the change per B neighbour of each shell
+// (sP[6 ta ..])
+__device__ __forceinline__ void pq_table(const long long* Dq, int ta, long long* sP) {
+  constexpr int z[5] = {8, 6, 12, 24, 8};
+  long long base = 0;
+  for (int s = 0; s < 5; ++s) {
+    const long long* D = Dq + ((s * 2 + ta) * 2 + 1 - ta) * 2;
+    base += z[s] * D[0];
+    sP[6 * ta + 1 + s] = D[1] - D[0];
+  }
+  sP[6 * ta] = base;
+}
+__device__ __forceinline__ long long pq_from_counts(const long long* sP, uint32_t w, int ta) {
+  long long pq = sP[6 * ta];
+#pragma unroll
+  for (int s = 0; s < 5; ++s) pq += (long long)((w >> (6 * s)) & 63u) * sP[6 * ta + 1 + s];
+  return pq;
+}
+
+// bound on the distance of the table's FP32 dE from the FP64 dE: tab_err for
+// the cubics' roundings in the 58 entries and the own change (2^-20 max(|c1| +
+// 2 |c2| + 3 |c3|) each: coefficients, argument, Horner), two roundings of
+// each entry, their sum in four chains of at most 15 additions (18 roundings;
+// 24 2^-24 of sum |entries| in all), and the final sums
+__device__ __forceinline__ float table_err(const MultiArgs& a, float pair, float own, float re, float ab) {
+  return fmaf(1.430511474609375e-06f, ab,
+              fmaf(4.76837158203125e-07f, fabsf(pair) + fabsf(own) + fabsf(re), a.tab_err));
+}
+
+// one axis of the entries (bytes of a float plane) of cells c - 2 .. c + 2, c = p
+// + q k (q >= 4): class and place steps.  The class depends on the step alone,
+// the place is k - 1, k or k + 1 (wrapped).
+__device__ __forceinline__ void rf_axis(int p, int k, int q, int nk, uint32_t class_step, uint32_t place_step,
+                                        uint32_t (&o)[5]) {
+  const uint32_t k0 = (uint32_t)k * place_step;
+  const uint32_t km = k == 0 ? (uint32_t)(nk - 1) * place_step : k0 - place_step;
+  const uint32_t kp = k == nk - 1 ? 0u : k0 + place_step;
+#pragma unroll
+  for (int d = -2; d <= 2; ++d) {
+    const int m = p + d;
+    o[d + 2] = m < 0 ? (uint32_t)(m + q) * class_step + km
+                     : (m >= q ? (uint32_t)(m - q) * class_step + kp : (uint32_t)m * class_step + k0);
+  }
+}
+
+// FP32 dE of a basis-B trial (cell p + q k per axis) of species ta from the
+// table; offsets within a replica's planes fit 32 bits (host-checked)
+template <int B>
+__device__ __forceinline__ float multi_screen_table(const MultiArgs& a, const long long* sP, int r, const int* p, int kx,
+                                                    int ky, int kz, int ta, long long* pq_out, float* err, bool* in) {
+  uint32_t xo[5], yo[5], zo[5];
+  const uint32_t D4 = 4u * (uint32_t)a.D;
+  rf_axis(p[0], kx, a.qx, a.nxq, D4, 4u, xo);
+  rf_axis(p[1], ky, a.qy, a.nyq, D4 * a.qx, 4u * a.nxq, yo);
+  rf_axis(p[2], kz, a.qz, a.nzq, D4 * a.qx * a.qy, 4u * a.nyq * a.nxq, zo);
+  const uint32_t plane = 2u * (uint32_t)a.rf_n, n4 = 4u * (uint32_t)a.rf_n;  // basis 1; one shell
+  const char* T = reinterpret_cast<const char*>(a.dtab + (long long)r * DTAB_PLANES * a.rf_n);
+  const uint32_t self = zo[2] + yo[2] + xo[2] + (B ? plane : 0u);
+  const uint32_t w = __ldcg(reinterpret_cast<const uint32_t*>(reinterpret_cast<const char*>(a.nbc + (long long)r * a.rf_n) + self));
+  const float own = __ldcg(reinterpret_cast<const float*>(T + (size_t)(10u * n4 + self)));
+  const uint32_t base = ta ? 5u * n4 : 0u;
+#pragma unroll
+  for (int d = 0; d < 5; ++d) zo[d] += base;
+  float v[MK_BCC5_N];
+#pragma unroll
+  for (int k = 0; k < MK_BCC5_N; ++k) {
+    const int code = mk_bcc5_code(k);
+    const int hx = (code & 15) - 4, hy = ((code >> 4) & 15) - 4, hz = ((code >> 8) & 15) - 4, s = code >> 12;
+    const int bb = B ^ (hx & 1);
+    const uint32_t o = zo[((B + hz - bb) >> 1) + 2] + yo[((B + hy - bb) >> 1) + 2] + xo[((B + hx - bb) >> 1) + 2] +
+                       (bb ? plane : 0u) + s * n4;
+    v[k] = __ldcg(reinterpret_cast<const float*>(T + (size_t)o));
+  }
+  const long long pq = pq_from_counts(sP, w, ta);
+  float re[4] = {0.f, 0.f, 0.f, 0.f}, ab[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+  for (int k = 0; k < MK_BCC5_N; ++k) {
+    re[k & 3] += v[k];
+    ab[k & 3] += fabsf(v[k]);
+  }
+  const float re_ = (re[0] + re[1]) + (re[2] + re[3]), ab_ = (ab[0] + ab[1]) + (ab[2] + ab[3]);
+  const float pair = __ll2float_rn(pq) * a.qscale32;
+  *pq_out = pq;
+  *in = re_ + own == re_ + own;
+  *err = table_err(a, pair, own, re_, ab_);
+  return (pair + own) + re_;
+}
+
 constexpr int kScreenIlp = 12;  // 125 registers, no spills; 4, 8, 12 measured within 3 %
 
 __device__ float multi_screen_bcc5(const MultiArgs& a, const long long* sDq, const float* sDfs, int* sw,
@@ -318,17 +469,16 @@ __device__ float multi_screen_bcc5(const MultiArgs& a, const long long* sDq, con
   const int tid = threadIdx.x;
   // wrapped offsets of cells -2..2: species index (sw[0..14]) and the
   // per-site floats' index (sw[15..29]); rplane: the basis-1 half of the latter
-  const int rrow = a.qx * a.rf_q;
-  const int rplane = a.nz * a.ny * rrow;
+  const int rplane = rfi_plane(a);
 #pragma unroll
   for (int d = -2; d <= 2; ++d) {
-    const int X = mk_wrap(cx + d, a.nx), xq = X / a.qx;
+    const int X = mk_wrap(cx + d, a.nx);
     sw[(d + 2) * MK_BLOCK + tid] = 2 * X;
     sw[(d + 7) * MK_BLOCK + tid] = 2 * a.nx * mk_wrap(cy + d, a.ny);
     sw[(d + 12) * MK_BLOCK + tid] = 2 * a.nx * a.ny * mk_wrap(cz + d, a.nz);
-    sw[(d + 17) * MK_BLOCK + tid] = (X - xq * a.qx) * a.rf_q + xq;
-    sw[(d + 22) * MK_BLOCK + tid] = rrow * mk_wrap(cy + d, a.ny);
-    sw[(d + 27) * MK_BLOCK + tid] = rrow * a.ny * mk_wrap(cz + d, a.nz);
+    sw[(d + 17) * MK_BLOCK + tid] = rfi_x(a, X);
+    sw[(d + 22) * MK_BLOCK + tid] = rfi_y(a, mk_wrap(cy + d, a.ny));
+    sw[(d + 27) * MK_BLOCK + tid] = rfi_z(a, mk_wrap(cz + d, a.nz));
   }
   const float2 ri = rf[sw[17 * MK_BLOCK + tid] + sw[22 * MK_BLOCK + tid] + sw[27 * MK_BLOCK + tid] + (i & 1) * rplane];
   unsigned cnt[5];
@@ -384,24 +534,24 @@ __device__ float multi_screen_bcc5(const MultiArgs& a, const long long* sDq, con
 // called by all 32 lanes.
 constexpr int MK_GROUP = 8;
 
+template <bool TAB>
 __device__ float multi_screen_group(const MultiArgs& a, const long long* sDq, const float* sDfs, int* gw,
                                     const int* scode, int r, int i, int cx, int cy, int cz, int ta, int tb, int gl,
                                     bool has, long long* pq_out, float* err, bool* in) {
   const uint8_t* ty = a.types + (long long)r * a.N;
   const float2* rf = a.rf + (long long)r * a.rf_n;
   const int K = a.K;
-  const int rrow = a.qx * a.rf_q;
-  const int rplane = a.nz * a.ny * rrow;
+  const int rplane = rfi_plane(a);
   for (int q = gl; has && q < 5; q += MK_GROUP) {
     const int dd = q - 2;
-    const int X = mk_wrap(cx + dd, a.nx), xq = X / a.qx;
+    const int X = mk_wrap(cx + dd, a.nx);
     const int Y = mk_wrap(cy + dd, a.ny), Z = mk_wrap(cz + dd, a.nz);
     gw[q] = 2 * X;
     gw[5 + q] = 2 * a.nx * Y;
     gw[10 + q] = 2 * a.nx * a.ny * Z;
-    gw[15 + q] = (X - xq * a.qx) * a.rf_q + xq;
-    gw[20 + q] = rrow * Y;
-    gw[25 + q] = rrow * a.ny * Z;
+    gw[15 + q] = rfi_x(a, X);
+    gw[20 + q] = rfi_y(a, Y);
+    gw[25 + q] = rfi_z(a, Z);
   }
   __syncwarp();
   long long pq = 0;
@@ -416,22 +566,35 @@ __device__ float multi_screen_group(const MultiArgs& a, const long long* sDq, co
       if (k < MK_BCC5_N) {
         const int dc = scode[k];
         const int ix = dc & 7, iy = (dc >> 3) & 7, iz = (dc >> 6) & 7, bb = (dc >> 9) & 1, sh = dc >> 10;
-        const int j = gw[ix] + gw[5 + iy] + gw[10 + iz] + bb;
         const int jr = gw[15 + ix] + gw[20 + iy] + gw[25 + iz] + (bb ? rplane : 0);
-        const int t = ty[j];
-        const float2 v = rf[jr];
-        pq += Dq[sh * K * K * K + t];
-        const float x1 = v.x + Df[sh * K * K];
-        ok &= emb32_in(a, v.x) & emb32_in(a, x1);
-        const float d = emb32_val(a, t, x1) - v.y;
+        float d;
+        if constexpr (TAB) {
+          d = __ldcg(a.dtab + ((long long)r * DTAB_PLANES + 5 * ta + sh) * a.rf_n + jr);
+          ok &= d == d;
+        } else {
+          const int j = gw[ix] + gw[5 + iy] + gw[10 + iz] + bb;
+          const int t = ty[j];
+          const float2 v = rf[jr];
+          pq += Dq[sh * K * K * K + t];
+          const float x1 = v.x + Df[sh * K * K];
+          ok &= emb32_in(a, v.x) & emb32_in(a, x1);
+          d = emb32_val(a, t, x1) - v.y;
+        }
         re += d;
         ab += fabsf(d);
       }
     }
     if (gl == 0) {
-      const float2 ri = rf[gw[17] + gw[22] + gw[27] + (i & 1) * rplane];
-      ok &= emb32_in(a, ri.x);
-      own = emb32_val(a, tb, ri.x) - ri.y;
+      const int self = gw[17] + gw[22] + gw[27] + (i & 1) * rplane;
+      if constexpr (TAB) {
+        pq = pq_from_counts(sDq, __ldcg(a.nbc + (long long)r * a.rf_n + self), ta);  // sDq: pq_table
+        own = __ldcg(a.dtab + ((long long)r * DTAB_PLANES + 10) * a.rf_n + self);
+        ok &= own == own;
+      } else {
+        const float2 ri = rf[self];
+        ok &= emb32_in(a, ri.x);
+        own = emb32_val(a, tb, ri.x) - ri.y;
+      }
     }
   }
 #pragma unroll
@@ -447,8 +610,9 @@ __device__ float multi_screen_group(const MultiArgs& a, const long long* sDq, co
   const float pair = __ll2float_rn(pq) * a.qscale32;
   *pq_out = pq;
   *in = ok;
-  *err = fmaf((float)(2 * MK_BCC5_N + 2), a.emb_err,
-              fmaf(3.814697265625e-06f, ab, 4.76837158203125e-07f * (fabsf(pair) + fabsf(own) + fabsf(re))));
+  *err = TAB ? table_err(a, pair, own, re, ab)
+             : fmaf((float)(2 * MK_BCC5_N + 2), a.emb_err,
+                    fmaf(3.814697265625e-06f, ab, 4.76837158203125e-07f * (fabsf(pair) + fabsf(own) + fabsf(re))));
   return (pair + own) + re;
 }
 
@@ -569,22 +733,20 @@ __device__ __forceinline__ int multi_target(const MultiArgs& a, const MRepParams
 __device__ __forceinline__ void multi_descriptor(const MultiArgs& a, int r, int cx, int cy, int cz, int b, int ti,
                                                  int (&own)[5], int (&nb)[5]) {
   const uint32_t* nc = a.nbc + (long long)r * a.rf_n;
-  const long long row = (long long)a.qx * a.rf_q;
-  const int lo = b ? 0 : -1;
-  int xp[2], yv[2], zv[2];
+  const int lo = b ? 0 : -1, plane = rfi_plane(a);
+  int xp[2], yp[2], zp[2];
 #pragma unroll
   for (int q = 0; q < 2; ++q) {
-    const int X = mk_wrap(cx + lo + q, a.nx), xq = X / a.qx;
-    xp[q] = (X - xq * a.qx) * a.rf_q + xq;
-    yv[q] = mk_wrap(cy + lo + q, a.ny);
-    zv[q] = mk_wrap(cz + lo + q, a.nz);
+    xp[q] = rfi_x(a, mk_wrap(cx + lo + q, a.nx));
+    yp[q] = rfi_y(a, mk_wrap(cy + lo + q, a.ny));
+    zp[q] = rfi_z(a, mk_wrap(cz + lo + q, a.nz));
   }
-  const uint32_t w0 = nc[((long long)(b * a.nz + cz) * a.ny + cy) * row + (b ? xp[0] : xp[1])];
-  const int nbb = 1 - b;
+  const int me = b ? 0 : 1;  // the site's own cell among the two of each axis
+  const uint32_t w0 = nc[zp[me] + yp[me] + xp[me] + (b ? plane : 0)];
   uint32_t xs = 0u, ys = 0u;
 #pragma unroll
   for (int q = 0; q < 8; ++q) {
-    const uint32_t w = nc[((long long)(nbb * a.nz + zv[q >> 2]) * a.ny + yv[(q >> 1) & 1]) * row + xp[q & 1]];
+    const uint32_t w = nc[zp[q >> 2] + yp[(q >> 1) & 1] + xp[q & 1] + (b ? 0 : plane)];
     xs += w & 0x3F03F03Fu;
     ys += (w >> 6) & 0x0003F03Fu;
   }
@@ -604,7 +766,10 @@ __device__ __forceinline__ void multi_descriptor(const MultiArgs& a, int r, int 
 // state and the last block of each replica takes the global decision; the
 // screened modes take step *base + j and leave the decision to the commit
 // launch, whose every block reads the step's complete sums.
-template <int MODE>
+// TAB (mode 3): the re-embedding terms come from the table (dtab), whose
+// entries are not offset by species; mode 2 with the table is
+// k_multi_propose_table.
+template <int MODE, bool TAB = false>
 __global__ void __launch_bounds__(MK_BLOCK, 4) k_multi_propose(MultiArgs a, int j) {
   constexpr bool REEMBED = MODE != 0;
   constexpr bool SCREEN = MODE >= 2;
@@ -615,7 +780,7 @@ __global__ void __launch_bounds__(MK_BLOCK, 4) k_multi_propose(MultiArgs a, int 
   __shared__ float sDfs[5 * MK_MAX * MK_MAX];
   // screened form: per-thread wrapped cell offsets and the block's
   // neighbour descriptors (unused otherwise)
-  __shared__ int sw[SCREEN ? 30 * MK_BLOCK : 1];
+  __shared__ int sw[MODE == 2 ? 30 * MK_BLOCK : 1];
   __shared__ int scode[SCREEN ? MK_BCC5_N : 1];
   __shared__ int s_fw[SCREEN ? MK_BLOCK / 32 : 1][15];
   // delayed acceptance: the block's stage-1 passes, queued for the exact
@@ -627,6 +792,7 @@ __global__ void __launch_bounds__(MK_BLOCK, 4) k_multi_propose(MultiArgs a, int 
   __shared__ int s_gw[MODE == 3 ? MK_BLOCK / MK_GROUP : 1][30];
   __shared__ uint64_t s_u2[MODE == 3 ? MK_BLOCK : 1];
   __shared__ int s_nq;
+  __shared__ long long s_pq[TAB ? 12 : 1];
   __shared__ uint4 s_wc;
   __shared__ int s_col[4];
   __shared__ int s_red[MK_BLOCK / 32][MK_MAX + 1];
@@ -643,6 +809,7 @@ __global__ void __launch_bounds__(MK_BLOCK, 4) k_multi_propose(MultiArgs a, int 
   if (!REEMBED && threadIdx.x < K * K) sDF[threadIdx.x] = a.dF[threadIdx.x];
   if (a.bcc5)
     for (int q = threadIdx.x; q < 5 * K * K * K; q += MK_BLOCK) sDq[q] = a.Dq[q];
+  if (TAB && threadIdx.x < 2) pq_table(a.Dq, threadIdx.x, s_pq);
   if (SCREEN)
     for (int q = threadIdx.x; q < 5 * K * K; q += MK_BLOCK) {
       const int sh = q / (K * K), x = (q / K) % K, y = q % K;
@@ -687,12 +854,12 @@ __global__ void __launch_bounds__(MK_BLOCK, 4) k_multi_propose(MultiArgs a, int 
   // site of trial d (ascending index within the colour) and its draw: they
   // depend on no earlier launch
   const int b = c & 1;
-  int cx = 0, cy = 0, cz = 0;
+  int cx = 0, cy = 0, cz = 0, kx = 0, ky = 0, kz = 0;
   if (d < a.D) {
     const int dq = mk_div(d, a.nxq, a.rcp_nxq);
-    const int kx = d - dq * a.nxq;
-    const int kz = mk_div(dq, a.nyq, a.rcp_nyq);
-    const int ky = dq - kz * a.nyq;
+    kx = d - dq * a.nxq;
+    kz = mk_div(dq, a.nyq, a.rcp_nyq);
+    ky = dq - kz * a.nyq;
     cx = s_col[1] + a.qx * kx;
     cy = s_col[2] + a.qy * ky;
     cz = s_col[3] + a.qz * kz;
@@ -708,6 +875,7 @@ __global__ void __launch_bounds__(MK_BLOCK, 4) k_multi_propose(MultiArgs a, int 
       s_u2[threadIdx.x] = top53(w2.x, w2.y);
     }
   }
+  if constexpr (SCREEN) pdl_trigger();  // the commit of this step: its prologue
   // screened form: launched after the previous step's commit with
   // programmatic dependent launch; the species, densities and this step's
   // accumulators are read after the wait (a no-op for an ordinary launch)
@@ -764,7 +932,7 @@ __global__ void __launch_bounds__(MK_BLOCK, 4) k_multi_propose(MultiArgs a, int 
       long long qpq = 0;
       float err;
       bool in;
-      const float e32 = multi_screen_group(a, sDq, sDfs, s_gw[threadIdx.x / MK_GROUP], scode, r, qa.x, qa.y, qa.z,
+      const float e32 = multi_screen_group<TAB>(a, TAB ? s_pq : sDq, sDfs, s_gw[threadIdx.x / MK_GROUP], scode, r, qa.x, qa.y, qa.z,
                                            qa.w, qo.x, 1 - qo.x, gl, has, &qpq, &err, &in);
       const bool lead = has && gl == 0;
       int dec2 = 0;
@@ -774,7 +942,7 @@ __global__ void __launch_bounds__(MK_BLOCK, 4) k_multi_propose(MultiArgs a, int 
         const float g = __int_as_float(qo.y);
         // -s g (exact) plus the own-site offset of the FP32 tables: two
         // roundings, inside 2^-21 (|g| + |offset|)
-        const float off = a.emb_off[qo.x * K + 1 - qo.x];
+        const float off = TAB ? 0.0f : a.emb_off[qo.x * K + 1 - qo.x];
         const float cm = (qo.x ? g : -g) + off;
         const float x32 = p.beta32 * (e32 + cm);
         const float dx =
@@ -981,6 +1149,42 @@ __global__ void __launch_bounds__(MK_BLOCK) k_multi_commit(MultiArgs a) {
   }
 }
 
+__device__ __forceinline__ uint64_t step_uniform(const MRepParams& p, long long step) {
+  const uint4 w = philox4x32_10(make_uint4((uint32_t)step, (uint32_t)((uint64_t)step >> 32), 0xFFFFFFFFu, TAG_STEP),
+                                p.key);
+  return top53(w.z, w.w);
+}
+
+// Global stage: u_g < min{1, exp(-Y)}, Y = beta sum_alpha kappa_p dn (dn + 2 (n -
+// n0)), decided as FP64 does: Y in FP32 with a bound on its rounding (beta
+// kappa_p, n and n0 to float, products and sums: 2^-21 of the sizes), FP64
+// where the screen cannot settle it (its chain of dependent FP64 operations
+// was a third of an idle commit's time).
+__device__ __forceinline__ int multi_global(const MultiArgs& a, const MRepParams& p, const int (&dn)[MK_MAX],
+                                            const long long (&c0)[MK_MAX], uint64_t ug, int* tie) {
+  float y = 0.f, dy = 0.f;
+  bool any = false;
+#pragma unroll
+  for (int al = 1; al < MK_MAX; ++al)
+    if (al < a.K) {
+      const float fd = (float)dn[al], n = (float)(int)c0[al], n0 = p.n0_32[al], bk = p.bk32[al];
+      const float term = bk * fd * fmaf(2.0f, n - n0, fd);
+      y += term;
+      dy += fabsf(bk * fd) * (fabsf(fd) + 2.0f * (n + fabsf(n0))) * 9.5367431640625e-07f;
+      any |= dn[al] != 0;
+    }
+  if (any && fabsf(y) > 1e-6f) {
+    const int dec = screen32(y, dy, ug);
+    if (dec >= 0) return dec;
+  }
+  double Y = 0.0;
+#pragma unroll
+  for (int al = 1; al < MK_MAX; ++al)
+    if (al < a.K)
+      Y += p.beta * p.kappa_p[al] * (double)dn[al] * ((double)dn[al] + 2.0 * ((double)c0[al] - p.n0[al]));
+  return metropolis(Y, ug, tie) ? 1 : 0;
+}
+
 // Screened form: one thread per (accept, neighbour) and one per accepted
 // site over all replicas that accepted their step, on a fixed grid: the
 // density change in FP64 with its float copy and the FP32 embedding value
@@ -997,8 +1201,26 @@ __global__ void __launch_bounds__(MK_BLOCK) k_multi_commit_screen(MultiArgs a, i
   __shared__ int4 s_off[MK_BCC5_N];
   __shared__ double s_df[5 * MK_MAX * MK_MAX];
   const int K = a.K;
+  // items of an accept: its neighbours' densities, floats and counts, and its
+  // own species
   constexpr int NI = MK_BCC5_N + 1;
   const long long step = *a.base + jl;  // the step the propose launch proposed
+  for (int q = threadIdx.x; q < MK_BCC5_N; q += MK_BLOCK) s_off[q] = a.off[q];
+  for (int q = threadIdx.x; q < 5 * K * K; q += MK_BLOCK) {
+    const int sh = q / (K * K), x = (q / K) % K, y = q % K;
+    s_df[q] = a.Fd[sh * K + y] - a.Fd[sh * K + x];
+  }
+  __shared__ uint64_t s_ug[MK_BLOCK];
+  if (threadIdx.x < a.R) s_ug[threadIdx.x] = step_uniform(a.rp[threadIdx.x], step);
+  __shared__ long long s_fix[10];  // +-(f_1 - f_0)(r_s) / h in fixed point
+  if (a.dtab && threadIdx.x < 10) {
+    const int s = threadIdx.x % 5;
+    const long long f = emb_fix(a, a.Fd[2 * s + 1] - a.Fd[2 * s]);
+    s_fix[threadIdx.x] = threadIdx.x < 5 ? f : -f;
+  }
+  // launched while the propose launch still runs: its sums and list after
+  // the wait
+  pdl_wait();
   // the global stage of every replica (Eq. trans_vcsgc_par2 per solute),
   // taken in every block from the step's complete sums: the same FP64
   // arithmetic everywhere, so the same decision.  Block 0 folds the step
@@ -1016,14 +1238,8 @@ __global__ void __launch_bounds__(MK_BLOCK) k_multi_commit_screen(MultiArgs a, i
     }
     int accept = 0, gtie = 0;
     if (nacc > 0) {
-      double Y = 0.0;
-#pragma unroll
-      for (int al = 1; al < MK_MAX; ++al)
-        if (al < K)
-          Y += p.beta * p.kappa_p[al] * (double)dn[al] * ((double)dn[al] + 2.0 * ((double)c0[al] - p.n0[al]));
-      const uint4 wc = philox4x32_10(
-          make_uint4((uint32_t)step, (uint32_t)((uint64_t)step >> 32), 0xFFFFFFFFu, TAG_STEP), p.key);
-      accept = metropolis(Y, top53(wc.z, wc.w), &gtie) ? 1 : 0;
+      const uint64_t ug = s_ug[r < MK_BLOCK ? r : 0];
+      accept = multi_global(a, p, dn, c0, r < MK_BLOCK ? ug : step_uniform(p, step), &gtie);
     }
     s_pre[r + 1] = accept ? nacc * NI : 0;
     if (blockIdx.x == 0) {
@@ -1071,11 +1287,6 @@ __global__ void __launch_bounds__(MK_BLOCK) k_multi_commit_screen(MultiArgs a, i
       B->sum_de = 0.0;
     }
   }
-  for (int q = threadIdx.x; q < MK_BCC5_N; q += MK_BLOCK) s_off[q] = a.off[q];
-  for (int q = threadIdx.x; q < 5 * K * K; q += MK_BLOCK) {
-    const int sh = q / (K * K), x = (q / K) % K, y = q % K;
-    s_df[q] = a.Fd[sh * K + y] - a.Fd[sh * K + x];
-  }
   __syncthreads();
   if (threadIdx.x == 0) {
     s_pre[0] = 0;
@@ -1087,31 +1298,131 @@ __global__ void __launch_bounds__(MK_BLOCK) k_multi_commit_screen(MultiArgs a, i
   for (int it = blockIdx.x * MK_BLOCK + threadIdx.x; it < total; it += gridDim.x * MK_BLOCK) {
     while (s_pre[r + 1] <= it) ++r;
     const int loc = it - s_pre[r];
-    const int q = loc / NI, k = loc - q * NI;
-    const int2 e = a.pend[(long long)r * a.D + q];
+    const int n = loc / NI, k = loc - n * NI;
+    const int2 e = a.pend[(long long)r * a.D + n];
     const int tb = e.y & 255, ta = e.y >> 8;
     uint8_t* ty = a.types + (long long)r * a.N;
-    float2* rf = a.rf + (long long)r * a.rf_n;
+    double* rho = a.rho + (long long)r * a.N;
     const int3 ph = multi_half(a, e.x);
+    // the item's site: its entry, the species and density it has from now on
+    int X = ph.x >> 1, Y = ph.y >> 1, Z = ph.z >> 1, bb = e.x & 1, t = tb;
+    double nr;
+    long long q;
     if (k < MK_BCC5_N) {
       const int4 h = s_off[k];
-      int X, Y, Z, bb;
       multi_nbr_cell(a, ph, h, X, Y, Z, bb);
-      const int j = ((Z * a.ny + Y) * a.nx + X) * 2 + bb;
-      double* rho = a.rho + (long long)r * a.N;
-      const double nr = rho[j] + s_df[(h.w * K + ta) * K + tb];
-      rho[j] = nr;
-      const float r32 = (float)nr;
-      const long long q = multi_rfi(a, X, Y, Z, bb);
-      rf[q] = make_float2(r32, emb32_val(a, ty[j], r32));
-      // delayed acceptance (K = 2): the flipped site is in shell h.w of j
-      if (a.da) a.nbc[(long long)r * a.rf_n + q] += (uint32_t)(tb - ta) << (6 * h.w);
+      const int jn = ((Z * a.ny + Y) * a.nx + X) * 2 + bb;
+      nr = rho[jn] + s_df[(h.w * K + ta) * K + tb];
+      rho[jn] = nr;
+      t = ty[jn];
+      q = multi_rfi(a, X, Y, Z, bb);
+      // the flipped site is in shell h.w of this one (da, dtab: K = 2)
+      if (a.dtab || a.da) a.nbc[(long long)r * a.rf_n + q] += (uint32_t)(tb - ta) << (6 * h.w);
     } else {
+      nr = rho[e.x];
       ty[e.x] = (uint8_t)tb;
-      const int b = e.x & 1;
-      const long long q = multi_rfi(a, (ph.x - b) >> 1, (ph.y - b) >> 1, (ph.z - b) >> 1, b);
-      rf[q].y = emb32_val(a, tb, rf[q].x);
+      q = multi_rfi(a, X, Y, Z, bb);
     }
+    if (a.dtab) {
+      float* D = a.dtab + (long long)r * DTAB_PLANES * a.rf_n + q;
+      const long long u = emb_fix(a, nr);
+      const EmbPoint p0 = emb_point(a, t, u);
+      D[10 * a.rf_n] = dtab_value(a, 1 - t, u, u, p0);
+#pragma unroll
+      for (int s = 0; s < 10; ++s) D[s * a.rf_n] = dtab_value(a, t, u + s_fix[s], u, p0);
+    } else {
+      const float r32 = (float)nr;
+      a.rf[(long long)r * a.rf_n + q] = make_float2(r32, emb32_val(a, t, r32));
+    }
+  }
+}
+
+// Propose of the plain rule for K = 2 with the re-embedding table: the screened
+// propose (k_multi_propose<2>) without the stages the table makes needless.
+// Bound: the 15 MB of entries of a step of 64,000 trials (DRAM, the table is
+// larger than L2) behind two dependent loads.
+__global__ void __launch_bounds__(MK_BLOCK, 4) k_multi_propose_table(MultiArgs a, int j) {
+  pdl_trigger();  // the commit of this step: its prologue
+  __shared__ long long sP[12];
+  __shared__ double sFd[10];
+  __shared__ int scode[MK_BCC5_N];
+  __shared__ int s_fw[MK_BLOCK / 32][15];
+  __shared__ int s_dn, s_ties;
+  const int r = blockIdx.y, tid = threadIdx.x;
+  if (tid >= MK_BLOCK - 2) pq_table(a.Dq, tid - (MK_BLOCK - 2), sP);
+  if (tid < 10) sFd[tid] = a.Fd[tid];
+  if (tid == 0) s_dn = s_ties = 0;
+  const MRepParams& p = a.rp[r];
+  const long long step = *a.base + j;
+  const int c = __ldg(a.ctab + r * MK_CTAB + j), pc = c >> 1, b = c & 1;
+  int cp[3];
+  const int pq = mk_div(pc, a.qx, __frcp_rn((float)a.qx));
+  cp[0] = pc - pq * a.qx;
+  cp[2] = mk_div(pq, a.qy, __frcp_rn((float)a.qy));
+  cp[1] = pq - cp[2] * a.qy;
+  if (tid < MK_BCC5_N) scode[tid] = b ? mk_bcc5_desc<1>(tid) : mk_bcc5_desc<0>(tid);
+  const int d = blockIdx.x * MK_BLOCK + tid, lane = tid & 31;
+  int kx = 0, ky = 0, kz = 0, site = 0;
+  uint64_t u53 = 0;
+  if (d < a.D) {
+    const int dq = mk_div(d, a.nxq, a.rcp_nxq);
+    kx = d - dq * a.nxq;
+    kz = mk_div(dq, a.nyq, a.rcp_nyq);
+    ky = dq - kz * a.nyq;
+    site = (((cp[2] + a.qz * kz) * a.ny + cp[1] + a.qy * ky) * a.nx + cp[0] + a.qx * kx) * 2 + b;
+    const uint4 w = philox4x32_10(make_uint4((uint32_t)step, (uint32_t)((uint64_t)step >> 32), (uint32_t)d, TAG_TRIAL),
+                                  p.key);
+    u53 = top53(w.z, w.w);
+  }
+  const float beta32 = p.beta32, cm0 = p.cmt32[0], cm1 = p.cmt32[1];
+  __syncthreads();
+  pdl_wait();
+  int acc = 0, tie = 0, ta = 0, dec = 0;
+  long long pqv = 0;
+  if (d < a.D) {
+    ta = a.types[(long long)r * a.N + site];
+    float err;
+    bool in;
+    const float e32 = b ? multi_screen_table<1>(a, sP, r, cp, kx, ky, kz, ta, &pqv, &err, &in)
+                        : multi_screen_table<0>(a, sP, r, cp, kx, ky, kz, ta, &pqv, &err, &in);
+    const float cm = ta ? cm1 : cm0;
+    const float x32 = beta32 * (e32 + cm);
+    const float dx = beta32 * fmaf(4.76837158203125e-07f, fabsf(e32) + fabsf(cm), err) * 1.0001f +
+                     fabsf(x32) * 4.76837158203125e-07f;
+    dec = in ? screen32(x32, dx, u53) : -1;
+    acc = dec > 0 ? 1 : 0;
+  }
+  // trials the screen left open: FP64 dE by the whole warp, one at a time
+  unsigned open = __ballot_sync(0xffffffffu, dec < 0);
+  while (open) {
+    const int src = __ffs(open) - 1;
+    open &= open - 1u;
+    const int si = __shfl_sync(0xffffffffu, site, src), sa = __shfl_sync(0xffffffffu, ta, src);
+    const double v = warp_sum(multi_emb_warp5(a, sFd, scode, s_fw[tid >> 5], r, si, sa, 1 - sa, lane));
+    if (lane == src) {
+      const double de64 = (double)pqv * a.qscale + v;
+      if (!isfinite(de64)) atomicOr(a.err, ERRF_NONFINITE);
+      acc = metropolis(p.beta * (de64 + (p.dmu0[1 - ta] - p.dmu0[ta])), u53, &tie) ? 1 : 0;
+    }
+  }
+  // compaction of the local accepts, dn and ties: one reservation per warp
+  MStepAcc* A = a.acc + 2 * r + (int)(step & 1);
+  const unsigned m = __ballot_sync(0xffffffffu, acc);
+  if (m) {
+    int base = 0;
+    const int dn = __reduce_add_sync(0xffffffffu, acc ? 1 - 2 * ta : 0);
+    if (lane == 0) {
+      base = atomicAdd(&A->nacc, __popc(m));
+      atomicAdd(&s_dn, dn);
+    }
+    base = __shfl_sync(0xffffffffu, base, 0);
+    if (acc) a.pend[(long long)r * a.D + base + __popc(m & ((1u << lane) - 1u))] = make_int2(site, (1 - ta) | (ta << 8));
+  }
+  if (tie) atomicAdd(&s_ties, tie);
+  __syncthreads();
+  if (tid == 0) {
+    if (s_dn) atomicAdd(&A->dn[1], s_dn);
+    if (s_ties) atomicAdd(&A->ties, s_ties);
   }
 }
 
@@ -1134,10 +1445,14 @@ void launch_multi_step(const MultiArgs& a, int j, cudaStream_t st, bool after_st
     cfg.attrs = attr;
     cfg.numAttrs = after_step ? 1 : 0;
     if (a.da)
-      cudaLaunchKernelEx(&cfg, k_multi_propose<3>, a, j);
+      a.dtab ? cudaLaunchKernelEx(&cfg, k_multi_propose<3, true>, a, j)
+             : cudaLaunchKernelEx(&cfg, k_multi_propose<3, false>, a, j);
     else
-      cudaLaunchKernelEx(&cfg, k_multi_propose<2>, a, j);
-    k_multi_commit_screen<<<4 * a.n_sm, MK_BLOCK, 0, st>>>(a, j);
+      a.dtab ? cudaLaunchKernelEx(&cfg, k_multi_propose_table, a, j)
+             : cudaLaunchKernelEx(&cfg, k_multi_propose<2, false>, a, j);
+    cfg.gridDim = dim3((unsigned)(4 * a.n_sm));
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, k_multi_commit_screen, a, j);
   } else if (a.reembed) {
     k_multi_propose<1><<<grid, MK_BLOCK, 0, st>>>(a, 0);
     k_multi_commit<1><<<cgrid, MK_BLOCK, 0, st>>>(a);
@@ -1425,7 +1740,21 @@ __global__ void __launch_bounds__(MK_BLOCK) k_multi_fused(MultiArgs a, int j) {
   }
 }
 
-__global__ void k_multi_advance(long long* base, int n) { *base += n; }
+// base += n; the colours of the next MK_CTAB steps (replica-major; every
+// thread's steps follow from the old base, which thread 0 of the one block
+// moves after the barrier)
+__global__ void k_multi_advance(MultiArgs a, long long* base, int n) {
+  const long long b0 = *base + n;
+  if (a.ctab)
+    for (int q = threadIdx.x; q < a.R * MK_CTAB; q += blockDim.x) {
+      const long long k = b0 + q % MK_CTAB;
+      const uint4 w = philox4x32_10(make_uint4((uint32_t)k, (uint32_t)((uint64_t)k >> 32), 0xFFFFFFFFu, TAG_STEP),
+                                    a.rp[q / MK_CTAB].key);
+      a.ctab[q] = (int)below64(w.x, w.y, (uint64_t)a.n_colours);
+    }
+  __syncthreads();
+  if (threadIdx.x == 0) *base = b0;
+}
 
 void launch_multi_fused(const MultiArgs& a, int j, bool propose, cudaStream_t st) {
   cudaLaunchConfig_t cfg = {};
@@ -1441,7 +1770,9 @@ void launch_multi_fused(const MultiArgs& a, int j, bool propose, cudaStream_t st
   else cudaLaunchKernelEx(&cfg, k_multi_fused<false>, a, j);
 }
 
-void launch_multi_advance(long long* base, int n, cudaStream_t st) { k_multi_advance<<<1, 1, 0, st>>>(base, n); }
+void launch_multi_advance(const MultiArgs& a, long long* base, int n, cudaStream_t st) {
+  k_multi_advance<<<1, a.ctab ? 512 : 32, 0, st>>>(a, base, n);
+}
 
 __global__ void k_multi_delta_e(MultiArgs a, int r, const long long* sites, const uint8_t* to, int n, double* out) {
   const int q = blockIdx.x * blockDim.x + threadIdx.x;
@@ -1458,26 +1789,26 @@ void launch_multi_delta_e(const MultiArgs& a, int r, const long long* sites, con
   k_multi_delta_e<<<(n + 127) / 128, 128, 0, st>>>(a, r, sites, to, n, out);
 }
 
-// Delayed acceptance (K = 2): per-site B counts in the five shells from the
-// species of every replica (shell s at bit 6 s of nbc, laid out like rf)
-__global__ void k_multi_nbc(MultiArgs a) {
-  const int r = blockIdx.y;
+// K = 2: per-site B counts in the five shells from the species of replicas
+// r0 ... (shell s at bit 6 s of nbc, laid out like rf)
+__global__ void k_multi_nbc(MultiArgs a, int r0) {
+  const int r = r0 + blockIdx.y;
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= a.N) return;
   const uint8_t* ty = a.types + (long long)r * a.N;
   uint32_t w = 0u;
+  const int3 p = multi_half(a, (int)i);
   for (int k = 0; k < a.n_off; ++k) {
     const int4 h = a.off[k];
-    w += (uint32_t)(ty[multi_nbr(a, (int)i, h)] == 1) << (6 * h.w);
+    w += (uint32_t)(ty[multi_nbr_at(a, p, h)] == 1) << (6 * h.w);
   }
-  const int3 p = multi_half(a, (int)i);
   const int b = (int)(i & 1);
   a.nbc[(long long)r * a.rf_n + multi_rfi(a, (p.x - b) >> 1, (p.y - b) >> 1, (p.z - b) >> 1, b)] = w;
 }
 
-void launch_multi_nbc(const MultiArgs& a, cudaStream_t st) {
-  const dim3 grid((unsigned)((a.N + 255) / 256), (unsigned)a.R);
-  k_multi_nbc<<<grid, 256, 0, st>>>(a);
+void launch_multi_nbc(const MultiArgs& a, int r0, int nrep, cudaStream_t st) {
+  const dim3 grid((unsigned)((a.N + 255) / 256), (unsigned)nrep);
+  k_multi_nbc<<<grid, 256, 0, st>>>(a, r0);
 }
 
 // Surrogate descriptors X[r N + i][10] (raw counts from nbc) and targets

@@ -3,6 +3,7 @@
 // Sec. III A of Sadigh et al.).
 #include "common.cuh"
 #include "kernels.h"
+#include "multi.cuh"
 
 namespace vcsgc {
 
@@ -477,6 +478,124 @@ void launch_energy(const McArgs& a, bool shell, int r, double* part, cudaStream_
     if (shell) k_energy<true, false><<<g, E_BLOCK, 0, st>>>(a, r, part);
     else k_energy<false, false><<<g, E_BLOCK, 0, st>>>(a, r, part);
   }
+}
+
+// ---------------------------------- densities and energy, five-shell lattice
+// A site's neighbours lie on five shells, so its density and its pair energy
+// depend on the B counts b_s of the shells alone:
+//   rho_i = sum_s [(z_s - b_s) f_A(r_s) + b_s f_B(r_s)]: five table entries;
+//   sum of pairs = 1/2 sum_s {z_s [N phi_AA + 2 n_B (phi_AB - phi_AA)] + (phi_BB -
+//   2 phi_AB + phi_AA) P_s}(r_s), P_s = sum over B sites of b_s: whole numbers.
+// Per site that leaves the embedding cubic and five additions in FP64 (GB300
+// has 2 FP64 lanes per SM and clock), against two table cubics for each of 58
+// neighbours: 80^3 x 8 replicas, densities and energies 28.5 -> 0.4 ms.  Every
+// replica in one launch.  shell: f_A, f_B, phi_AA, phi_AB, phi_BB at the five
+// radii.  part[r][blocks]: sums of F over a block's sites; tot[r][6]: P_s, n_B.
+constexpr int SS_BLOCK = 256, SS_SITES = 4;
+
+__global__ void k_shell_values(Tables tab, Tables32 tab32, int mixed, const double* shell_tab, double* out,
+                               unsigned* err) {
+  const int s = threadIdx.x;
+  if (s >= 5) return;
+  const Tables32* t32 = mixed ? &tab32 : nullptr;
+  const double r = shell_tab[11 + s];
+  const int q[5] = {3, 4, 0, 1, 2};
+  for (int k = 0; k < 5; ++k) out[5 * k + s] = tab_val(tab, t32, q[k], r, err);
+}
+
+void launch_shell_values(const McArgs& a, double* out, cudaStream_t st) {
+  k_shell_values<<<1, 32, 0, st>>>(a.tab, a.tab32, a.mixed, a.shell_tab, out, a.err);
+}
+
+template <int B>
+__device__ __forceinline__ void shell_counts(const uint8_t* ty, int nx, int ny, int nz, int cx, int cy, int cz,
+                                             int (&b)[5]) {
+  int xo[5], yo[5], zo[5];
+#pragma unroll
+  for (int d = -2; d <= 2; ++d) {
+    const int X = cx + d, Y = cy + d, Z = cz + d;
+    xo[d + 2] = 2 * (X < 0 ? X + nx : (X >= nx ? X - nx : X));
+    yo[d + 2] = 2 * nx * (Y < 0 ? Y + ny : (Y >= ny ? Y - ny : Y));
+    zo[d + 2] = 2 * nx * ny * (Z < 0 ? Z + nz : (Z >= nz ? Z - nz : Z));
+  }
+#pragma unroll
+  for (int s = 0; s < 5; ++s) b[s] = 0;
+#pragma unroll
+  for (int k = 0; k < MK_BCC5_N; ++k) {
+    const int code = mk_bcc5_code(k);
+    const int hx = (code & 15) - 4, hy = ((code >> 4) & 15) - 4, hz = ((code >> 8) & 15) - 4;
+    const int bb = B ^ (hx & 1);
+    b[code >> 12] += ty[zo[((B + hz - bb) >> 1) + 2] + yo[((B + hy - bb) >> 1) + 2] + xo[((B + hx - bb) >> 1) + 2] + bb];
+  }
+}
+
+__global__ void __launch_bounds__(SS_BLOCK)
+    k_shell_state(McArgs a, int nx, int ny, int nz, const double* shell, int r0, double* rho, double* part,
+                  unsigned long long* tot) {
+  const int r = r0 + blockIdx.y;
+  __shared__ double s_t[5][25];  // (z - b) f_A + b f_B
+  __shared__ double s_e[SS_BLOCK / 32];
+  for (int q = threadIdx.x; q < 125; q += SS_BLOCK) {
+    constexpr int z[5] = {8, 6, 12, 24, 8};
+    const int s = q / 25, b = q - 25 * s;
+    s_t[s][b] = b <= z[s] ? (double)(z[s] - b) * shell[s] + (double)b * shell[5 + s] : 0.0;
+  }
+  __syncthreads();
+  const uint8_t* ty = a.types + (long long)r * a.N;
+  // a warp takes sites of one basis (its lanes run one of the two unrolled
+  // neighbour tables): site 2 cell + basis
+  double e = 0.0;
+  int P[6] = {0, 0, 0, 0, 0, 0};
+  const long long half = a.N >> 1;
+#pragma unroll 1
+  for (int u = 0; u < SS_SITES; ++u) {
+    const long long cell = ((long long)blockIdx.x * (SS_SITES / 2) + (u >> 1)) * SS_BLOCK + threadIdx.x;
+    const int basis = u & 1;
+    if (cell >= half) continue;
+    const int cx = (int)(cell % nx), cyz = (int)(cell / nx);
+    const int cy = cyz % ny, cz = cyz / ny;
+    int b[5];
+    if (basis) shell_counts<1>(ty, nx, ny, nz, cx, cy, cz, b);
+    else shell_counts<0>(ty, nx, ny, nz, cx, cy, cz, b);
+    double d = s_t[0][b[0]];
+#pragma unroll
+    for (int s = 1; s < 5; ++s) d += s_t[s][b[s]];
+    const long long i = 2 * cell + basis;
+    if (rho) rho[(long long)r * a.N + i] = d;
+    const int t = ty[i];
+    e += spline_val(a.tab.sp[5 + t], d, a.err);
+    if (t) {
+#pragma unroll
+      for (int s = 0; s < 5; ++s) P[s] += b[s];
+      P[5] += 1;
+    }
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
+  if ((threadIdx.x & 31) == 0) s_e[threadIdx.x >> 5] = e;
+#pragma unroll
+  for (int s = 0; s < 6; ++s) {
+    const int v = __reduce_add_sync(0xffffffffu, P[s]);
+    if ((threadIdx.x & 31) == 0 && v) atomicAdd(tot + 6 * blockIdx.y + s, (unsigned long long)v);
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double v = 0.0;
+    for (int w = 0; w < SS_BLOCK / 32; ++w) v += s_e[w];
+    part[(long long)blockIdx.y * gridDim.x + blockIdx.x] = v;
+  }
+}
+
+int shell_state_blocks(long long N) {
+  const long long per = (long long)SS_BLOCK * (SS_SITES / 2);
+  return (int)((N / 2 + per - 1) / per);
+}
+
+void launch_shell_state(const McArgs& a, const int n3[3], const double* shell, int r0, int nrep, double* rho,
+                        double* part, unsigned long long* tot, cudaStream_t st) {
+  cudaMemsetAsync(tot, 0, sizeof(unsigned long long) * 6 * nrep, st);
+  k_shell_state<<<dim3((unsigned)shell_state_blocks(a.N), (unsigned)nrep), SS_BLOCK, 0, st>>>(
+      a, n3[0], n3[1], n3[2], shell, r0, rho, part, tot);
 }
 
 }  // namespace vcsgc

@@ -16,6 +16,8 @@ constexpr int MK_MAX_SH = 8;      // neighbour shells
 constexpr int MK_MAX_OFF = 96;    // neighbour offsets (5 BCC shells: 58)
 constexpr int MK_BLOCK = 128;
 constexpr int MK_SCREEN_MAX_R = 1024;  // replicas of the screened form
+constexpr int MK_CTAB = 64;        // steps whose colours the advance kernel prepares
+constexpr int DTAB_PLANES = 11;  // 2 x 5 shells, own change
 constexpr uint32_t TAG_SPECIES = 6u;  // (step, domain rank): the proposed species
 
 // Per-replica parameters: index alpha = 0..K-1, entry 0 (the solvent) zero.
@@ -32,6 +34,8 @@ struct MRepParams {
   float c32[MK_MAX * MK_MAX];
   // the same with re-embedding: dmu0_b - dmu0_a rounded to float
   float cmu32[MK_MAX * MK_MAX];
+  float bk32[MK_MAX], n0_32[MK_MAX];  // beta kappa_p, n0
+  float cmt32[2];  // K = 2: dmu0_{1-a} - dmu0_a rounded to float, [a]
 };
 
 struct MRepState {
@@ -100,6 +104,7 @@ struct MultiArgs {
   int* slot;            // [R][D] site of trial d's pending flip, or -1
   long long* nstart;    // [R][2][MK_MAX] counts at the start of a step, by parity
   const long long* base;  // step of launch j = 0
+  int* ctab;            // [R][MK_CTAB] colours of steps *base + j (with dtab)
   // screened form (re-embedding, five-shell table): the local decision is
   // taken on an FP32 dE with a rigorous error bound, FP64 only where the
   // bound cannot decide.  The embedding cubics rounded to float
@@ -119,12 +124,11 @@ struct MultiArgs {
   float emb_off[MK_MAX * MK_MAX];
   float qscale32;       // 2^-qbits as a float (exact)
   // (rho_i as float, the offset table's F32_{t_i} of that) per site,
-  // [R][rf_n], laid out by
-  // (basis, z, y, x mod qx, x div qx): the lanes of a warp, trials qx
-  // cells apart along x, read neighbours at one offset from consecutive
-  // entries.  rf_q = ceil(nx / qx); rf_n = 2 nz ny qx rf_q
+  // [R][rf_n], rf_n = N, laid out by (basis, z mod qz, y mod qy, x mod qx;
+  // z div qz, y div qy, x div qx): the neighbours at one offset of a colour's
+  // trials are one contiguous run in trial order (but for the wraps), so a
+  // warp's loads fill their sectors.  Not kept with dtab.
   float2* rf;
-  int rf_q;
   long long rf_n;
   int n_sm;             // multiprocessors of the device (commit grid)
   // delayed acceptance (K = 2, screened form): a trial first passes a
@@ -132,10 +136,22 @@ struct MultiArgs {
   // stage on the exact dE - s g.  The surrogate's descriptor comes from
   // nbc[R][rf_n] (laid out like rf): per site the B sites in each of its
   // five shells, 6 bits per shell (shell s at bit 6 s), kept up to date by
-  // the commit while da is set.
+  // the commit while da is set or dtab is there.
   int da;
   MlpW mlp;
   uint32_t* nbc;
+  // re-embedding table of the screened form for K = 2 (null: K > 2 or not
+  // enough memory), laid out like rf, [R][DTAB_PLANES][rf_n] floats: per site
+  // the change F_t(rho + f_b(r_s) - f_a(r_s)) - F_t(rho) for 0 -> 1 and 1 -> 0
+  // and each shell s, and the own change F_{1-t}(rho) - F_t(rho); NaN where an
+  // argument leaves [emb_lo, emb_hi] (as x / h in fixed point, 32 fraction
+  // bits: [fix_lo, fix_hi]).  emb_s, emb_lo0: the cubics as floats with c0 in
+  // two parts; tab_err: bound of the cubics' roundings over a trial's entries
+  float* dtab;
+  const float4* emb_s;
+  const float* emb_lo0;
+  long long fix_lo, fix_hi;
+  float tab_err;
 };
 
 // site index of trial d of colour c (ascending site index within a colour)
@@ -179,11 +195,24 @@ __device__ __forceinline__ void multi_nbr_cell(const MultiArgs& a, int3 p, int4 
   Z += Z < 0 ? a.nz : (Z >= a.nz ? -a.nz : 0);
 }
 
-// entry of cell (X, Y, Z), basis b in the screened form's per-site floats
+// entry of cell (X, Y, Z), basis b in the screened form's per-site arrays: the
+// site's sublattice class first, then its place among the class's sites (the
+// trial index of that colour).  The index is a sum of one term per axis.
+__device__ __forceinline__ int rfi_x(const MultiArgs& a, int X) {
+  const int q = X / a.qx;
+  return (X - q * a.qx) * a.D + q;
+}
+__device__ __forceinline__ int rfi_y(const MultiArgs& a, int Y) {
+  const int q = Y / a.qy;
+  return (Y - q * a.qy) * (a.qx * a.D) + q * a.nxq;
+}
+__device__ __forceinline__ int rfi_z(const MultiArgs& a, int Z) {
+  const int q = Z / a.qz;
+  return (Z - q * a.qz) * (a.qy * a.qx * a.D) + q * (a.nyq * a.nxq);
+}
+__device__ __forceinline__ int rfi_plane(const MultiArgs& a) { return (int)(a.rf_n >> 1); }  // basis 1
 __device__ __forceinline__ long long multi_rfi(const MultiArgs& a, int X, int Y, int Z, int b) {
-  const int xq = X / a.qx;
-  return ((long long)(b * a.nz + Z) * a.ny + Y) * ((long long)a.qx * a.rf_q) + (long long)(X - xq * a.qx) * a.rf_q +
-         xq;
+  return rfi_x(a, X) + rfi_y(a, Y) + rfi_z(a, Z) + (b ? rfi_plane(a) : 0);
 }
 
 __device__ __forceinline__ int multi_nbr(const MultiArgs& a, int i, int4 h) {
@@ -232,7 +261,9 @@ void launch_multi_delta_e(const MultiArgs& a, int r, const long long* sites, con
 // delayed acceptance (K = 2, five-shell table): the per-site shell counts of
 // every replica from its species; descriptors and exact targets of every
 // site (rows r N + i) from those counts
-void launch_multi_nbc(const MultiArgs& a, cudaStream_t st);
+void launch_multi_nbc(const MultiArgs& a, int r0, int nrep, cudaStream_t st);
+// re-embedding table of replicas r0 ... from their rf and species
+void launch_multi_table(const MultiArgs& a, int r0, int nrep, cudaStream_t st);
 void launch_multi_features(const MultiArgs& a, float* X, float* Y, cudaStream_t st);
 // one colour step (propose and commit); after_step: the previous launch on
 // the stream is this context's commit (the screened form then overlaps).
@@ -242,6 +273,6 @@ void launch_multi_step(const MultiArgs& a, int j, cudaStream_t st, bool after_st
 // fused form: step base + j (propose = false: only the commit and the
 // bookkeeping of the previous step), and base += n
 void launch_multi_fused(const MultiArgs& a, int j, bool propose, cudaStream_t st);
-void launch_multi_advance(long long* base, int n, cudaStream_t st);
+void launch_multi_advance(const MultiArgs& a, long long* base, int n, cudaStream_t st);
 
 }  // namespace vcsgc

@@ -9,6 +9,8 @@ namespace vcsgc {
 
 // running state of replica r (the pending step applied first)
 int multi_get_state(void* m, int r, MRepState* out);
+// running states of every replica in one transfer
+int multi_get_states(void* m, MRepState* out);
 // replace it (forms without a deferred commit only)
 int multi_set_state(void* m, int r, const MRepState* in);
 // densities rho_i of replica r (N doubles, host)

@@ -170,6 +170,11 @@ struct Ctx {
   int* sp_count = nullptr;
   int* sp_cursor = nullptr;
   int sp_ndom = 0;
+  // species-dependent densities on the five-shell lattice: table and partials
+  // of launch_shell_state (ss_shell null: another neighbourhood)
+  double* ss_shell = nullptr;
+  double* ss_part = nullptr;
+  unsigned long long* ss_tot = nullptr;
   // species-dependent densities on the period-q sublattice: the colour steps
   // run through a two-species multicomponent object (its FP32-screened
   // kernels with compile-time offsets); this context mirrors its species and
@@ -681,8 +686,46 @@ int positions_host(Ctx* c, std::vector<double>& hx, std::vector<double>& hy, std
 }
 
 // --------------------------------------------------------------- energy
+// compensated sum of block partials
+double sum_parts(const double* h, size_t n) {
+  double s = 0.0, c = 0.0;
+  for (size_t q = 0; q < n; ++q) {
+    const double v = h[q], t = s + v;
+    c += std::fabs(s) >= std::fabs(v) ? (s - t) + v : (v - t) + s;
+    s = t;
+  }
+  return s + c;
+}
+
+// energies of replicas r0 .. r0 + n - 1 (five-shell lattice, species-dependent
+// densities) from the species bytes; densities: written to c->rho too
+int shell_energies(Ctx* c, int r0, int n, bool densities, double* out) {
+  const int nb = shell_state_blocks(c->N);
+  const int n3[3] = {c->nx, c->ny, c->nz};
+  launch_shell_state(c->mc, n3, c->ss_shell, r0, n, densities ? c->rho : nullptr, c->ss_part, c->ss_tot, c->st);
+  CK(cudaGetLastError());
+  std::vector<double> part((size_t)nb * n), sh(25);
+  std::vector<unsigned long long> tot((size_t)6 * n);
+  CK(cudaMemcpyAsync(part.data(), c->ss_part, sizeof(double) * part.size(), cudaMemcpyDeviceToHost, c->st));
+  CK(cudaMemcpyAsync(tot.data(), c->ss_tot, sizeof(unsigned long long) * tot.size(), cudaMemcpyDeviceToHost, c->st));
+  CK(cudaMemcpyAsync(sh.data(), c->ss_shell, sizeof(double) * 25, cudaMemcpyDeviceToHost, c->st));
+  TRY(check_device_error(c));
+  constexpr double z[5] = {8, 6, 12, 24, 8};
+  for (int q = 0; q < n; ++q) {
+    const double nB = (double)tot[6 * q + 5];
+    double pair = 0.0;
+    for (int s = 0; s < 5; ++s) {
+      const double aa = sh[10 + s], ab = sh[15 + s], bb = sh[20 + s];
+      pair += z[s] * ((double)c->N * aa + 2.0 * nB * (ab - aa)) + (bb - 2.0 * ab + aa) * (double)tot[6 * q + s];
+    }
+    out[q] = sum_parts(part.data() + (size_t)nb * q, nb) + 0.5 * pair;
+  }
+  return VCSGC_OK;
+}
+
 int energy_of(Ctx* c, int r, double* out) {
   TRY(sync_bytes(c, r));
+  if (c->ss_shell) return shell_energies(c, r, 1, false, out);
   if (!c->subs.empty()) {
     CK(cudaStreamSynchronize(c->st));
     const int rc = energy_of(c->subs[r], 0, out);
@@ -694,20 +737,18 @@ int energy_of(Ctx* c, int r, double* out) {
   std::vector<double> h(c->part_n);
   CK(cudaMemcpyAsync(h.data(), c->part, sizeof(double) * c->part_n, cudaMemcpyDeviceToHost, c->st));
   TRY(check_device_error(c));
-  // compensated sum of the block partials
-  double s = 0.0, comp = 0.0;
-  for (double v : h) {
-    const double t = s + v;
-    comp += std::fabs(s) >= std::fabs(v) ? (s - t) + v : (v - t) + s;
-    s = t;
-  }
-  *out = s + comp;
+  *out = sum_parts(h.data(), h.size());
   return VCSGC_OK;
 }
 
 // recompute rho (and dF) of replica r, or of the shared array
 int refresh_rho(Ctx* c, int r) {
-  launch_rho(c->mc, c->shell, r, c->st);
+  if (c->ss_shell) {
+    const int n3[3] = {c->nx, c->ny, c->nz};
+    launch_shell_state(c->mc, n3, c->ss_shell, r, 1, c->rho, c->ss_part, c->ss_tot, c->st);
+  } else {
+    launch_rho(c->mc, c->shell, r, c->st);
+  }
   if (c->screen) launch_fill_rf(c->mc, r, c->st);
   CK(cudaGetLastError());
   return VCSGC_OK;
@@ -717,12 +758,16 @@ int refresh_rho(Ctx* c, int r) {
 // recompute them before anything reads the replica states
 int refresh_energies(Ctx* c) {
   if (!c->screen || !c->energy_stale) return VCSGC_OK;
-  for (int r = 0; r < c->R; ++r) {
-    double e;
-    TRY(energy_of(c, r, &e));
-    CK(cudaMemcpyAsync(&c->rs[r].energy, &e, sizeof(double), cudaMemcpyHostToDevice, c->st));
-    CK(cudaStreamSynchronize(c->st));
+  std::vector<double> e(c->R);
+  if (c->ss_shell) {
+    TRY(sync_bytes(c, -1));
+    TRY(shell_energies(c, 0, c->R, false, e.data()));
+  } else {
+    for (int r = 0; r < c->R; ++r) TRY(energy_of(c, r, &e[r]));
   }
+  for (int r = 0; r < c->R; ++r)
+    CK(cudaMemcpyAsync(&c->rs[r].energy, &e[r], sizeof(double), cudaMemcpyHostToDevice, c->st));
+  CK(cudaStreamSynchronize(c->st));
   c->energy_stale = false;
   return VCSGC_OK;
 }
@@ -966,33 +1011,40 @@ int run_steps(Ctx* c, long long n) {
 // multicomponent object after its steps (the energy is recomputed when read)
 int sync_from_multi(Ctx* c) {
   if (!c->multi || !c->multi_dirty) return VCSGC_OK;
-  for (int r = 0; r < c->R; ++r) {
-    MRepState ms;
-    const int rc = multi_get_state(c->multi, r, &ms);
-    if (rc != VCSGC_OK) return fail(c, rc, vcsgc_multi_last_error(c->multi));
-    const uint8_t* t = multi_types_device(c->multi, r);
-    if (!t) return fail(c, VCSGC_ERR_CUDA, vcsgc_multi_last_error(c->multi));
-    CK(cudaMemcpyAsync(c->rep_types[r], t, c->N, cudaMemcpyDeviceToDevice, c->st));
-    TRY(refresh_rho(c, r));
-    RepState s;
-    std::memset(&s, 0, sizeof(s));
-    s.n = ms.cnt[1];
-    s.step = ms.step;
-    s.fin_step = ms.fin_step;
-    s.trials = ms.trials;
-    s.local_acc = ms.local_acc;
-    s.global_trials = ms.global_trials;
-    s.global_acc = ms.global_acc;
-    s.flips = ms.flips;
-    s.near_ties = ms.near_ties;
-    s.steps = ms.steps;
-    s.sum_c = ms.sum_c[1];
-    s.sum_c2 = ms.sum_c2[1];
-    s.s1_acc = ms.s1_acc;
-    CK(cudaMemcpyAsync(c->rs + r, &s, sizeof(RepState), cudaMemcpyHostToDevice, c->st));
+  std::vector<MRepState> ms(c->R);
+  const int rc = multi_get_states(c->multi, ms.data());
+  if (rc != VCSGC_OK) return fail(c, rc, vcsgc_multi_last_error(c->multi));
+  const uint8_t* t = multi_types_device(c->multi, 0);  // all replicas back to back, as here
+  if (!t) return fail(c, VCSGC_ERR_CUDA, vcsgc_multi_last_error(c->multi));
+  CK(cudaMemcpyAsync(c->types, t, (size_t)c->R * c->N, cudaMemcpyDeviceToDevice, c->st));
+  std::vector<double> e(c->R, 0.0);
+  if (c->ss_shell) {
+    TRY(shell_energies(c, 0, c->R, true, e.data()));
+  } else {
+    for (int r = 0; r < c->R; ++r) TRY(refresh_rho(c, r));
   }
+  std::vector<RepState> rs(c->R);
+  for (int r = 0; r < c->R; ++r) {
+    RepState& s = rs[r];
+    std::memset(&s, 0, sizeof(s));
+    s.n = ms[r].cnt[1];
+    s.step = ms[r].step;
+    s.fin_step = ms[r].fin_step;
+    s.energy = e[r];
+    s.trials = ms[r].trials;
+    s.local_acc = ms[r].local_acc;
+    s.global_trials = ms[r].global_trials;
+    s.global_acc = ms[r].global_acc;
+    s.flips = ms[r].flips;
+    s.near_ties = ms[r].near_ties;
+    s.steps = ms[r].steps;
+    s.sum_c = ms[r].sum_c[1];
+    s.sum_c2 = ms[r].sum_c2[1];
+    s.s1_acc = ms[r].s1_acc;
+  }
+  CK(cudaMemcpyAsync(c->rs, rs.data(), sizeof(RepState) * c->R, cudaMemcpyHostToDevice, c->st));
   CK(cudaStreamSynchronize(c->st));
-  c->energy_stale = true;
+  c->energy_stale = !c->ss_shell;
   c->multi_dirty = false;
   return VCSGC_OK;
 }
@@ -1070,17 +1122,6 @@ double nhc_step(int M, const double* Q, double* xi, double* eta, double K2, doub
   return scale;
 }
 
-// sum of block partials (compensated)
-double sum_parts(const std::vector<double>& h) {
-  double s = 0.0, c = 0.0;
-  for (double v : h) {
-    const double t = s + v;
-    c += std::fabs(s) >= std::fabs(v) ? (s - t) + v : (v - t) + s;
-    s = t;
-  }
-  return s + c;
-}
-
 // sum m v^2 (eV) of replica 0's atoms, with the pending scale applied
 int twice_ke_dev(Ctx* c, double* out) {
   const int nb = kinetic_blocks(c->N);
@@ -1090,7 +1131,7 @@ int twice_ke_dev(Ctx* c, double* out) {
   std::vector<double> h(nb);
   CK(cudaMemcpyAsync(h.data(), c->cg_part, sizeof(double) * nb, cudaMemcpyDeviceToHost, c->st));
   CK(cudaStreamSynchronize(c->st));
-  *out = 2.0 * sum_parts(h) * c->nh.vs * c->nh.vs;
+  *out = 2.0 * sum_parts(h.data(), h.size()) * c->nh.vs * c->nh.vs;
   return VCSGC_OK;
 }
 
@@ -1513,18 +1554,27 @@ static int init_impl(Ctx* c, const vcsgc_lattice* L, const uint8_t* types, const
   // ---- screened re-embedding on the rigid lattice
   if (c->kind == 0 && c->reembed && c->shell && c->mc.n_shells > 0) TRY(screen_setup(c));
   // ---- rho, dF and energies (A2)
-  if (c->reembed) {
-    for (int r = 0; r < c->R; ++r) TRY(refresh_rho(c, r));
+  if (c->kind == 0 && c->reembed && c->shell && c->mc.n_shells == 5 && c->K == MK_BCC5_N) {
+    TRY(dalloc(c, &c->ss_part, (size_t)shell_state_blocks(c->N) * c->R));
+    TRY(dalloc(c, &c->ss_tot, (size_t)6 * c->R));
+    TRY(dalloc(c, &c->ss_shell, 25));
+    launch_shell_values(c->mc, c->ss_shell, c->st);
+    CK(cudaGetLastError());
+  }
+  std::vector<double> e0(c->R);
+  if (c->ss_shell) {
+    TRY(shell_energies(c, 0, c->R, true, e0.data()));
+    if (c->screen)
+      for (int r = 0; r < c->R; ++r) launch_fill_rf(c->mc, r, c->st);
+    CK(cudaGetLastError());
   } else {
-    TRY(refresh_rho(c, 0));
+    for (int r = 0; r < (c->reembed ? c->R : 1); ++r) TRY(refresh_rho(c, r));
+    TRY(check_device_error(c));
+    for (int r = 0; r < c->R; ++r) TRY(energy_of(c, r, &e0[r]));
   }
-  TRY(check_device_error(c));
-  for (int r = 0; r < c->R; ++r) {
-    double e;
-    TRY(energy_of(c, r, &e));
-    CK(cudaMemcpyAsync(&c->rs[r].energy, &e, sizeof(double), cudaMemcpyHostToDevice, c->st));
-    CK(cudaStreamSynchronize(c->st));
-  }
+  for (int r = 0; r < c->R; ++r)
+    CK(cudaMemcpyAsync(&c->rs[r].energy, &e0[r], sizeof(double), cudaMemcpyHostToDevice, c->st));
+  CK(cudaStreamSynchronize(c->st));
   if (c->kind == 1 && c->R == 1) TRY(md_forces(c));
   TRY(check_device_error(c));
   TRY(setup_fast(c, hs));
@@ -2863,7 +2913,7 @@ int vcsgc_minimize(void* ctx, double ftol, int64_t max_iter, int64_t* iters, dou
     CK(cudaGetLastError());
     CK(cudaMemcpyAsync(hp.data(), c->cg_part, sizeof(double) * nb, cudaMemcpyDeviceToHost, c->st));
     CK(cudaStreamSynchronize(c->st));
-    *out = sum_parts(hp);
+    *out = sum_parts(hp.data(), hp.size());
     return VCSGC_OK;
   };
   auto maxnorm = [&](const double* a, double* out) -> int {

@@ -146,6 +146,10 @@ int load_replica(Multi* m, int r, const uint8_t* t, bool reset_counters) {
   m->acc_stale = true;
   MCK(cudaMemcpyAsync(m->args.types + (long long)r * m->N, t, m->N, cudaMemcpyHostToDevice, m->st));
   launch_multi_rho(m->args, r, 1, m->st);
+  if (m->args.dtab) {
+    launch_multi_nbc(m->args, r, 1, m->st);
+    launch_multi_table(m->args, r, 1, m->st);
+  }
   MCK(cudaGetLastError());
   double e = 0.0;
   MTRY(energy_of(m, r, &e));
@@ -180,7 +184,7 @@ int run_steps_fused(Multi* m, long long n) {
     cudaGraph_t g;
     MCK(cudaStreamBeginCapture(m->st, cudaStreamCaptureModeThreadLocal));
     for (int q = 0; q < G; ++q) launch_multi_fused(m->args, q, true, m->st);
-    launch_multi_advance(m->d_base, G, m->st);
+    launch_multi_advance(m->args, m->d_base, G, m->st);
     cudaError_t e1 = cudaGetLastError();
     MCK(cudaStreamEndCapture(m->st, &g));
     if (e1 != cudaSuccess) {
@@ -197,7 +201,7 @@ int run_steps_fused(Multi* m, long long n) {
   }
   if (n > 0) {
     for (long long q = 0; q < n; ++q) launch_multi_fused(m->args, (int)q, true, m->st);
-    launch_multi_advance(m->d_base, (int)n, m->st);
+    launch_multi_advance(m->args, m->d_base, (int)n, m->st);
     m->h_base += n;
   }
   MCK(cudaGetLastError());
@@ -206,8 +210,8 @@ int run_steps_fused(Multi* m, long long n) {
 
 // delayed acceptance: per-site shell counts from the species, if stale
 int nbc_fresh(Multi* m) {
-  if (!m->nbc_stale) return VCSGC_OK;
-  launch_multi_nbc(m->args, m->st);
+  if (!m->nbc_stale || m->args.dtab) return VCSGC_OK;
+  launch_multi_nbc(m->args, 0, m->R, m->st);
   MCK(cudaGetLastError());
   m->nbc_stale = false;
   return VCSGC_OK;
@@ -228,6 +232,8 @@ int screen_acc_ready(Multi* m) {
   for (int r = 0; r < m->R; ++r)
     MCK(cudaMemcpyAsync(m->args.acc + 2 * r + par, &acc[r], sizeof(MStepAcc), cudaMemcpyHostToDevice, m->st));
   MCK(cudaMemcpyAsync(m->d_base, &m->h_base, sizeof(long long), cudaMemcpyHostToDevice, m->st));
+  if (m->args.ctab) launch_multi_advance(m->args, m->d_base, 0, m->st);  // its colours
+  MCK(cudaGetLastError());
   MCK(cudaStreamSynchronize(m->st));
   m->acc_stale = false;
   return VCSGC_OK;
@@ -244,7 +250,7 @@ int run_steps(Multi* m, long long n) {
     cudaGraph_t g;
     MCK(cudaStreamBeginCapture(m->st, cudaStreamCaptureModeThreadLocal));
     for (int q = 0; q < G; ++q) launch_multi_step(m->args, q, m->st, q > 0);
-    if (m->args.screen) launch_multi_advance(m->d_base, G, m->st);
+    if (m->args.screen) launch_multi_advance(m->args, m->d_base, G, m->st);
     cudaError_t e1 = cudaGetLastError();
     MCK(cudaStreamEndCapture(m->st, &g));
     if (e1 != cudaSuccess) {
@@ -263,7 +269,7 @@ int run_steps(Multi* m, long long n) {
     for (long long q = 0; q < n; ++q) launch_multi_step(m->args, (int)q, m->st, q > 0);
     // the base is read before the next propose's wait: it moves by an
     // ordinary launch, and the next run starts with an ordinary launch
-    if (m->args.screen) launch_multi_advance(m->d_base, (int)n, m->st);
+    if (m->args.screen) launch_multi_advance(m->args, m->d_base, (int)n, m->st);
     m->h_base += n;
   }
   MCK(cudaGetLastError());
@@ -364,9 +370,47 @@ int screen_setup(Multi* m, const std::vector<double>& hFd) {
   a.emb_lo = (float)lo;
   a.emb_hi = (float)hi;
   a.emb_err = (float)err;
-  a.rf_q = (m->nx + a.qx - 1) / a.qx;
-  a.rf_n = 2LL * m->nz * m->ny * a.qx * a.rf_q;
-  MTRY(malloc_dev(m, &a.rf, (size_t)m->R * a.rf_n));
+  a.rf_n = m->N;
+  // K = 2: the re-embedding table while it takes at most a quarter of the free
+  // memory (else, and for K > 2, whose accepted steps would refresh 3 K^2
+  // times as many entries for 1.4 % of the trials, the trials evaluate the
+  // embedding cubics: quaternary 80^3 x 8, 31 us per step against 68)
+  const size_t table = sizeof(float) * (size_t)m->R * DTAB_PLANES * a.rf_n;
+  const size_t counts = sizeof(uint32_t) * (size_t)m->R * a.rf_n;
+  size_t free_b = 0, total_b = 0;
+  MCK(cudaMemGetInfo(&free_b, &total_b));
+  // (offsets within a replica's planes are 32-bit byte offsets)
+  if (m->K == 2 && table + counts <= free_b / 4 && sizeof(float) * (size_t)DTAB_PLANES * a.rf_n < (1ull << 32)) {
+    MTRY(malloc_dev(m, &a.ctab, (size_t)m->R * MK_CTAB));
+    MTRY(malloc_dev(m, &a.nbc, counts / sizeof(uint32_t)));
+    MTRY(malloc_dev(m, &a.dtab, table / sizeof(float)));
+    std::vector<float4> hs4((size_t)2 * n);
+    std::vector<float> hlo((size_t)2 * n);
+    const int j0 = std::max(0, (int)std::floor(lo / h) - 1), j1 = std::min(n - 1, (int)std::floor(hi / h) + 1);
+    double dm = 0.0;
+    for (int al = 0; al < 2; ++al)
+      for (int j = 0; j < n; ++j) {
+        const Cubic& q = hc[al][j];
+        const float c0 = (float)q.x;
+        hs4[(size_t)al * n + j] = make_float4(c0, (float)q.y, (float)q.z, (float)q.w);
+        hlo[(size_t)al * n + j] = (float)(q.x - (double)c0);
+        if (j >= j0 && j <= j1) dm = std::max(dm, std::fabs(q.y) + 2.0 * std::fabs(q.z) + 3.0 * std::fabs(q.w));
+      }
+    float4* s4 = nullptr;
+    float* lo0 = nullptr;
+    MTRY(malloc_dev(m, &s4, hs4.size()));
+    MTRY(malloc_dev(m, &lo0, hlo.size()));
+    MCK(cudaMemcpyAsync(s4, hs4.data(), sizeof(float4) * hs4.size(), cudaMemcpyHostToDevice, m->st));
+    MCK(cudaMemcpyAsync(lo0, hlo.data(), sizeof(float) * hlo.size(), cudaMemcpyHostToDevice, m->st));
+    MCK(cudaStreamSynchronize(m->st));
+    a.emb_s = s4;
+    a.emb_lo0 = lo0;
+    a.fix_lo = (long long)std::ceil(lo / h * 4294967296.0);
+    a.fix_hi = (long long)std::floor(hi / h * 4294967296.0);
+    a.tab_err = (float)((MK_BCC5_N + 1) * std::ldexp(dm, -20));
+  } else {
+    MTRY(malloc_dev(m, &a.rf, (size_t)m->R * a.rf_n));
+  }
   return VCSGC_OK;
 }
 
@@ -583,6 +627,11 @@ int init(Multi* m, const vcsgc_lattice* L, const uint8_t* types, const vcsgc_mul
         const double off = a.screen ? m->fref[y] - m->fref[x] : 0.0;
         p.cmu32[x * m->K + y] = (float)(p.dmu0[y] - p.dmu0[x] + off);
       }
+    for (int al = 1; al < m->K; ++al) {
+      p.bk32[al] = (float)(p.beta * p.kappa_p[al]);
+      p.n0_32[al] = (float)p.n0[al];
+    }
+    for (int x = 0; x < 2; ++x) p.cmt32[x] = (float)(p.dmu0[1 - x] - p.dmu0[x]);
   }
   MCK(cudaMemcpyAsync(rp, m->h_rp.data(), sizeof(MRepParams) * R, cudaMemcpyHostToDevice, m->st));
   MCK(cudaStreamSynchronize(m->st));
@@ -811,6 +860,16 @@ int multi_get_state(void* h, int r, MRepState* out) {
   MCK(cudaSetDevice(m->device));
   MTRY(flush(m));
   MCK(cudaMemcpyAsync(out, m->args.rs + r, sizeof(MRepState), cudaMemcpyDeviceToHost, m->st));
+  MCK(cudaStreamSynchronize(m->st));
+  return device_error(m);
+}
+
+int multi_get_states(void* h, MRepState* out) {
+  Multi* m = as_multi(h);
+  if (!m || !out) return VCSGC_ERR_INVALID_ARG;
+  MCK(cudaSetDevice(m->device));
+  MTRY(flush(m));
+  MCK(cudaMemcpyAsync(out, m->args.rs, sizeof(MRepState) * m->R, cudaMemcpyDeviceToHost, m->st));
   MCK(cudaStreamSynchronize(m->st));
   return device_error(m);
 }
