@@ -154,6 +154,88 @@ __device__ __forceinline__ double rsqrt_nr(double r2) {
   return fma(0.5 * y, e, y);
 }
 
+// ---- FP64 pair geometry with few FP64 instructions
+// GB300 issues two FP64 lanes per SM and clock: a warp instruction occupies the
+// pipe 16 cycles, conversions between double and float or int as much as an
+// FMA.  The pair loops of the explicit-position forms are bound by that pipe,
+// so what can be done on the bits of a double (integer pipe, 30 times as fast)
+// is done there.
+
+// double of a float, by bits (zero and denormals give zero)
+__device__ __forceinline__ double widen(float f) {
+  const uint32_t b = __float_as_uint(f);
+  const uint32_t hi = ((b & 0x7FFFFFFFu) >> 3) + 0x38000000u, lo = b << 29;
+  return (b & 0x7F800000u) ? __hiloint2double((int)(hi | (b & 0x80000000u)), (int)lo) : 0.0;
+}
+// float of a normal positive double in float's range, truncated
+__device__ __forceinline__ float narrow_pos(double d) {
+  return __uint_as_float((((uint32_t)__double2hiint(d) - 0x38000000u) << 3) | ((uint32_t)__double2loint(d) >> 29));
+}
+// r = sqrt(r2), and 1/r: y = rsqrt(r2) in FP32 from the truncated bits (relative
+// error below 2^-21), then one third-order step, with e = 1 - r2 y^2:
+//   sqrt(r2) = r2 y (1 + e/2 + 3 e^2 / 8 + O(e^3)), e^3 < 2^-59
+// -- five FP64 operations for r, six for both, where two Newton steps with
+// their two conversions took eleven.
+__device__ __forceinline__ double sqrt3(double r2, double& ir) {
+  const double y = widen(rsqrtf(narrow_pos(r2)));
+  const double s = r2 * y, e = fma(-s, y, 1.0), q = e * fma(0.375, e, 0.5);
+  ir = fma(y, q, y);
+  return fma(s, q, s);
+}
+// minimum image of d = x_j - x_i for positions in [0, L) of a pair closer than
+// L/2 - (L/2) 2^-20 (others may keep either image): shifted by L when |d|
+// exceeds L/2 in its high word.  Few pairs cross a face, so the shift is a
+// branch and a pair costs one FP64 subtraction per axis.
+struct PairBox {
+  double L[3];
+  int half_hi[3];  // high words of L/2
+};
+__device__ __forceinline__ PairBox pair_box(const double (&box)[3]) {
+  PairBox b;
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    b.L[q] = box[q];
+    b.half_hi[q] = __double2hiint(0.5 * box[q]);
+  }
+  return b;
+}
+__device__ __forceinline__ bool beyond(double d, int half_hi) { return (__double2hiint(d) & 0x7FFFFFFF) > half_hi; }
+// squared distance; dx, dy, dz become the minimum image
+__device__ __forceinline__ double pair_r2(const PairBox& b, double& dx, double& dy, double& dz) {
+  if (beyond(dx, b.half_hi[0]) | beyond(dy, b.half_hi[1]) | beyond(dz, b.half_hi[2])) {
+    asm volatile("");  // keeps this a branch: predicated additions would take the pipe from every pair
+    if (beyond(dx, b.half_hi[0])) dx = __double2hiint(dx) < 0 ? dx + b.L[0] : dx - b.L[0];
+    if (beyond(dy, b.half_hi[1])) dy = __double2hiint(dy) < 0 ? dy + b.L[1] : dy - b.L[1];
+    if (beyond(dz, b.half_hi[2])) dz = __double2hiint(dz) < 0 ? dz + b.L[2] : dz - b.L[2];
+  }
+  return fma(dz, dz, fma(dy, dy, dx * dx));
+}
+// r2 >= rc2 for a squared distance, by the bits; NaN is not outside (as with
+// the comparison), so that a lost atom's forces are NaN and the error is seen
+__device__ __forceinline__ bool outside(double r2, double rc2) {
+  const unsigned long long c = (unsigned long long)__double_as_longlong(rc2);
+  return (unsigned long long)__double_as_longlong(r2) - c <= 0x7FF0000000000000ull - c;
+}
+// interval j = (int)u of 0 <= u <= n_int < 2^19 and offset t = u - j (the last
+// interval at u = n_int): the integer part read from u's bits (NaN: interval 0,
+// t = NaN)
+__device__ __forceinline__ int locate_bits(double u, int n_int, double& t) {
+  const int hi = __double2hiint(u);
+  const int s = 1043 - (hi >> 20);  // 20 - exponent: fraction bits of the high word
+  int j = 0;
+  double fl = 0.0;
+  if ((unsigned)s <= 20u) {  // u >= 1
+    j = ((hi & 0xFFFFF) | 0x100000) >> s;
+    fl = __hiloint2double((hi >> s) << s, 0);
+    if (j > n_int - 1) {
+      j = n_int - 1;
+      fl = widen((float)j);
+    }
+  }
+  t = u - fl;
+  return j;
+}
+
 // ------------------------------------------------- FP32 tables (mixed form)
 // The mixed-precision form evaluates pair, density and embedding-table
 // interpolants in FP32 from the same coefficients rounded to float; sums

@@ -301,7 +301,10 @@ struct MdArgs {
   const int* cnt_h;
   int same_dens;         // f_A = f_B: one density table value serves both ends
   const uint8_t* types;
-  double *x, *y, *z, *vx, *vy, *vz, *fx, *fy, *fz;
+  double *x, *y, *z, *vx, *vy, *vz;
+  double *fx, *fy, *fz;  // one allocation of 3 N
+  Cubic* p4;             // (x, y, z, species in the low word) per atom (FP64 half-list passes)
+  uint4* u4;             // (ux, uy, uz, species) per atom (mixed half-list passes)
   double* rho;
   double* dFp;   // F'(rho_i)
   float* dFp32;  // the same in FP32 (mixed form)
@@ -313,6 +316,7 @@ struct MdArgs {
   double rc;
   double mass[2];
   double dt, c1, c2, kT;
+  double im[2], sig[2];  // FTM / mass, c2 sqrt(kT FTM / mass) per species
   uint2 key;
   Tables tab;
   Tables32 tab32;
@@ -325,7 +329,8 @@ struct MdArgs {
 // u = x / L 2^32 mod 2^32 per axis (fix_diff)
 void launch_fix_positions(long long N, const double* x, const double* y, const double* z, const double box[3],
                           uint32_t* ux, uint32_t* uy, uint32_t* uz, cudaStream_t st);
-// the mixed form refreshes the fixed-point positions first
+// densities (the half-list passes refresh their records, the mixed form its
+// fixed-point positions, first); launch_md_force follows on the same positions
 void launch_md_rho(const MdArgs& m, cudaStream_t st);
 void launch_md_force(const MdArgs& m, cudaStream_t st);
 void launch_md_first_half(const MdArgs& m, long long md_step, cudaStream_t st);

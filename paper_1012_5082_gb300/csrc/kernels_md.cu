@@ -56,103 +56,140 @@ __global__ void k_md_rho(MdArgs m) {
 // end is already known (no range test)
 __device__ __forceinline__ int locate_in(const Spline& s, double r, double& t) {
   const double u = r * s.inv_h;
+  if (s.n_int < (1 << 19)) return locate_bits(u, s.n_int, t);
   int j = (int)u;
   j = j < s.n_int - 1 ? j : s.n_int - 1;
   t = u - (double)j;
   return j;
 }
 
-// FP64 form on the half list (each pair once, j > i): rho_i and rho_j both
-// receive the pair's density (atomic adds into rho, zeroed before); with one
-// density function (same_dens) one table value serves both ends.
-__global__ void k_md_rho_half(MdArgs m) {
+// Position and species of every atom in one 32-byte record (FP64 passes) or
+// one 16-byte one (mixed): a neighbour is one sector instead of four.
+__global__ void k_md_records(MdArgs m) {
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= m.N) return;
-  const int* row = m.nbr_h + i * m.K;
-  const int cnt = m.cnt_h[i];
-  const double xi = m.x[i], yi = m.y[i], zi = m.z[i];
-  const double ix = 1.0 / m.box[0], iy = 1.0 / m.box[1], iz = 1.0 / m.box[2];
+  if (m.mixed) m.u4[i] = make_uint4(m.ux[i], m.uy[i], m.uz[i], (uint32_t)m.types[i]);
+  else m.p4[i] = Cubic{m.x[i], m.y[i], m.z[i], __hiloint2double(0, (int)m.types[i])};
+}
+__device__ __forceinline__ int record_type(const Cubic& p) { return __double2loint(p.w); }
+
+// sum of v over the LPA lanes of an atom (every lane of the warp takes part)
+template <int LPA>
+__device__ __forceinline__ double lane_sum(double v) {
+#pragma unroll
+  for (int o = LPA / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
+// The passes on the half list (each pair once, j > i) give LPA lanes to an
+// atom: they share its row, so a warp's rows differ less in length (8 atoms
+// instead of 32) and a row of 30 is a chain of 8 pairs instead of 30.
+//
+// FP64: bound by the FP64 pipe (86 % active), 17 instructions per pair for the
+// density and 27 for the force where the straightforward form took 31 and 46.
+// 1.36 M atoms, 39 M pairs within the cutoff and 12 M of skin: density 1.80 ms,
+// force 2.97 ms, a whole step 10.2 -> 5.8 ms; mixed 2.81 -> 2.06 ms.
+// rho_i and rho_j both receive the pair's density (atomic adds into rho, zeroed
+// before); with one density function (SAME) one table value serves both ends.
+template <int LPA, bool SAME>
+__global__ void __launch_bounds__(128) k_md_rho_half(MdArgs m) {
+  const long long g = (long long)blockIdx.x * 128 + threadIdx.x;
+  const long long i = g / LPA;
+  const int sub = (int)(g % LPA);
+  const bool live = i < m.N;
+  const int* row = m.nbr_h + (live ? i : 0) * m.K;
+  const int cnt = live ? m.cnt_h[i] : 0;
+  const Cubic pi = m.p4[live ? i : 0];
+  const PairBox box = pair_box(m.box);
   const double rc2 = m.rc * m.rc;
-  const int ti = m.types[i];
+  const int ti = record_type(pi);
   double rho = 0.0;
-  for (int k = 0; k < cnt; ++k) {
+  for (int k = sub; k < cnt; k += LPA) {
     const int j = row[k];
-    const double dx = mimg(m.x[j] - xi, m.box[0], ix);
-    const double dy = mimg(m.y[j] - yi, m.box[1], iy);
-    const double dz = mimg(m.z[j] - zi, m.box[2], iz);
-    const double r2 = dx * dx + dy * dy + dz * dz;
-    if (r2 >= rc2) continue;
-    const double r = r2 * rsqrt_nr(r2);
-    const int tj = m.types[j];
-    double t;
+    const Cubic pj = m.p4[j];
+    double dx = pj.x - pi.x, dy = pj.y - pi.y, dz = pj.z - pi.z;
+    const double r2 = pair_r2(box, dx, dy, dz);
+    if (outside(r2, rc2)) continue;
+    double ir, t;
+    const double r = sqrt3(r2, ir);
     const int q = locate_in(m.tab.sp[3], r, t);
-    const double fj = spline_val_at(m.tab.sp[3 + tj], q, t);  // density of j at i
-    const double fi = m.same_dens ? fj : spline_val_at(m.tab.sp[3 + ti], q, t);
+    const double fj = spline_val_at(m.tab.sp[SAME ? 3 : 3 + record_type(pj)], q, t);  // density of j at i
+    const double fi = SAME ? fj : spline_val_at(m.tab.sp[3 + ti], q, t);
     rho += fj;
     atomicAdd(m.rho + j, fi);
   }
-  atomicAdd(m.rho + i, rho);
+  rho = lane_sum<LPA>(rho);
+  if (live && sub == 0) atomicAdd(m.rho + i, rho);
 }
 
 // mixed form on the half list: FP32 geometry and tables, FP64 sums
-__global__ void k_md_rho_half32(MdArgs m) {
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= m.N) return;
-  const int* row = m.nbr_h + i * m.K;
-  const int cnt = m.cnt_h[i];
-  const uint32_t uxi = m.ux[i], uyi = m.uy[i], uzi = m.uz[i];
+template <int LPA>
+__global__ void __launch_bounds__(128) k_md_rho_half32(MdArgs m) {
+  const long long g = (long long)blockIdx.x * 128 + threadIdx.x;
+  const long long i = g / LPA;
+  const int sub = (int)(g % LPA);
+  const bool live = i < m.N;
+  const int* row = m.nbr_h + (live ? i : 0) * m.K;
+  const int cnt = live ? m.cnt_h[i] : 0;
+  const uint4 ui = m.u4[live ? i : 0];
   const float rc2 = (float)(m.rc * m.rc);
-  const int ti = m.types[i];
+  const int ti = (int)ui.w;
   double rho = 0.0;
-  for (int k = 0; k < cnt; ++k) {
+  for (int k = sub; k < cnt; k += LPA) {
     const int j = row[k];
-    const float dx = fix_diff(m.ux[j], uxi, m.ul[0]);
-    const float dy = fix_diff(m.uy[j], uyi, m.ul[1]);
-    const float dz = fix_diff(m.uz[j], uzi, m.ul[2]);
+    const uint4 uj = m.u4[j];
+    const float dx = fix_diff(uj.x, ui.x, m.ul[0]);
+    const float dy = fix_diff(uj.y, ui.y, m.ul[1]);
+    const float dz = fix_diff(uj.z, ui.z, m.ul[2]);
     const float r2 = dx * dx + dy * dy + dz * dz;
     if (r2 >= rc2) continue;
-    const int tj = m.types[j];
+    const int tj = (int)uj.w;
     float t;
     const int q = spline32_locate(m.tab32.sp[3], sqrtf(r2), t, m.err);
     const float fj = spline32_val_at(m.tab32.sp[3 + tj], q, t);
     const float fi = m.same_dens ? fj : spline32_val_at(m.tab32.sp[3 + ti], q, t);
-    rho += (double)fj;
-    atomicAdd(m.rho + j, (double)fi);
+    rho += widen(fj);
+    atomicAdd(m.rho + j, widen(fi));
   }
-  atomicAdd(m.rho + i, rho);
+  rho = lane_sum<LPA>(rho);
+  if (live && sub == 0) atomicAdd(m.rho + i, rho);
 }
 
-__global__ void k_md_force_half32(MdArgs m) {
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= m.N) return;
-  const int* row = m.nbr_h + i * m.K;
-  const int cnt = m.cnt_h[i];
-  const uint32_t uxi = m.ux[i], uyi = m.uy[i], uzi = m.uz[i];
-  const int ti = m.types[i];
-  const float Fi = m.dFp32[i];
+template <int LPA>
+__global__ void __launch_bounds__(128) k_md_force_half32(MdArgs m) {
+  const long long g = (long long)blockIdx.x * 128 + threadIdx.x;
+  const long long i = g / LPA;
+  const int sub = (int)(g % LPA);
+  const bool live = i < m.N;
+  const int* row = m.nbr_h + (live ? i : 0) * m.K;
+  const int cnt = live ? m.cnt_h[i] : 0;
+  const uint4 ui = m.u4[live ? i : 0];
+  const int ti = (int)ui.w;
+  const float Fi = m.dFp32[live ? i : 0];
   const float rc2 = (float)(m.rc * m.rc);
   double fx = 0.0, fy = 0.0, fz = 0.0;
-  for (int k = 0; k < cnt; ++k) {
+  for (int k = sub; k < cnt; k += LPA) {
     const int j = row[k];
-    const float dx = fix_diff(m.ux[j], uxi, m.ul[0]);
-    const float dy = fix_diff(m.uy[j], uyi, m.ul[1]);
-    const float dz = fix_diff(m.uz[j], uzi, m.ul[2]);
+    const uint4 uj = m.u4[j];
+    const float dx = fix_diff(uj.x, ui.x, m.ul[0]);
+    const float dy = fix_diff(uj.y, ui.y, m.ul[1]);
+    const float dz = fix_diff(uj.z, ui.z, m.ul[2]);
     const float r2 = dx * dx + dy * dy + dz * dz;
     if (r2 >= rc2) continue;
     const float ir = rsqrtf(r2);
-    const int tj = m.types[j];
+    const int tj = (int)uj.w;
     float t;
     const int q = spline32_locate(m.tab32.sp[0], r2 * ir, t, m.err);
     const float Fj = m.dFp32[j];
-    float g;
+    float gg;
     if (m.same_dens) {
-      g = fmaf(Fi + Fj, spline32_dval_at(m.tab32.dsp[3], q, t), spline32_dval_at(m.tab32.dsp[ti + tj], q, t));
+      gg = fmaf(Fi + Fj, spline32_dval_at(m.tab32.dsp[3], q, t), spline32_dval_at(m.tab32.dsp[ti + tj], q, t));
     } else {
-      g = fmaf(Fj, spline32_dval_at(m.tab32.dsp[3 + ti], q, t),
-               fmaf(Fi, spline32_dval_at(m.tab32.dsp[3 + tj], q, t), spline32_dval_at(m.tab32.dsp[ti + tj], q, t)));
+      gg = fmaf(Fj, spline32_dval_at(m.tab32.dsp[3 + ti], q, t),
+                fmaf(Fi, spline32_dval_at(m.tab32.dsp[3 + tj], q, t), spline32_dval_at(m.tab32.dsp[ti + tj], q, t)));
     }
-    const float gr = g * ir;
-    const double gx = (double)(gr * dx), gy = (double)(gr * dy), gz = (double)(gr * dz);
+    const float gr = gg * ir;
+    const double gx = widen(gr * dx), gy = widen(gr * dy), gz = widen(gr * dz);
     fx += gx;
     fy += gy;
     fz += gz;
@@ -161,9 +198,14 @@ __global__ void k_md_force_half32(MdArgs m) {
     atomicAdd(m.fz + j, -gz);
   }
   if (!isfinite(fx) || !isfinite(fy) || !isfinite(fz)) atomicOr(m.err, ERRF_NONFINITE);
-  atomicAdd(m.fx + i, fx);
-  atomicAdd(m.fy + i, fy);
-  atomicAdd(m.fz + i, fz);
+  fx = lane_sum<LPA>(fx);
+  fy = lane_sum<LPA>(fy);
+  fz = lane_sum<LPA>(fz);
+  if (live && sub == 0) {
+    atomicAdd(m.fx + i, fx);
+    atomicAdd(m.fy + i, fy);
+    atomicAdd(m.fz + i, fz);
+  }
 }
 
 // F'(rho_i) and F_B(rho_i) - F_A(rho_i) once rho is complete
@@ -192,55 +234,58 @@ __device__ __forceinline__ void add_virial(const MdArgs& m, double vir) {
 // g = phi'_{ti tj} + F'_i f'_{tj} + F'_j f'_{ti} (one density derivative
 // when same_dens); force arrays zeroed before.  The virial term of the
 // pair, r_ij . F_ij = -g r, goes to *m.vir when it is set.
-__device__ __forceinline__ void force_half_row(const MdArgs& m, long long i, double& vir) {
-  const int* row = m.nbr_h + i * m.K;
-  const int cnt = m.cnt_h[i];
-  const double xi = m.x[i], yi = m.y[i], zi = m.z[i];
-  const int ti = m.types[i];
-  const double Fi = m.dFp[i];
-  const double ix = 1.0 / m.box[0], iy = 1.0 / m.box[1], iz = 1.0 / m.box[2];
+template <int LPA, bool SAME, bool VIR>
+__global__ void __launch_bounds__(128) k_md_force_half(MdArgs m) {
+  const long long g = (long long)blockIdx.x * 128 + threadIdx.x;
+  const long long i = g / LPA;
+  const int sub = (int)(g % LPA);
+  const bool live = i < m.N;
+  const int* row = m.nbr_h + (live ? i : 0) * m.K;
+  const int cnt = live ? m.cnt_h[i] : 0;
+  const Cubic pi = m.p4[live ? i : 0];
+  const int ti = record_type(pi);
+  const double Fi = m.dFp[live ? i : 0];
+  const PairBox box = pair_box(m.box);
   const double rc2 = m.rc * m.rc;
-  double fx = 0.0, fy = 0.0, fz = 0.0;
-  for (int k = 0; k < cnt; ++k) {
+  double fx = 0.0, fy = 0.0, fz = 0.0, vir = 0.0;
+  for (int k = sub; k < cnt; k += LPA) {
     const int j = row[k];
-    const double dx = mimg(m.x[j] - xi, m.box[0], ix);
-    const double dy = mimg(m.y[j] - yi, m.box[1], iy);
-    const double dz = mimg(m.z[j] - zi, m.box[2], iz);
-    const double r2 = dx * dx + dy * dy + dz * dz;
-    if (r2 >= rc2) continue;
-    const double ir = rsqrt_nr(r2);
-    const int tj = m.types[j];
-    double t;
-    const int q = locate_in(m.tab.sp[0], r2 * ir, t);
+    const Cubic pj = m.p4[j];
     const double Fj = m.dFp[j];
-    double g;
-    if (m.same_dens) {
-      g = fma(Fi + Fj, spline_dval_at(m.tab.dsp[3], q, t), spline_dval_at(m.tab.dsp[ti + tj], q, t));
+    double dx = pj.x - pi.x, dy = pj.y - pi.y, dz = pj.z - pi.z;
+    const double r2 = pair_r2(box, dx, dy, dz);
+    if (outside(r2, rc2)) continue;
+    double ir, t;
+    const double r = sqrt3(r2, ir);
+    const int tj = record_type(pj);
+    const int q = locate_in(m.tab.sp[0], r, t);
+    double gg;
+    if (SAME) {
+      gg = fma(Fi + Fj, spline_dval_at(m.tab.dsp[3], q, t), spline_dval_at(m.tab.dsp[ti + tj], q, t));
     } else {
-      g = fma(Fj, spline_dval_at(m.tab.dsp[3 + ti], q, t),
-              fma(Fi, spline_dval_at(m.tab.dsp[3 + tj], q, t), spline_dval_at(m.tab.dsp[ti + tj], q, t)));
+      gg = fma(Fj, spline_dval_at(m.tab.dsp[3 + ti], q, t),
+               fma(Fi, spline_dval_at(m.tab.dsp[3 + tj], q, t), spline_dval_at(m.tab.dsp[ti + tj], q, t)));
     }
-    const double gr = g * ir;
+    const double gr = -gg * ir;  // the force on j: a negated operand costs nothing, a negated result a pass
     const double gx = gr * dx, gy = gr * dy, gz = gr * dz;
-    fx += gx;
-    fy += gy;
-    fz += gz;
-    vir -= gr * r2;
-    atomicAdd(m.fx + j, -gx);
-    atomicAdd(m.fy + j, -gy);
-    atomicAdd(m.fz + j, -gz);
+    fx -= gx;
+    fy -= gy;
+    fz -= gz;
+    if (VIR) vir = fma(gr, r2, vir);
+    atomicAdd(m.fx + j, gx);
+    atomicAdd(m.fy + j, gy);
+    atomicAdd(m.fz + j, gz);
   }
   if (!isfinite(fx) || !isfinite(fy) || !isfinite(fz)) atomicOr(m.err, ERRF_NONFINITE);
-  atomicAdd(m.fx + i, fx);
-  atomicAdd(m.fy + i, fy);
-  atomicAdd(m.fz + i, fz);
-}
-
-__global__ void k_md_force_half(MdArgs m) {
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  double vir = 0.0;
-  if (i < m.N) force_half_row(m, i, vir);
-  add_virial(m, vir);
+  fx = lane_sum<LPA>(fx);
+  fy = lane_sum<LPA>(fy);
+  fz = lane_sum<LPA>(fz);
+  if (live && sub == 0) {
+    atomicAdd(m.fx + i, fx);
+    atomicAdd(m.fy + i, fy);
+    atomicAdd(m.fz + i, fz);
+  }
+  if (VIR) add_virial(m, vir);
 }
 
 template <bool MIXED>
@@ -309,11 +354,38 @@ __global__ void k_md_force(MdArgs m) {
   if (!MIXED) add_virial(m, vir);
 }
 
+// v - L floor(v / L): a drift leaves the box by less than its length but for
+// runaway atoms, so the division (a dozen FP64 instructions) is the exception
 __device__ __forceinline__ double wrap_box(double v, double L) {
-  double w = v - L * floor(v / L);
+  double w = v;
+  if (v < 0.0) w = v + L;
+  else if (v >= L) w = v - L;
+  if (!(w >= 0.0 && w <= L)) w = v - L * floor(v / L);
   if (w >= L) w -= L;
   if (w < 0.0) w = 0.0;
   return w;
+}
+// minimum image of a difference of two positions in [0, L)
+__device__ __forceinline__ double mimg_box(double d, double L) {
+  return d > 0.5 * L ? d - L : (d < -0.5 * L ? d + L : d);
+}
+// largest squared displacement: block maximum, then one atomic per block (one
+// per atom on a single address took most of a drift kernel's time).
+// Non-negative doubles order like their bit patterns.
+__device__ __forceinline__ void max_displacement(const MdArgs& m, double d2) {
+  unsigned long long b = (unsigned long long)__double_as_longlong(d2);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const unsigned long long q = __shfl_xor_sync(0xffffffffu, b, o);
+    b = q > b ? q : b;
+  }
+  __shared__ unsigned long long s_max[4];
+  if ((threadIdx.x & 31) == 0) s_max[threadIdx.x >> 5] = b;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < 4; ++w) b = s_max[w] > b ? s_max[w] : b;
+    atomicMax(m.max_disp2_bits, b);
+  }
 }
 
 // Box-Muller: two standard normals from two uniforms
@@ -327,48 +399,49 @@ __device__ __forceinline__ void normals(uint4 w, double& z0, double& z1) {
   z1 = rr * s;
 }
 
-__global__ void k_md_first_half(MdArgs m, long long step) {
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= m.N) return;
-  const int ti = m.types[i];
-  const double im = FTM / m.mass[ti];
-  const double h = 0.5 * m.dt;
-  double vx = m.vx[i] + h * m.fx[i] * im;
-  double vy = m.vy[i] + h * m.fy[i] * im;
-  double vz = m.vz[i] + h * m.fz[i] * im;
-  double x = m.x[i] + h * vx, y = m.y[i] + h * vy, z = m.z[i] + h * vz;
-  if (m.c2 > 0.0) {
-    const double sig = m.c2 * sqrt(m.kT * im);
-    const uint4 c0 = make_uint4((uint32_t)step, (uint32_t)((uint64_t)step >> 32), (uint32_t)i, TAG_NOISE0);
-    const uint4 c1 = make_uint4((uint32_t)step, (uint32_t)((uint64_t)step >> 32), (uint32_t)i, TAG_NOISE1);
-    double z0, z1, z2, z3;
-    normals(philox4x32_10(c0, m.key), z0, z1);
-    normals(philox4x32_10(c1, m.key), z2, z3);
-    vx = m.c1 * vx + sig * z0;
-    vy = m.c1 * vy + sig * z1;
-    vz = m.c1 * vz + sig * z2;
+__global__ void __launch_bounds__(128) k_md_first_half(MdArgs m, long long step) {
+  const long long i = (long long)blockIdx.x * 128 + threadIdx.x;
+  double d2 = 0.0;
+  if (i < m.N) {
+    const int ti = m.types[i];
+    const double im = m.im[ti];
+    const double h = 0.5 * m.dt;
+    double vx = m.vx[i] + h * m.fx[i] * im;
+    double vy = m.vy[i] + h * m.fy[i] * im;
+    double vz = m.vz[i] + h * m.fz[i] * im;
+    double x = m.x[i] + h * vx, y = m.y[i] + h * vy, z = m.z[i] + h * vz;
+    if (m.c2 > 0.0) {
+      const double sig = m.sig[ti];  // c2 sqrt(kT / mass)
+      const uint4 c0 = make_uint4((uint32_t)step, (uint32_t)((uint64_t)step >> 32), (uint32_t)i, TAG_NOISE0);
+      const uint4 c1 = make_uint4((uint32_t)step, (uint32_t)((uint64_t)step >> 32), (uint32_t)i, TAG_NOISE1);
+      double z0, z1, z2, z3;
+      normals(philox4x32_10(c0, m.key), z0, z1);
+      normals(philox4x32_10(c1, m.key), z2, z3);
+      vx = m.c1 * vx + sig * z0;
+      vy = m.c1 * vy + sig * z1;
+      vz = m.c1 * vz + sig * z2;
+    }
+    x = wrap_box(x + h * vx, m.box[0]);
+    y = wrap_box(y + h * vy, m.box[1]);
+    z = wrap_box(z + h * vz, m.box[2]);
+    m.vx[i] = vx;
+    m.vy[i] = vy;
+    m.vz[i] = vz;
+    m.x[i] = x;
+    m.y[i] = y;
+    m.z[i] = z;
+    const double dx = mimg_box(x - m.x0[i], m.box[0]);
+    const double dy = mimg_box(y - m.y0[i], m.box[1]);
+    const double dz = mimg_box(z - m.z0[i], m.box[2]);
+    d2 = dx * dx + dy * dy + dz * dz;
   }
-  x = wrap_box(x + h * vx, m.box[0]);
-  y = wrap_box(y + h * vy, m.box[1]);
-  z = wrap_box(z + h * vz, m.box[2]);
-  m.vx[i] = vx;
-  m.vy[i] = vy;
-  m.vz[i] = vz;
-  m.x[i] = x;
-  m.y[i] = y;
-  m.z[i] = z;
-  const double dx = mimg(x - m.x0[i], m.box[0], 1.0 / m.box[0]);
-  const double dy = mimg(y - m.y0[i], m.box[1], 1.0 / m.box[1]);
-  const double dz = mimg(z - m.z0[i], m.box[2], 1.0 / m.box[2]);
-  const double d2 = dx * dx + dy * dy + dz * dz;
-  // non-negative doubles order like their bit patterns
-  atomicMax(m.max_disp2_bits, (unsigned long long)__double_as_longlong(d2));
+  max_displacement(m, d2);
 }
 
 __global__ void k_md_second_half(MdArgs m) {
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= m.N) return;
-  const double im = FTM / m.mass[m.types[i]];
+  const double im = m.im[m.types[i]];
   const double h = 0.5 * m.dt;
   m.vx[i] += h * m.fx[i] * im;
   m.vy[i] += h * m.fy[i] * im;
@@ -391,44 +464,50 @@ __global__ void k_md_snapshot(MdArgs m) {
 __global__ void k_nh_kick(MdArgs m, double s, double e1, double he2) {
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= m.N) return;
-  const double im = FTM / m.mass[m.types[i]];
+  const double im = m.im[m.types[i]];
   const double se = s * e1, ke = he2 * im;
   m.vx[i] = fma(m.vx[i], se, m.fx[i] * ke);
   m.vy[i] = fma(m.vy[i], se, m.fy[i] * ke);
   m.vz[i] = fma(m.vz[i], se, m.fz[i] * ke);
 }
 
-__global__ void k_nh_drift(MdArgs m, double e1, double e2dt) {
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= m.N) return;
-  const double x = wrap_box(fma(m.x[i], e1, m.vx[i] * e2dt), m.box[0]);
-  const double y = wrap_box(fma(m.y[i], e1, m.vy[i] * e2dt), m.box[1]);
-  const double z = wrap_box(fma(m.z[i], e1, m.vz[i] * e2dt), m.box[2]);
-  m.x[i] = x;
-  m.y[i] = y;
-  m.z[i] = z;
-  const double dx = mimg(x - m.x0[i] * m.lam, m.box[0], 1.0 / m.box[0]);
-  const double dy = mimg(y - m.y0[i] * m.lam, m.box[1], 1.0 / m.box[1]);
-  const double dz = mimg(z - m.z0[i] * m.lam, m.box[2], 1.0 / m.box[2]);
-  atomicMax(m.max_disp2_bits, (unsigned long long)__double_as_longlong(dx * dx + dy * dy + dz * dz));
+__global__ void __launch_bounds__(128) k_nh_drift(MdArgs m, double e1, double e2dt) {
+  const long long i = (long long)blockIdx.x * 128 + threadIdx.x;
+  double d2 = 0.0;
+  if (i < m.N) {
+    const double x = wrap_box(fma(m.x[i], e1, m.vx[i] * e2dt), m.box[0]);
+    const double y = wrap_box(fma(m.y[i], e1, m.vy[i] * e2dt), m.box[1]);
+    const double z = wrap_box(fma(m.z[i], e1, m.vz[i] * e2dt), m.box[2]);
+    m.x[i] = x;
+    m.y[i] = y;
+    m.z[i] = z;
+    const double dx = mimg(x - m.x0[i] * m.lam, m.box[0], 1.0 / m.box[0]);
+    const double dy = mimg(y - m.y0[i] * m.lam, m.box[1], 1.0 / m.box[1]);
+    const double dz = mimg(z - m.z0[i] * m.lam, m.box[2], 1.0 / m.box[2]);
+    d2 = dx * dx + dy * dy + dz * dz;
+  }
+  max_displacement(m, d2);
 }
 
 // positions x0 + alpha d (conjugate-gradient line search), wrapped, with the
 // displacement check of the MD step
-__global__ void k_cg_place(MdArgs m, const double* x0, const double* d, double alpha) {
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= m.N) return;
-  const long long N = m.N;
-  const double x = wrap_box(fma(alpha, d[i], x0[i]), m.box[0]);
-  const double y = wrap_box(fma(alpha, d[N + i], x0[N + i]), m.box[1]);
-  const double z = wrap_box(fma(alpha, d[2 * N + i], x0[2 * N + i]), m.box[2]);
-  m.x[i] = x;
-  m.y[i] = y;
-  m.z[i] = z;
-  const double dx = mimg(x - m.x0[i], m.box[0], 1.0 / m.box[0]);
-  const double dy = mimg(y - m.y0[i], m.box[1], 1.0 / m.box[1]);
-  const double dz = mimg(z - m.z0[i], m.box[2], 1.0 / m.box[2]);
-  atomicMax(m.max_disp2_bits, (unsigned long long)__double_as_longlong(dx * dx + dy * dy + dz * dz));
+__global__ void __launch_bounds__(128) k_cg_place(MdArgs m, const double* x0, const double* d, double alpha) {
+  const long long i = (long long)blockIdx.x * 128 + threadIdx.x;
+  double d2 = 0.0;
+  if (i < m.N) {
+    const long long N = m.N;
+    const double x = wrap_box(fma(alpha, d[i], x0[i]), m.box[0]);
+    const double y = wrap_box(fma(alpha, d[N + i], x0[N + i]), m.box[1]);
+    const double z = wrap_box(fma(alpha, d[2 * N + i], x0[2 * N + i]), m.box[2]);
+    m.x[i] = x;
+    m.y[i] = y;
+    m.z[i] = z;
+    const double dx = mimg_box(x - m.x0[i], m.box[0]);
+    const double dy = mimg_box(y - m.y0[i], m.box[1]);
+    const double dz = mimg_box(z - m.z0[i], m.box[2]);
+    d2 = dx * dx + dy * dy + dz * dz;
+  }
+  max_displacement(m, d2);
 }
 
 constexpr int DOT_BLOCK = 256;
@@ -501,12 +580,37 @@ void launch_fix_positions(long long N, const double* x, const double* y, const d
                                               uz);
 }
 
+// lanes per atom of the half-list passes: 4, or 16 while 4 leave the GPU short
+// of warps (a row is then a chain of two pairs).  Below 20000 atoms 4 lanes are
+// under 2500 warps, 16 per SM.  A step of 3456 atoms took 294 us with a thread
+// per atom and 97 with 16 lanes.
+constexpr long long MD_FEW = 20000;
+
+template <int LPA>
+static void rho_half(const MdArgs& m, cudaStream_t st) {
+  const unsigned g = grid_of(m.N * LPA);
+  if (m.mixed) k_md_rho_half32<LPA><<<g, 128, 0, st>>>(m);
+  else if (m.same_dens) k_md_rho_half<LPA, true><<<g, 128, 0, st>>>(m);
+  else k_md_rho_half<LPA, false><<<g, 128, 0, st>>>(m);
+}
+
+template <int LPA>
+static void force_half(const MdArgs& m, cudaStream_t st) {
+  const unsigned g = grid_of(m.N * LPA);
+  if (m.mixed) k_md_force_half32<LPA><<<g, 128, 0, st>>>(m);
+  else if (m.vir && m.same_dens) k_md_force_half<LPA, true, true><<<g, 128, 0, st>>>(m);
+  else if (m.vir) k_md_force_half<LPA, false, true><<<g, 128, 0, st>>>(m);
+  else if (m.same_dens) k_md_force_half<LPA, true, false><<<g, 128, 0, st>>>(m);
+  else k_md_force_half<LPA, false, false><<<g, 128, 0, st>>>(m);
+}
+
 void launch_md_rho(const MdArgs& m, cudaStream_t st) {
   if (m.mixed) launch_fix_positions(m.N, m.x, m.y, m.z, m.box, m.ux, m.uy, m.uz, st);
   if (m.nbr_h) {
+    k_md_records<<<grid_of(m.N), 128, 0, st>>>(m);
     cudaMemsetAsync(m.rho, 0, sizeof(double) * m.N, st);
-    if (m.mixed) k_md_rho_half32<<<grid_of(m.N), 128, 0, st>>>(m);
-    else k_md_rho_half<<<grid_of(m.N), 128, 0, st>>>(m);
+    if (m.N < MD_FEW) rho_half<16>(m, st);
+    else rho_half<4>(m, st);
     k_md_embed<<<grid_of(m.N), 128, 0, st>>>(m);
   } else if (m.mixed) {
     k_md_rho<true><<<grid_of(m.N), 128, 0, st>>>(m);
@@ -516,11 +620,9 @@ void launch_md_rho(const MdArgs& m, cudaStream_t st) {
 }
 void launch_md_force(const MdArgs& m, cudaStream_t st) {
   if (m.nbr_h) {
-    cudaMemsetAsync(m.fx, 0, sizeof(double) * m.N, st);
-    cudaMemsetAsync(m.fy, 0, sizeof(double) * m.N, st);
-    cudaMemsetAsync(m.fz, 0, sizeof(double) * m.N, st);
-    if (m.mixed) k_md_force_half32<<<grid_of(m.N), 128, 0, st>>>(m);
-    else k_md_force_half<<<grid_of(m.N), 128, 0, st>>>(m);
+    cudaMemsetAsync(m.fx, 0, sizeof(double) * 3 * m.N, st);
+    if (m.N < MD_FEW) force_half<16>(m, st);
+    else force_half<4>(m, st);
   } else if (m.mixed) {
     k_md_force<true><<<grid_of(m.N), 128, 0, st>>>(m);
   } else {

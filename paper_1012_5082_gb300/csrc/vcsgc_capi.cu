@@ -53,6 +53,8 @@ struct Ctx {
   double *fx = nullptr, *fy = nullptr, *fz = nullptr;
   double *x0 = nullptr, *y0 = nullptr, *z0 = nullptr;
   uint32_t *ux = nullptr, *uy = nullptr, *uz = nullptr;  // fixed-point positions (mixed, kind 1)
+  Cubic* p4 = nullptr;             // records of the half-list passes (FP64, mixed)
+  uint4* u4 = nullptr;
   unsigned long long* max_disp2 = nullptr;
   int* nbr = nullptr;
   int* nbr_cnt = nullptr;
@@ -98,6 +100,7 @@ struct Ctx {
   double dt = 2.0, gamma = 0.01, T_md = 0.0;
   uint64_t md_seed = 0;
   bool forces_valid = false;
+  bool vir_valid = false;  // d_vir belongs to the forces
   // Nose-Hoover chains and the MTK barostat (kind 0: Langevin BAOAB)
   struct Nh {
     int kind = 0, chain = 3;
@@ -320,6 +323,8 @@ void fill_args(Ctx* c) {
   m.x = c->x; m.y = c->y; m.z = c->z;
   m.vx = c->vx; m.vy = c->vy; m.vz = c->vz;
   m.fx = c->fx; m.fy = c->fy; m.fz = c->fz;
+  m.p4 = c->p4;
+  m.u4 = c->u4;
   m.rho = c->rho;
   m.dFp = c->dFp;
   m.dF = c->dF;
@@ -336,6 +341,10 @@ void fill_args(Ctx* c) {
   m.c1 = std::exp(-c->gamma * c->dt);
   m.c2 = std::sqrt(std::max(0.0, 1.0 - m.c1 * m.c1));
   m.kT = KB_EV * c->T_md;
+  for (int q = 0; q < 2; ++q) {
+    m.im[q] = FTM / m.mass[q];
+    m.sig[q] = m.c2 * std::sqrt(m.kT * m.im[q]);
+  }
   m.key = make_uint2((uint32_t)c->md_seed, (uint32_t)(c->md_seed >> 32));
   m.tab = c->mc.tab;
   m.tab32 = c->mc.tab32;
@@ -1076,12 +1085,16 @@ int push_to_multi(Ctx* c, int r, const uint8_t* host_types, const RepState* s) {
 }
 
 // ------------------------------------------------------------------- MD
-int md_forces(Ctx* c) {
-  if (c->d_vir) CK(cudaMemsetAsync(c->d_vir, 0, sizeof(double), c->st));
-  launch_md_rho(c->md, c->st);
-  launch_md_force(c->md, c->st);
+// forces and, where the caller reads it (vir), the virial
+int md_forces(Ctx* c, bool vir = false) {
+  MdArgs m = c->md;
+  if (!vir) m.vir = nullptr;
+  if (m.vir) CK(cudaMemsetAsync(m.vir, 0, sizeof(double), c->st));
+  launch_md_rho(m, c->st);
+  launch_md_force(m, c->st);
   CK(cudaGetLastError());
   c->forces_valid = true;
+  c->vir_valid = vir;
   return VCSGC_OK;
 }
 
@@ -1157,10 +1170,10 @@ int md_run_nh(Ctx* c, long long n) {
   const bool npt = nh.kind == 2;
   const double dt = c->dt, h = 0.5 * dt, kT = KB_EV * c->T_md, nf = 3.0 * (double)c->N;
   const double alpha = 1.0 + 3.0 / nf;
-  if (!c->forces_valid) TRY(md_forces(c));
+  if (!c->forces_valid || (npt && !c->vir_valid)) TRY(md_forces(c, npt));
   double K2 = 0.0, vir = 0.0;
   TRY(twice_ke_dev(c, &K2));
-  TRY(read_virial(c, &vir));
+  if (npt) TRY(read_virial(c, &vir));
   for (long long q = 0; q < n; ++q) {
     // thermostats, barostat velocity, velocity half kick
     const double s1 = nhc_step(nh.chain, nh.Q, nh.xi, nh.eta, K2, nf * kT, kT, h);
@@ -1190,7 +1203,7 @@ int md_run_nh(Ctx* c, long long n) {
       TRY(md_rebuild(c));
       fill_args(c);
     }
-    TRY(md_forces(c));
+    TRY(md_forces(c, npt));
     launch_nh_kick(c->md, 1.0, e1, he2, c->st);
     CK(cudaGetLastError());
     TRY(twice_ke_dev(c, &K2));
@@ -1227,8 +1240,7 @@ int md_run(Ctx* c, long long n) {
     double d2;
     std::memcpy(&d2, &bits, sizeof(d2));
     if (d2 > half_skin2) TRY(md_rebuild(c));
-    launch_md_rho(c->md, c->st);
-    launch_md_force(c->md, c->st);
+    TRY(md_forces(c));
     launch_md_second_half(c->md, c->st);
     CK(cudaGetLastError());
     c->md_step++;
@@ -1498,9 +1510,13 @@ static int init_impl(Ctx* c, const vcsgc_lattice* L, const uint8_t* types, const
   TRY(dalloc(c, &c->dF, c->N));
   TRY(dalloc(c, &c->dFp, c->N));
   TRY(dalloc(c, &c->dFp32, c->N));
-  TRY(dalloc(c, &c->fx, c->N));
-  TRY(dalloc(c, &c->fy, c->N));
-  TRY(dalloc(c, &c->fz, c->N));
+  TRY(dalloc(c, &c->fx, 3 * c->N));
+  c->fy = c->fx + c->N;
+  c->fz = c->fy + c->N;
+  if (c->kind == 1 && c->R == 1) {
+    if (c->mixed) TRY(dalloc(c, &c->u4, c->N));
+    else TRY(dalloc(c, &c->p4, c->N));
+  }
   TRY(dalloc(c, &c->x0, c->N));
   TRY(dalloc(c, &c->y0, c->N));
   TRY(dalloc(c, &c->z0, c->N));
@@ -2867,7 +2883,7 @@ int vcsgc_md_state(void* ctx, double* out) {
   double K2 = 0.0, pe = 0.0, vir = 0.0;
   if (c->have_v) TRY(twice_ke_dev(c, &K2));
   TRY(energy_of(c, 0, &pe));
-  TRY(md_forces(c));
+  TRY(md_forces(c, true));
   TRY(read_virial(c, &vir));
   TRY(check_device_error(c));
   const Ctx::Nh& nh = c->nh;
