@@ -15,6 +15,7 @@
 #include "common.cuh"
 #include "kernels.h"
 #include "multi_host.h"
+#include "readout.h"
 #include "screen.h"
 #include "trace.h"
 
@@ -2591,7 +2592,7 @@ int vcsgc_get_types(void* ctx, int32_t r, uint8_t* out) {
   Ctx* c = static_cast<Ctx*>(ctx);
   if (!c || !out || r < 0 || r >= c->R) return VCSGC_ERR_INVALID_ARG;
   TRY(sync_bytes(c, r));
-  CK(cudaMemcpyAsync(out, c->rep_types[r], c->rep_n[r], cudaMemcpyDeviceToHost, c->st));
+  CK(read_back(out, c->rep_types[r], c->rep_n[r], c->st));
   return check_device_error(c);
 }
 
@@ -2693,8 +2694,9 @@ int vcsgc_get_types_all(void* ctx, uint8_t* out) {
     off += c->rep_n[r];
   }
   if (contiguous) {
-    CK(cudaMemcpyAsync(out, c->rep_types[0], off, cudaMemcpyDeviceToHost, c->st));
+    CK(read_back(out, c->rep_types[0], off, c->st));
   } else {
+    make_present(&out, 1, off);
     off = 0;
     for (int r = 0; r < c->R; ++r) {
       CK(cudaMemcpyAsync(out + off, c->rep_types[r], c->rep_n[r], cudaMemcpyDeviceToHost, c->st));
@@ -2752,7 +2754,7 @@ int vcsgc_get_rho(void* ctx, int32_t r, double* out) {
   TRY(sync_from_multi(c));
   if (!c->subs.empty()) return vcsgc_get_rho(c->subs[r], 0, out);
   const double* src = c->rho + (c->reembed ? (long long)r * c->N : 0);
-  CK(cudaMemcpyAsync(out, src, sizeof(double) * c->N, cudaMemcpyDeviceToHost, c->st));
+  CK(read_back(out, src, sizeof(double) * c->N, c->st));
   return check_device_error(c);
 }
 
@@ -2780,7 +2782,7 @@ int vcsgc_delta_e(void* ctx, int32_t r, const int64_t* sites, int64_t n, double*
     launch_delta_e_list(c->mc, c->shell, c->reembed, r, c->sites_buf, (int)n, c->de_buf, c->st);
   }
   CK(cudaGetLastError());
-  CK(cudaMemcpyAsync(out, c->de_buf, sizeof(double) * n, cudaMemcpyDeviceToHost, c->st));
+  CK(read_back(out, c->de_buf, sizeof(double) * n, c->st));
   return check_device_error(c);
 }
 
@@ -2797,6 +2799,8 @@ int vcsgc_forces(void* ctx, double* fx, double* fy, double* fz) {
   if (!c || !fx || !fy || !fz) return VCSGC_ERR_INVALID_ARG;
   if (!c->subs.empty()) return fail(c, VCSGC_ERR_STATE, "forces are not defined for a batch");
   if (!c->forces_valid) TRY(md_forces(c));
+  double* const f[3] = {fx, fy, fz};
+  make_present(f, 3, sizeof(double) * c->N);
   CK(cudaMemcpyAsync(fx, c->fx, sizeof(double) * c->N, cudaMemcpyDeviceToHost, c->st));
   CK(cudaMemcpyAsync(fy, c->fy, sizeof(double) * c->N, cudaMemcpyDeviceToHost, c->st));
   CK(cudaMemcpyAsync(fz, c->fz, sizeof(double) * c->N, cudaMemcpyDeviceToHost, c->st));
@@ -2809,6 +2813,7 @@ int vcsgc_get_md(void* ctx, double* x, double* y, double* z, double* vx, double*
   if (!c->subs.empty()) return fail(c, VCSGC_ERR_STATE, "positions are per replica in a batch");
   double* dst[6] = {x, y, z, vx, vy, vz};
   double* src[6] = {c->x, c->y, c->z, c->vx, c->vy, c->vz};
+  make_present(dst, 6, sizeof(double) * c->N);  // before the first copy, which waits for the device
   for (int q = 0; q < 6; ++q) {
     if (!dst[q]) continue;
     if (!src[q]) return fail(c, VCSGC_ERR_STATE, "velocities not set");

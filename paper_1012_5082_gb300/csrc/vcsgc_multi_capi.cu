@@ -10,6 +10,7 @@
 
 #include "kernels.h"
 #include "multi.cuh"
+#include "readout.h"
 #include "screen.h"
 #include "trace.h"
 #include "vcsgc.h"
@@ -736,7 +737,7 @@ int vcsgc_multi_get_types(void* h, int32_t r, uint8_t* out) {
   if (!m || !out || r < 0 || r >= m->R) return VCSGC_ERR_INVALID_ARG;
   MCK(cudaSetDevice(m->device));
   MTRY(flush(m));
-  MCK(cudaMemcpyAsync(out, m->args.types + (long long)r * m->N, m->N, cudaMemcpyDeviceToHost, m->st));
+  MCK(read_back(out, m->args.types + (long long)r * m->N, m->N, m->st));
   MCK(cudaStreamSynchronize(m->st));
   return VCSGC_OK;
 }
@@ -768,7 +769,7 @@ int vcsgc_multi_delta_e(void* h, int32_t r, const int64_t* sites, const uint8_t*
   MCK(cudaMemcpyAsync(m->d_to, to, n, cudaMemcpyHostToDevice, m->st));
   launch_multi_delta_e(m->args, r, m->d_sites, m->d_to, (int)n, m->d_out, m->st);
   MCK(cudaGetLastError());
-  MCK(cudaMemcpyAsync(out, m->d_out, sizeof(double) * n, cudaMemcpyDeviceToHost, m->st));
+  MCK(read_back(out, m->d_out, sizeof(double) * n, m->st));
   MCK(cudaStreamSynchronize(m->st));
   return device_error(m);
 }
@@ -893,7 +894,7 @@ int multi_get_rho(void* h, int r, double* out) {
   if (!m || !out || r < 0 || r >= m->R) return VCSGC_ERR_INVALID_ARG;
   MCK(cudaSetDevice(m->device));
   MTRY(flush(m));
-  MCK(cudaMemcpyAsync(out, m->args.rho + (long long)r * m->N, sizeof(double) * m->N, cudaMemcpyDeviceToHost, m->st));
+  MCK(read_back(out, m->args.rho + (long long)r * m->N, sizeof(double) * m->N, m->st));
   MCK(cudaStreamSynchronize(m->st));
   return VCSGC_OK;
 }
