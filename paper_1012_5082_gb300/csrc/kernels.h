@@ -41,17 +41,15 @@ void launch_lattice_energy_table(Tables tab, const Tables32* tab32, const double
 void launch_lattice_neighbours(int nx, int ny, int nz, const int3* hoff, int K, int* nbr, int* cnt,
                                cudaStream_t st);
 // Explicit positions: cell binning (side >= rl, >= 3 cells per axis) and a
-// full neighbour list within rl; rows longer than K set ERRF_OVERFLOW.
+// full neighbour list within rl; rows longer than K set ERRF_OVERFLOW.  nbr_h,
+// cnt_h (null: not wanted): its entries j > i, with the same stride.
 struct CellList {
   int nc[3];
-  float* x32;      // [N] float copies of the positions (list criterion only)
-  float* y32;
-  float* z32;
+  float4* p4;      // [N] cell-sorted (x, y, z as floats, index)
   int* cell_of;    // [N]
   int* cell_count; // [ncell]
   int* cell_start; // [ncell + 1]
   int* cell_cursor;// [ncell]
-  int* sorted;     // [N]
 };
 // Distance margin of the list's FP32 criterion: rows hold every pair within
 // rl and may hold pairs up to rl + cell_list_margin(box).
@@ -61,7 +59,7 @@ inline double cell_list_margin(const double box[3]) {
 }
 void launch_cell_neighbours(long long N, const double* x, const double* y, const double* z,
                             const double box[3], double rl, CellList cl, int K, int* nbr, int* cnt,
-                            unsigned* err, cudaStream_t st);
+                            int* nbr_h, int* cnt_h, unsigned* err, cudaStream_t st);
 // SPATIAL colour schedule on the device: dom_start[ndom + 1] and
 // dom_sites[N] (atoms by domain, ascending within one) from the positions;
 // dom_of_block[nb0 nb1 nb2] gives each box's domain rank; dom_of[N],
@@ -69,9 +67,6 @@ void launch_cell_neighbours(long long N, const double* x, const double* y, const
 void launch_spatial_schedule(long long N, const double* x, const double* y, const double* z, const double box[3],
                              const int nb[3], const int* dom_of_block, int ndom, int* dom_of, int* count,
                              int* cursor, int* dom_start, int* dom_sites, cudaStream_t st);
-// half list: the entries j > i of each full row (same stride K)
-void launch_half_list(long long N, int K, const int* nbr, const int* cnt, int* nbr_h, int* cnt_h,
-                      cudaStream_t st);
 
 // ---- density, energy (kernels_nbr.cu)
 // rho_i of replica r (shared array when !per_rep) and, if dF != nullptr,

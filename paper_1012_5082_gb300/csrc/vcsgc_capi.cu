@@ -244,6 +244,17 @@ int dalloc(Ctx* c, T** p, size_t count) {
     if (rc_ != VCSGC_OK) return rc_; \
   } while (0)
 
+// gives a buffer of dalloc back before the context closes
+template <typename T>
+void dfree(Ctx* c, T** p) {
+  const auto it = std::find(c->allocs.begin(), c->allocs.end(), (void*)*p);
+  if (*p && it != c->allocs.end()) {
+    cudaFree(*p);
+    c->allocs.erase(it);
+  }
+  *p = nullptr;
+}
+
 // the device error bits e (already copied to the host) as a status
 int device_error_status(Ctx* c, unsigned e) {
   if (!e) return VCSGC_OK;
@@ -402,11 +413,8 @@ int build_cell_list(Ctx* c) {
   }
   const int ncell = c->cl.nc[0] * c->cl.nc[1] * c->cl.nc[2];
   if (!c->cl.cell_of) {
-    TRY(dalloc(c, &c->cl.x32, c->N));
-    TRY(dalloc(c, &c->cl.y32, c->N));
-    TRY(dalloc(c, &c->cl.z32, c->N));
+    TRY(dalloc(c, &c->cl.p4, c->N));
     TRY(dalloc(c, &c->cl.cell_of, c->N));
-    TRY(dalloc(c, &c->cl.sorted, c->N));
   }
   if (ncell > c->ncell_cap) {
     // the box can grow under a barostat
@@ -416,27 +424,23 @@ int build_cell_list(Ctx* c) {
     c->ncell_cap = ncell;
   }
   for (int attempt = 0; attempt < 6; ++attempt) {
+    if (c->R == 1 && c->K_h != c->K) {
+      // half list for the MD passes (each pair once)
+      dfree(c, &c->nbr_h);
+      c->K_h = 0;
+      TRY(dalloc(c, &c->nbr_h, (size_t)c->N * c->K));
+      if (!c->cnt_h) TRY(dalloc(c, &c->cnt_h, c->N));
+      c->K_h = c->K;
+      fill_args(c);
+    }
     CK(cudaMemsetAsync(c->derr, 0, sizeof(unsigned), c->st));
     launch_cell_neighbours(c->N, c->x, c->y, c->z, c->box, c->rl, c->cl, c->K, c->nbr, c->nbr_cnt,
-                           c->derr, c->st);
+                           c->R == 1 ? c->nbr_h : nullptr, c->cnt_h, c->derr, c->st);
     CK(cudaGetLastError());
     unsigned e = 0;
     CK(cudaMemcpyAsync(&e, c->derr, sizeof(unsigned), cudaMemcpyDeviceToHost, c->st));
     CK(cudaStreamSynchronize(c->st));
-    if (!(e & ERRF_OVERFLOW)) {
-      if (c->R == 1) {
-        // half list for the MD passes (each pair once)
-        if (c->K_h != c->K) {
-          TRY(dalloc(c, &c->nbr_h, (size_t)c->N * c->K));
-          if (!c->cnt_h) TRY(dalloc(c, &c->cnt_h, c->N));
-          c->K_h = c->K;
-          fill_args(c);
-        }
-        launch_half_list(c->N, c->K, c->nbr, c->nbr_cnt, c->nbr_h, c->cnt_h, c->st);
-        CK(cudaGetLastError());
-      }
-      return VCSGC_OK;
-    }
+    if (!(e & ERRF_OVERFLOW)) return VCSGC_OK;
     // grow the rows and rebuild
     const int K2 = ((c->K * 3 / 2) + 7) / 8 * 8;
     int* nb = nullptr;

@@ -28,8 +28,7 @@ using vcsgc::CellList;
 constexpr long long NL_MAX_ATOMS = 262144;  // 2^18 positions
 constexpr long long NL_MAX_CELLS = 65536;   // 2^16 binning cells
 
-// layout (4-byte words): x32, y32, z32 [MAX_ATOMS each, float] |
-//         cell_of[MAX_ATOMS] | sorted[MAX_ATOMS] | count[MAX_CELLS] |
+// layout (4-byte words): p4[MAX_ATOMS float4] | cell_of[MAX_ATOMS] | count[MAX_CELLS] |
 //         start[MAX_CELLS + 1] | cursor[MAX_CELLS] | err (one word)
 constexpr long long NL_SCRATCH_INTS = 5 * NL_MAX_ATOMS + 3 * NL_MAX_CELLS + 1 + 1;
 
@@ -82,11 +81,8 @@ extern "C" int vcsgc_neighbour_list_noalloc(int64_t n, const double* d_x, const 
   cl.nc[0] = nc[0];
   cl.nc[1] = nc[1];
   cl.nc[2] = nc[2];
-  cl.x32 = reinterpret_cast<float*>(base);
-  cl.y32 = reinterpret_cast<float*>(base + NL_MAX_ATOMS);
-  cl.z32 = reinterpret_cast<float*>(base + 2 * NL_MAX_ATOMS);
-  cl.cell_of = base + 3 * NL_MAX_ATOMS;
-  cl.sorted = base + 4 * NL_MAX_ATOMS;
+  cl.p4 = reinterpret_cast<float4*>(base);
+  cl.cell_of = base + 4 * NL_MAX_ATOMS;
   cl.cell_count = base + 5 * NL_MAX_ATOMS;
   cl.cell_start = cl.cell_count + NL_MAX_CELLS;
   cl.cell_cursor = cl.cell_start + NL_MAX_CELLS + 1;
@@ -94,7 +90,7 @@ extern "C" int vcsgc_neighbour_list_noalloc(int64_t n, const double* d_x, const 
   // counts and cursors are cleared by the build itself; the error word here
   e = cudaMemsetAsync(err, 0, sizeof(unsigned), st);
   if (e != cudaSuccess) return nl_fail_cuda("cudaMemsetAsync", e);
-  vcsgc::launch_cell_neighbours(n, d_x, d_y, d_z, box, rl, cl, K, d_nbr, d_cnt, err, st);
+  vcsgc::launch_cell_neighbours(n, d_x, d_y, d_z, box, rl, cl, K, d_nbr, d_cnt, nullptr, nullptr, err, st);
   e = cudaGetLastError();
   if (e != cudaSuccess) return nl_fail_cuda("launch", e);
   unsigned h_err = 0;
