@@ -174,11 +174,15 @@ __device__ __forceinline__ float narrow_pos(double d) {
 // r = sqrt(r2), and 1/r: y = rsqrt(r2) in FP32 from the truncated bits (relative
 // error below 2^-21), then one third-order step, with e = 1 - r2 y^2:
 //   sqrt(r2) = r2 y (1 + e/2 + 3 e^2 / 8 + O(e^3)), e^3 < 2^-59
-// -- five FP64 operations for r, six for both, where two Newton steps with
-// their two conversions took eleven.
+// -- four FP64 operations for r, five for both, where two Newton steps with
+// their two conversions took eleven.  The term 3 e^2 / 8 < 2^-41 is formed in
+// FP32 (below 2^-63 of the result).
 __device__ __forceinline__ double sqrt3(double r2, double& ir) {
   const double y = widen(rsqrtf(narrow_pos(r2)));
-  const double s = r2 * y, e = fma(-s, y, 1.0), q = e * fma(0.375, e, 0.5);
+  const double s = r2 * y, e = fma(-s, y, 1.0);
+  const uint32_t eh = (uint32_t)__double2hiint(e) & 0x7FFFFFFFu;
+  const float ea = eh < 0x38100000u ? 0.0f : __uint_as_float(((eh - 0x38000000u) << 3) | ((uint32_t)__double2loint(e) >> 29));
+  const double q = fma(0.5, e, widen(0.375f * ea * ea));
   ir = fma(y, q, y);
   return fma(s, q, s);
 }
@@ -195,21 +199,25 @@ __device__ __forceinline__ PairBox pair_box(const double (&box)[3]) {
 #pragma unroll
   for (int q = 0; q < 3; ++q) {
     b.L[q] = box[q];
-    b.half_hi[q] = __double2hiint(0.5 * box[q]);
+    b.half_hi[q] = __double2hiint(box[q]) - 0x100000;
   }
   return b;
 }
 __device__ __forceinline__ bool beyond(double d, int half_hi) { return (__double2hiint(d) & 0x7FFFFFFF) > half_hi; }
-// squared distance; dx, dy, dz become the minimum image
-__device__ __forceinline__ double pair_r2(const PairBox& b, double& dx, double& dy, double& dz) {
+__device__ __forceinline__ void pair_image(const PairBox& b, double& dx, double& dy, double& dz) {
   if (beyond(dx, b.half_hi[0]) | beyond(dy, b.half_hi[1]) | beyond(dz, b.half_hi[2])) {
     asm volatile("");  // keeps this a branch: predicated additions would take the pipe from every pair
     if (beyond(dx, b.half_hi[0])) dx = __double2hiint(dx) < 0 ? dx + b.L[0] : dx - b.L[0];
     if (beyond(dy, b.half_hi[1])) dy = __double2hiint(dy) < 0 ? dy + b.L[1] : dy - b.L[1];
     if (beyond(dz, b.half_hi[2])) dz = __double2hiint(dz) < 0 ? dz + b.L[2] : dz - b.L[2];
   }
+}
+// squared distance; dx, dy, dz become the minimum image
+__device__ __forceinline__ double pair_r2(const PairBox& b, double& dx, double& dy, double& dz) {
+  pair_image(b, dx, dy, dz);
   return fma(dz, dz, fma(dy, dy, dx * dx));
 }
+__device__ __forceinline__ bool not_finite(double v) { return (__double2hiint(v) & 0x7FF00000) == 0x7FF00000; }
 // r2 >= rc2 for a squared distance, by the bits; NaN is not outside (as with
 // the comparison), so that a lost atom's forces are NaN and the error is seen
 __device__ __forceinline__ bool outside(double r2, double rc2) {

@@ -300,6 +300,13 @@ struct MdArgs {
   double *fx, *fy, *fz;  // one allocation of 3 N
   Cubic* p4;             // (x, y, z, species in the low word) per atom (FP64 half-list passes)
   uint4* u4;             // (ux, uy, uz, species) per atom (mixed half-list passes)
+  // FP64 pair blocks (null: none): the density pass leaves the pairs of each
+  // group of atoms there (kernels_md.cu), from entry 32 pair_off[group]
+  float4* f4;               // (x, y, z, -) per atom
+  uint32_t* pair_off;
+  int* pair_rows;           // rows of 32 entries in use
+  uint32_t* pair_j;         // j, and the atom's place in its group in the top four bits
+  double2* pair_ui;         // r in table intervals, 1 / r
   double* rho;
   double* dFp;   // F'(rho_i)
   float* dFp32;  // the same in FP32 (mixed form)
@@ -326,6 +333,11 @@ void launch_fix_positions(long long N, const double* x, const double* y, const d
                           uint32_t* ux, uint32_t* uy, uint32_t* uz, cudaStream_t st);
 // densities (the half-list passes refresh their records, the mixed form its
 // fixed-point positions, first); launch_md_force follows on the same positions
+// atoms of a pair block, and how many blocks
+int md_pair_group(long long N);
+// places of the pair blocks for the present half list, in rows of 32 entries
+// of *total in all (zeroed before)
+void launch_md_pair_offsets(long long N, const int* cnt_h, uint32_t* pair_off, unsigned* total, cudaStream_t st);
 void launch_md_rho(const MdArgs& m, cudaStream_t st);
 void launch_md_force(const MdArgs& m, cudaStream_t st);
 void launch_md_first_half(const MdArgs& m, long long md_step, cudaStream_t st);

@@ -54,14 +54,14 @@ __global__ void k_md_rho(MdArgs m) {
 
 // interval and offset of r on a table grid when 0 <= r < r_c <= the grid's
 // end is already known (no range test)
-__device__ __forceinline__ int locate_in(const Spline& s, double r, double& t) {
-  const double u = r * s.inv_h;
+__device__ __forceinline__ int locate_u(const Spline& s, double u, double& t) {
   if (s.n_int < (1 << 19)) return locate_bits(u, s.n_int, t);
   int j = (int)u;
   j = j < s.n_int - 1 ? j : s.n_int - 1;
   t = u - (double)j;
   return j;
 }
+__device__ __forceinline__ int locate_in(const Spline& s, double r, double& t) { return locate_u(s, r * s.inv_h, t); }
 
 // Position and species of every atom in one 32-byte record (FP64 passes) or
 // one 16-byte one (mixed): a neighbour is one sector instead of four.
@@ -69,7 +69,11 @@ __global__ void k_md_records(MdArgs m) {
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= m.N) return;
   if (m.mixed) m.u4[i] = make_uint4(m.ux[i], m.uy[i], m.uz[i], (uint32_t)m.types[i]);
-  else m.p4[i] = Cubic{m.x[i], m.y[i], m.z[i], __hiloint2double(0, (int)m.types[i])};
+  else {
+    const Cubic p{m.x[i], m.y[i], m.z[i], __hiloint2double(0, (int)m.types[i])};
+    m.p4[i] = p;
+    if (m.pair_ui) m.f4[i] = make_float4((float)p.x, (float)p.y, (float)p.z, 0.0f);
+  }
 }
 __device__ __forceinline__ int record_type(const Cubic& p) { return __double2loint(p.w); }
 
@@ -85,10 +89,11 @@ __device__ __forceinline__ double lane_sum(double v) {
 // atom: they share its row, so a warp's rows differ less in length (8 atoms
 // instead of 32) and a row of 30 is a chain of 8 pairs instead of 30.
 //
-// FP64: bound by the FP64 pipe (86 % active), 17 instructions per pair for the
-// density and 27 for the force where the straightforward form took 31 and 46.
-// 1.36 M atoms, 39 M pairs within the cutoff and 12 M of skin: density 1.80 ms,
-// force 2.97 ms, a whole step 10.2 -> 5.8 ms; mixed 2.81 -> 2.06 ms.
+// FP64: bound by the FP64 pipe (86 % active), 16 instructions per pair for the
+// density and 26 for the force where the straightforward form took 31 and 46.
+// 1.36 M atoms, 39 M pairs within the cutoff: density 1.80 ms, force 2.97 ms, a
+// whole step 10.2 -> 5.8 ms; mixed 2.81 -> 2.06 ms.  They serve single forces
+// and what has no memory for pair blocks (below).
 // rho_i and rho_j both receive the pair's density (atomic adds into rho, zeroed
 // before); with one density function (SAME) one table value serves both ends.
 template <int LPA, bool SAME>
@@ -120,6 +125,215 @@ __global__ void __launch_bounds__(128) k_md_rho_half(MdArgs m) {
   }
   rho = lane_sum<LPA>(rho);
   if (live && sub == 0) atomicAdd(m.rho + i, rho);
+}
+
+__device__ __forceinline__ void add_virial(const MdArgs& m, double vir) {
+  if (!m.vir) return;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) vir += __shfl_xor_sync(0xffffffffu, vir, o);
+  if ((threadIdx.x & 31) == 0 && vir != 0.0) atomicAdd(m.vir, vir);
+}
+
+// The same passes with pair blocks (MD proper).  Rows differ in length (29 on
+// average, deviation 9 near a crystal's faces) and hold pairs beyond r_c, so
+// that a warp's FP64 lanes were 65 % full, and the force pass formed every r
+// and 1 / r again.  Here a warp takes the rows of GROUP atoms:
+//  1. it screens them in FP32, a row at a time (a margin keeps every pair within
+//     r_c; the FP32 pipe is 30 times as wide), into one list in shared memory;
+//  2. each lane takes an equal stretch of that list, so all lanes are busy but
+//     in the last row, sums an atom's density over its stretch and adds it when
+//     the stretch passes on to the next atom;
+//  3. r (in table intervals) and 1 / r stay in the pair block, stored lane by
+//     lane as the force pass reads them, which then needs 17 FP64 operations
+//     per pair instead of 26, for 40 bytes of memory traffic.
+// Both are bound by the FP64 pipe.  1.36 M atoms: density 1.80 -> 1.42 ms, force
+// 2.97 -> 1.41, a whole step 5.6 -> 3.6 ms.
+constexpr int PAIR_LIST = 544;  // longest list; taken when more than PAIR_LIST - 32 are in it
+constexpr double PAIR_NONE = -1.0;
+constexpr uint32_t PAIR_ATOM = (1u << 28) - 1u;
+
+template <int GROUP, bool SAME>
+__global__ void __launch_bounds__(128) k_md_rho_pairs(MdArgs m) {
+  __shared__ uint32_t s_list[4][PAIR_LIST];
+  __shared__ Cubic s_p[4][GROUP];
+  __shared__ float4 s_f[4][GROUP];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const long long grp = (long long)blockIdx.x * 4 + w, i0 = grp * GROUP;
+  if (i0 >= m.N) return;
+  const int na = m.N - i0 < GROUP ? (int)(m.N - i0) : GROUP;
+  int cnt = 0;
+  if (lane < na) {
+    cnt = m.cnt_h[i0 + lane];
+    s_p[w][lane] = m.p4[i0 + lane];
+    s_f[w][lane] = m.f4[i0 + lane];
+  }
+  __syncwarp();
+  const PairBox box = pair_box(m.box);
+  const double rc2 = m.rc * m.rc;
+  const float bx = (float)m.box[0], by = (float)m.box[1], bz = (float)m.box[2];
+  const float bm = bx > by ? (bx > bz ? bx : bz) : (by > bz ? by : bz);
+  const float rm = (float)m.rc + 0.01f + 1e-6f * bm, rm2 = rm * rm;
+  const unsigned below = (1u << lane) - 1u;
+  uint32_t* list = s_list[w];
+  const long long p0 = 32ll * m.pair_off[grp];
+  int rows = 0, T = 0;
+
+  const auto take = [&]() {
+    __syncwarp();
+    const int per = (T + 31) >> 5, e0 = lane * per;
+    int cur = -1;
+    double rho = 0.0;
+    Cubic pi{};
+    for (int it = 0; it < per; ++it) {
+      const int e = e0 + it;
+      const long long at = p0 + 32ll * (rows + it) + lane;
+      double2 keep = make_double2(PAIR_NONE, 0.0);
+      if (e < T) {
+        const uint32_t v = list[e];
+        const int a = (int)(v >> 28), j = (int)(v & PAIR_ATOM);
+        if (a != cur) {
+          if (cur >= 0) atomicAdd(m.rho + i0 + cur, rho);
+          cur = a;
+          rho = 0.0;
+          pi = s_p[w][a];
+        }
+        const Cubic pj = m.p4[j];
+        double dx = pj.x - pi.x, dy = pj.y - pi.y, dz = pj.z - pi.z;
+        const double r2 = pair_r2(box, dx, dy, dz);
+        m.pair_j[at] = v;
+        if (!outside(r2, rc2)) {
+          double ir, t;
+          const double u = sqrt3(r2, ir) * m.tab.sp[3].inv_h;
+          const int q = locate_u(m.tab.sp[3], u, t);
+          keep = make_double2(u, ir);
+          const double fj = spline_val_at(m.tab.sp[SAME ? 3 : 3 + record_type(pj)], q, t);  // density of j at i
+          const double fi = SAME ? fj : spline_val_at(m.tab.sp[3 + record_type(pi)], q, t);
+          rho += fj;
+          atomicAdd(m.rho + j, fi);
+        }
+      }
+      m.pair_ui[at] = keep;
+    }
+    if (cur >= 0) atomicAdd(m.rho + i0 + cur, rho);
+    rows += per;
+    T = 0;
+    __syncwarp();
+  };
+
+#pragma unroll 2
+  for (int a = 0; a < na; ++a) {
+    const int n = __shfl_sync(0xffffffffu, cnt, a);
+    const int* row = m.nbr_h + (i0 + a) * m.K;
+    const float4 fi = s_f[w][a];
+    for (int k0 = 0; k0 < n; k0 += 32) {
+      int j = 0;
+      bool near = false;
+      if (k0 + lane < n) {
+        j = row[k0 + lane];
+        const float4 f = m.f4[j];
+        float dx = fabsf(f.x - fi.x), dy = fabsf(f.y - fi.y), dz = fabsf(f.z - fi.z);
+        dx = dx > 0.5f * bx ? bx - dx : dx;
+        dy = dy > 0.5f * by ? by - dy : dy;
+        dz = dz > 0.5f * bz ? bz - dz : dz;
+        near = !(dx * dx + dy * dy + dz * dz >= rm2);  // NaN goes on to the FP64 test
+      }
+      const unsigned bal = __ballot_sync(0xffffffffu, near);
+      if (near) list[T + __popc(bal & below)] = (uint32_t)j | (uint32_t)a << 28;
+      T += __popc(bal);
+      if (T > PAIR_LIST - 32) take();
+    }
+  }
+  if (T > 0) take();
+  if (lane == 0) m.pair_rows[grp] = rows;
+}
+
+template <int GROUP, bool SAME, bool VIR>
+__global__ void __launch_bounds__(128) k_md_force_pairs(MdArgs m) {
+  __shared__ Cubic s_p[4][GROUP];
+  __shared__ double s_F[4][GROUP];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const long long grp = (long long)blockIdx.x * 4 + w, i0 = grp * GROUP;
+  if (i0 >= m.N) return;
+  if (lane < GROUP && i0 + lane < m.N) {
+    s_p[w][lane] = m.p4[i0 + lane];
+    s_F[w][lane] = m.dFp[i0 + lane];
+  }
+  __syncwarp();
+  const int rows = m.pair_rows[grp];
+  const long long p0 = 32ll * m.pair_off[grp] + lane;
+  const PairBox box = pair_box(m.box);
+  double fx = 0.0, fy = 0.0, fz = 0.0, vir = 0.0, Fi = 0.0;
+  Cubic pi{};
+  int cur = -1;
+  bool bad = false;
+  const auto flush = [&]() {
+    bad |= not_finite(fx) | not_finite(fy) | not_finite(fz);
+    atomicAdd(m.fx + i0 + cur, fx);
+    atomicAdd(m.fy + i0 + cur, fy);
+    atomicAdd(m.fz + i0 + cur, fz);
+  };
+  for (int it = 0; it < rows; ++it) {
+    const double2 ui = m.pair_ui[p0 + 32ll * it];
+    if (__double2hiint(ui.x) == __double2hiint(PAIR_NONE)) continue;
+    const uint32_t v = m.pair_j[p0 + 32ll * it];
+    const int a = (int)(v >> 28), j = (int)(v & PAIR_ATOM);
+    const Cubic pj = m.p4[j];
+    const double Fj = m.dFp[j];
+    if (a != cur) {
+      if (cur >= 0) flush();
+      cur = a;
+      fx = fy = fz = 0.0;
+      pi = s_p[w][a];
+      Fi = s_F[w][a];
+    }
+    double dx = pj.x - pi.x, dy = pj.y - pi.y, dz = pj.z - pi.z;
+    pair_image(box, dx, dy, dz);
+    double t;
+    const int q = locate_u(m.tab.sp[0], ui.x, t);
+    const int ti = record_type(pi), tj = record_type(pj);
+    double gg;
+    if (SAME) {
+      gg = fma(Fi + Fj, spline_dval_at(m.tab.dsp[3], q, t), spline_dval_at(m.tab.dsp[ti + tj], q, t));
+    } else {
+      gg = fma(Fj, spline_dval_at(m.tab.dsp[3 + ti], q, t),
+               fma(Fi, spline_dval_at(m.tab.dsp[3 + tj], q, t), spline_dval_at(m.tab.dsp[ti + tj], q, t)));
+    }
+    const double gr = -gg * ui.y;  // the force on j
+    const double gx = gr * dx, gy = gr * dy, gz = gr * dz;
+    fx -= gx;
+    fy -= gy;
+    fz -= gz;
+    if (VIR) vir = fma(gr, fma(dz, dz, fma(dy, dy, dx * dx)), vir);
+    atomicAdd(m.fx + j, gx);
+    atomicAdd(m.fy + j, gy);
+    atomicAdd(m.fz + j, gz);
+  }
+  if (cur >= 0) flush();
+  if (bad) atomicOr(m.err, ERRF_NONFINITE);
+  if (VIR) add_virial(m, vir);
+}
+
+// rows of 32 entries that a group's pairs can need: all of its half rows, and
+// what the lists of PAIR_LIST - 31 entries and more leave of their last row
+__global__ void k_md_pair_offsets(long long N, int group, const int* cnt_h, uint32_t* off, unsigned* total) {
+  const long long g = (long long)blockIdx.x * 128 + threadIdx.x;
+  const int lane = threadIdx.x & 31;
+  unsigned need = 0u;
+  if (g * group < N) {
+    int sum = 0;
+    for (int a = 0; a < group && g * group + a < N; ++a) sum += cnt_h[g * group + a];
+    need = (unsigned)(sum / 32 + sum / 448 + 2);
+  }
+  unsigned at = need;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned q = __shfl_up_sync(0xffffffffu, at, o);
+    if (lane >= o) at += q;
+  }
+  unsigned first = 0u;
+  if (lane == 31) first = atomicAdd(total, at);
+  first = __shfl_sync(0xffffffffu, first, 31);
+  if (g * group < N) off[g] = first + at - need;
 }
 
 // mixed form on the half list: FP32 geometry and tables, FP64 sums
@@ -197,7 +411,7 @@ __global__ void __launch_bounds__(128) k_md_force_half32(MdArgs m) {
     atomicAdd(m.fy + j, -gy);
     atomicAdd(m.fz + j, -gz);
   }
-  if (!isfinite(fx) || !isfinite(fy) || !isfinite(fz)) atomicOr(m.err, ERRF_NONFINITE);
+  if (not_finite(fx) | not_finite(fy) | not_finite(fz)) atomicOr(m.err, ERRF_NONFINITE);
   fx = lane_sum<LPA>(fx);
   fy = lane_sum<LPA>(fy);
   fz = lane_sum<LPA>(fz);
@@ -223,13 +437,6 @@ __global__ void k_md_embed(MdArgs m) {
 
 // warp sum of the per-thread virial terms, one atomic per warp (every lane
 // of the warp reaches this point)
-__device__ __forceinline__ void add_virial(const MdArgs& m, double vir) {
-  if (!m.vir) return;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) vir += __shfl_xor_sync(0xffffffffu, vir, o);
-  if ((threadIdx.x & 31) == 0 && vir != 0.0) atomicAdd(m.vir, vir);
-}
-
 // FP64 forces on the half list: F_i += g (x_j - x_i) / r, F_j -= the same,
 // g = phi'_{ti tj} + F'_i f'_{tj} + F'_j f'_{ti} (one density derivative
 // when same_dens); force arrays zeroed before.  The virial term of the
@@ -276,7 +483,7 @@ __global__ void __launch_bounds__(128) k_md_force_half(MdArgs m) {
     atomicAdd(m.fy + j, gy);
     atomicAdd(m.fz + j, gz);
   }
-  if (!isfinite(fx) || !isfinite(fy) || !isfinite(fz)) atomicOr(m.err, ERRF_NONFINITE);
+  if (not_finite(fx) | not_finite(fy) | not_finite(fz)) atomicOr(m.err, ERRF_NONFINITE);
   fx = lane_sum<LPA>(fx);
   fy = lane_sum<LPA>(fy);
   fz = lane_sum<LPA>(fz);
@@ -399,6 +606,13 @@ __device__ __forceinline__ void normals(uint4 w, double& z0, double& z1) {
   z1 = rr * s;
 }
 
+// the first of the two only
+__device__ __forceinline__ double normal(uint4 w) {
+  const double u1 = (double)top53(w.x, w.y) * 0x1p-53;
+  const double u2 = (double)top53(w.z, w.w) * 0x1p-53;
+  return sqrt(-2.0 * log(1.0 - u1)) * cospi(2.0 * u2);
+}
+
 __global__ void __launch_bounds__(128) k_md_first_half(MdArgs m, long long step) {
   const long long i = (long long)blockIdx.x * 128 + threadIdx.x;
   double d2 = 0.0;
@@ -414,9 +628,9 @@ __global__ void __launch_bounds__(128) k_md_first_half(MdArgs m, long long step)
       const double sig = m.sig[ti];  // c2 sqrt(kT / mass)
       const uint4 c0 = make_uint4((uint32_t)step, (uint32_t)((uint64_t)step >> 32), (uint32_t)i, TAG_NOISE0);
       const uint4 c1 = make_uint4((uint32_t)step, (uint32_t)((uint64_t)step >> 32), (uint32_t)i, TAG_NOISE1);
-      double z0, z1, z2, z3;
+      double z0, z1;
       normals(philox4x32_10(c0, m.key), z0, z1);
-      normals(philox4x32_10(c1, m.key), z2, z3);
+      const double z2 = normal(philox4x32_10(c1, m.key));
       vx = m.c1 * vx + sig * z0;
       vy = m.c1 * vy + sig * z1;
       vz = m.c1 * vz + sig * z2;
@@ -586,6 +800,33 @@ void launch_fix_positions(long long N, const double* x, const double* y, const d
 // per atom and 97 with 16 lanes.
 constexpr long long MD_FEW = 20000;
 
+// atoms of a pair block.  16 fill 14.5 rows of 32 lanes with their 464 pairs;
+// fewer leave more lanes idle in the last row but give the GPU more warps.  A
+// step with 2 / 4 / 16: 5488 atoms 90 / 101 / 178 us, 86 k (nanocrystal) 321 /
+// 327 / 380, 351 k 1110 / 1073 / 1086, 1.36 M 3932 / 3791 / 3645.
+int md_pair_group(long long N) { return N < 100000 ? 2 : N < 500000 ? 4 : 16; }
+
+void launch_md_pair_offsets(long long N, const int* cnt_h, uint32_t* pair_off, unsigned* total, cudaStream_t st) {
+  const int group = md_pair_group(N);
+  k_md_pair_offsets<<<grid_of((N + group - 1) / group), 128, 0, st>>>(N, group, cnt_h, pair_off, total);
+}
+
+template <int GROUP>
+static void rho_pairs(const MdArgs& m, cudaStream_t st) {
+  const unsigned g = grid_of((m.N + GROUP - 1) / GROUP * 32);
+  if (m.same_dens) k_md_rho_pairs<GROUP, true><<<g, 128, 0, st>>>(m);
+  else k_md_rho_pairs<GROUP, false><<<g, 128, 0, st>>>(m);
+}
+
+template <int GROUP>
+static void force_pairs(const MdArgs& m, cudaStream_t st) {
+  const unsigned g = grid_of((m.N + GROUP - 1) / GROUP * 32);
+  if (m.vir && m.same_dens) k_md_force_pairs<GROUP, true, true><<<g, 128, 0, st>>>(m);
+  else if (m.vir) k_md_force_pairs<GROUP, false, true><<<g, 128, 0, st>>>(m);
+  else if (m.same_dens) k_md_force_pairs<GROUP, true, false><<<g, 128, 0, st>>>(m);
+  else k_md_force_pairs<GROUP, false, false><<<g, 128, 0, st>>>(m);
+}
+
 template <int LPA>
 static void rho_half(const MdArgs& m, cudaStream_t st) {
   const unsigned g = grid_of(m.N * LPA);
@@ -609,7 +850,10 @@ void launch_md_rho(const MdArgs& m, cudaStream_t st) {
   if (m.nbr_h) {
     k_md_records<<<grid_of(m.N), 128, 0, st>>>(m);
     cudaMemsetAsync(m.rho, 0, sizeof(double) * m.N, st);
-    if (m.N < MD_FEW) rho_half<16>(m, st);
+    if (m.pair_ui && md_pair_group(m.N) == 2) rho_pairs<2>(m, st);
+    else if (m.pair_ui && md_pair_group(m.N) == 4) rho_pairs<4>(m, st);
+    else if (m.pair_ui) rho_pairs<16>(m, st);
+    else if (m.N < MD_FEW) rho_half<16>(m, st);
     else rho_half<4>(m, st);
     k_md_embed<<<grid_of(m.N), 128, 0, st>>>(m);
   } else if (m.mixed) {
@@ -621,7 +865,10 @@ void launch_md_rho(const MdArgs& m, cudaStream_t st) {
 void launch_md_force(const MdArgs& m, cudaStream_t st) {
   if (m.nbr_h) {
     cudaMemsetAsync(m.fx, 0, sizeof(double) * 3 * m.N, st);
-    if (m.N < MD_FEW) force_half<16>(m, st);
+    if (m.pair_ui && md_pair_group(m.N) == 2) force_pairs<2>(m, st);
+    else if (m.pair_ui && md_pair_group(m.N) == 4) force_pairs<4>(m, st);
+    else if (m.pair_ui) force_pairs<16>(m, st);
+    else if (m.N < MD_FEW) force_half<16>(m, st);
     else force_half<4>(m, st);
   } else if (m.mixed) {
     k_md_force<true><<<grid_of(m.N), 128, 0, st>>>(m);

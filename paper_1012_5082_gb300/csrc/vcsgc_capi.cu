@@ -56,6 +56,16 @@ struct Ctx {
   uint32_t *ux = nullptr, *uy = nullptr, *uz = nullptr;  // fixed-point positions (mixed, kind 1)
   Cubic* p4 = nullptr;             // records of the half-list passes (FP64, mixed)
   uint4* u4 = nullptr;
+  // pair blocks of the FP64 MD passes, held once MD has run (md_pairs; see
+  // ensure_pairs): 20 bytes per pair within the list radius
+  bool md_pairs = false;
+  float4* f4 = nullptr;
+  uint32_t* pair_off = nullptr;
+  int* pair_rows = nullptr;
+  uint32_t* pair_j = nullptr;
+  double2* pair_ui = nullptr;
+  unsigned* pair_total = nullptr;
+  size_t pair_cap = 0, pair_need = 0;  // entries held, entries of the present list
   unsigned long long* max_disp2 = nullptr;
   int* nbr = nullptr;
   int* nbr_cnt = nullptr;
@@ -337,6 +347,12 @@ void fill_args(Ctx* c) {
   m.fx = c->fx; m.fy = c->fy; m.fz = c->fz;
   m.p4 = c->p4;
   m.u4 = c->u4;
+  const bool pairs = c->md_pairs && c->pair_cap && c->pair_need <= c->pair_cap;
+  m.f4 = c->f4;
+  m.pair_off = c->pair_off;
+  m.pair_rows = c->pair_rows;
+  m.pair_j = c->pair_j;
+  m.pair_ui = pairs ? c->pair_ui : nullptr;
   m.rho = c->rho;
   m.dFp = c->dFp;
   m.dF = c->dF;
@@ -404,6 +420,49 @@ void drop_graph(Ctx* c) {
 }
 
 // ----------------------------------------------------------- neighbours
+// Pair blocks for the present half list, an eighth more than it needs.  They
+// take 20 bytes per pair (0.75 kB per atom at 37 pairs), so only what lies within
+// a quarter of the free memory; without them the passes form r twice.
+int ensure_pairs(Ctx* c) {
+  if (!c->md_pairs) return VCSGC_OK;
+  CK(cudaMemsetAsync(c->pair_total, 0, sizeof(unsigned), c->st));
+  launch_md_pair_offsets(c->N, c->cnt_h, c->pair_off, c->pair_total, c->st);
+  CK(cudaGetLastError());
+  unsigned rows = 0;
+  CK(cudaMemcpyAsync(&rows, c->pair_total, sizeof(rows), cudaMemcpyDeviceToHost, c->st));
+  CK(cudaStreamSynchronize(c->st));
+  c->pair_need = 32 * (size_t)rows;
+  if (c->pair_need > c->pair_cap) {
+    dfree(c, &c->pair_j);
+    dfree(c, &c->pair_ui);
+    c->pair_cap = 0;
+    const size_t want = c->pair_need + c->pair_need / 8;
+    size_t free_b = 0, total_b = 0;
+    CK(cudaMemGetInfo(&free_b, &total_b));
+    if (want * (sizeof(uint32_t) + sizeof(double2)) <= free_b / 4 && dalloc(c, &c->pair_j, want) == VCSGC_OK) {
+      if (dalloc(c, &c->pair_ui, want) == VCSGC_OK) c->pair_cap = want;
+      else dfree(c, &c->pair_j);
+    }
+  }
+  fill_args(c);
+  return VCSGC_OK;
+}
+
+// pair blocks from now on (MD and minimisation, whose list serves many passes)
+int enable_pairs(Ctx* c) {
+  if (c->md_pairs || !c->p4 || !c->nbr_h || c->N > (1ll << 28)) return VCSGC_OK;
+  size_t free_b = 0, total_b = 0;
+  CK(cudaMemGetInfo(&free_b, &total_b));
+  if ((size_t)c->N * (sizeof(float4) + 2 * sizeof(int)) > free_b / 4) return VCSGC_OK;
+  const long long groups = (c->N + md_pair_group(c->N) - 1) / md_pair_group(c->N);
+  TRY(dalloc(c, &c->f4, c->N));
+  TRY(dalloc(c, &c->pair_off, groups));
+  TRY(dalloc(c, &c->pair_rows, groups));
+  TRY(dalloc(c, &c->pair_total, 1));
+  c->md_pairs = true;
+  return ensure_pairs(c);
+}
+
 int build_cell_list(Ctx* c) {
   for (int q = 0; q < 3; ++q) {
     c->cl.nc[q] = (int)std::floor(c->box[q] / c->rl);
@@ -440,7 +499,7 @@ int build_cell_list(Ctx* c) {
     unsigned e = 0;
     CK(cudaMemcpyAsync(&e, c->derr, sizeof(unsigned), cudaMemcpyDeviceToHost, c->st));
     CK(cudaStreamSynchronize(c->st));
-    if (!(e & ERRF_OVERFLOW)) return VCSGC_OK;
+    if (!(e & ERRF_OVERFLOW)) return ensure_pairs(c);
     // grow the rows and rebuild
     const int K2 = ((c->K * 3 / 2) + 7) / 8 * 8;
     int* nb = nullptr;
@@ -1233,6 +1292,7 @@ int md_run_nh(Ctx* c, long long n) {
 int md_run(Ctx* c, long long n) {
   if (!c->have_v) return fail(c, VCSGC_ERR_STATE, "md_steps needs velocities (vcsgc_set_velocities)");
   if (c->kind != 1 || c->R != 1) return fail(c, VCSGC_ERR_STATE, "md_steps needs explicit positions and one replica");
+  if (n > 0) TRY(enable_pairs(c));
   if (c->nh.kind) return md_run_nh(c, n);
   if (!c->forces_valid) TRY(md_forces(c));
   const double half_skin2 = 0.25 * c->skin * c->skin;
@@ -2924,6 +2984,7 @@ int vcsgc_minimize(void* ctx, double ftol, int64_t max_iter, int64_t* iters, dou
   if (!c || !(ftol > 0.0) || max_iter < 0) return VCSGC_ERR_INVALID_ARG;
   if (c->kind != 1 || c->R != 1) return fail(c, VCSGC_ERR_STATE, "needs explicit positions and one replica");
   const long long N = c->N, n3 = 3 * N;
+  TRY(enable_pairs(c));
   if (!c->cg_x0) {
     TRY(dalloc(c, &c->cg_x0, n3));
     TRY(dalloc(c, &c->cg_d, n3));

@@ -60,3 +60,42 @@ def test_forces_mixed(V, cells, dens_b):
     for a in range(3):
         assert np.max(np.abs(Fg[a] - Fo[a])) < 2e-5
     g.close()
+
+
+@pytest.mark.parametrize("dens_b", [1.0, 1.25])
+@pytest.mark.parametrize("cells", [(6, 6, 6), (7, 6, 9), (36, 37, 38), (63, 64, 63)])
+def test_pair_blocks_match_the_direct_passes(V, cells, dens_b):
+    """MD passes leave each pair's distance for the force pass, in blocks of 2,
+    4 or 16 atoms by size; the passes of a context that has not run MD do not.
+    Same bounds as against the oracle."""
+    orc, g, lat = _pair(V, cells, dens_b, V.PREC_FP64)
+    want = [np.array(F) for F in g.forces()]
+    p0 = g.ensemble_state()["pressure_bar"]
+    g.minimize(ftol=1e-3, max_iter=0)
+    got = g.forces()
+    for a in range(3):
+        assert np.max(np.abs(got[a] - want[a])) < 1e-10
+    sg = g.ensemble_state()
+    assert abs(sg["pressure_bar"] - p0) <= 1e-10 * abs(p0)
+    got = g.forces()
+    for a in range(3):
+        assert np.max(np.abs(got[a] - want[a])) < 1e-10
+    g.close()
+
+
+def test_long_rows_take_several_lists(V):
+    """A cutoff of 9 A: 132 pairs per half row, four atoms of a block overflow
+    its list."""
+    tab = I.eam_tables(I.EAMParams(rc=9.0, r_in=8.5))
+    rng = np.random.default_rng(2)
+    lat = I.bcc_lattice(37, 37, 38)
+    q = [(x + rng.uniform(-0.05, 0.05, lat.n)) % b for x, b in zip((lat.x, lat.y, lat.z), lat.box)]
+    lat = I.Lattice(x=q[0], y=q[1], z=q[2], box=lat.box.copy())
+    t = I.random_types(lat.n, lat.n // 4, seed=1)
+    orc = O.System(lat, t, tab)
+    g = V.Context(lat, t, tab, -2.0, 10.0, 700.0, schedule=V.SCHED_SPATIAL, sched=(2, 2, 2, 2, 2, 2))
+    g.minimize(ftol=1e-3, max_iter=0)
+    Fg, Fo = g.forces(), orc.forces()
+    for a in range(3):
+        assert np.max(np.abs(Fg[a] - Fo[a])) < 1e-10
+    g.close()
