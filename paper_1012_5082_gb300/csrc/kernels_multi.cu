@@ -65,6 +65,28 @@ void launch_multi_fixed(const double* V, int n_sh, int K, int qbits, long long* 
 }
 
 // rho_i = sum_j f_{t_j}(r_ij)
+// A packed argument X = x << 2 | t: x = rho / h in fixed point (fx_bits fraction
+// bits) of species t's FP32 cubics, in range.  The argument of a density and a
+// shell's difference is within 2 2^-fx_bits intervals (two roundings, and the
+// species bits left below the fraction), which the host checks against the
+// share of the screen's bound that a float argument takes.
+__device__ __forceinline__ float fix_val(const MultiArgs& a, uint32_t X) {
+  const float4 c = __ldg(a.emb32 + ((X & 3u) * (uint32_t)a.emb_n + (X >> (a.fx_bits + 2))));
+  const float u = __uint_as_float(__funnelshift_r(X << (30 - a.fx_bits), 0x7Fu, 9)) - 1.0f;
+  return fmaf(u, fmaf(u, fmaf(u, c.w, c.z), c.y), c.x);
+}
+__device__ __forceinline__ uint32_t fix_clamp(const MultiArgs& a, uint32_t X) {
+  return X < a.fx_lo ? a.fx_lo : (X > a.fx_hi ? a.fx_hi : X);
+}
+// a site's entry; an argument out of range is stored as 0, which no shell's
+// difference brings into range
+__device__ __forceinline__ uint2 fix_entry(const MultiArgs& a, int t, double rho) {
+  const double v = rho * a.fx_scale;
+  const uint32_t X = v > 0.0 && v < 1073741823.0 ? __double2uint_rn(v) << 2 | (uint32_t)t : 0u;
+  const bool in = fix_clamp(a, X) == X;
+  return make_uint2(in ? X : (uint32_t)t, in ? __float_as_uint(fix_val(a, X)) : 0u);
+}
+
 __global__ void k_multi_rho(MultiArgs a, int r0) {
   const int r = r0 + blockIdx.y;
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -76,6 +98,11 @@ __global__ void k_multi_rho(MultiArgs a, int r0) {
     rho += a.Fd[h.w * a.K + ty[multi_nbr(a, (int)i, h)]];
   }
   a.rho[(long long)r * a.N + i] = rho;
+  if (a.rfu) {
+    const int3 h = multi_half(a, (int)i);
+    const int b = (int)(i & 1);
+    a.rfu[(long long)r * a.rf_n + multi_rfi(a, (h.x - b) >> 1, (h.y - b) >> 1, (h.z - b) >> 1, b)] = fix_entry(a, ty[i], rho);
+  }
   if (a.rf) {
     const float r32 = (float)rho;
     const int3 h = multi_half(a, (int)i);
@@ -301,6 +328,18 @@ __host__ __device__ constexpr int mk_bcc5_desc(int k) {
          ((((B + (((mk_bcc5_code(k) >> 8) & 15) - 4) - (B ^ (((mk_bcc5_code(k) & 15) - 4) & 1))) >> 1) + 2) << 6) |
          ((B ^ (((mk_bcc5_code(k) & 15) - 4) & 1)) << 9) | ((mk_bcc5_code(k) >> 12) << 10);
 }
+// the same for a neighbour known at run time (computed from the switch it is a
+// chain of branches in every block's prologue)
+struct Bcc5Desc {
+  int v[2][MK_BCC5_N];
+  constexpr Bcc5Desc() : v() {
+    for (int k = 0; k < MK_BCC5_N; ++k) {
+      v[0][k] = mk_bcc5_desc<0>(k);
+      v[1][k] = mk_bcc5_desc<1>(k);
+    }
+  }
+};
+__device__ const Bcc5Desc c_bcc5_desc{};
 
 // first neighbour of shell s in the five-shell order (8, 6, 12, 24, 8 sites)
 __host__ __device__ constexpr int mk_shell0(int s) {
@@ -759,6 +798,8 @@ __device__ __forceinline__ void multi_descriptor(const MultiArgs& a, int r, int 
   nb[4] = (int)(xs >> 24);
 }
 
+__device__ __noinline__ void multi_fold(const MultiArgs& a, int r, long long step);
+
 // MODE 0: no re-embedding; 1: re-embedding, FP64 dE (any neighbour table);
 // 2: re-embedding, five-shell table, FP32 screen (the dE sum of an accepted
 // step is then taken by the commit launch, in FP64); 3: mode 2 with delayed
@@ -842,7 +883,7 @@ __global__ void __launch_bounds__(MK_BLOCK, 4) k_multi_propose(MultiArgs a, int 
   if constexpr (SCREEN) {
     if (threadIdx.x < MK_BCC5_N) {
       const int k = threadIdx.x;
-      scode[k] = (c & 1) ? mk_bcc5_desc<1>(k) : mk_bcc5_desc<0>(k);
+      scode[k] = c_bcc5_desc.v[c & 1][k];
     }
     __syncthreads();
   }
@@ -879,7 +920,13 @@ __global__ void __launch_bounds__(MK_BLOCK, 4) k_multi_propose(MultiArgs a, int 
   // screened form: launched after the previous step's commit with
   // programmatic dependent launch; the species, densities and this step's
   // accumulators are read after the wait (a no-op for an ordinary launch)
-  if constexpr (SCREEN) pdl_wait();
+  if constexpr (SCREEN) {
+    pdl_wait();
+    if (blockIdx.x == gridDim.x - 1) {  // the block past the trials
+      if (threadIdx.x == 0) multi_fold(a, r, step - 1);
+      return;
+    }
+  }
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   int s1 = 0;
   if constexpr (MODE == 3) {
@@ -1016,7 +1063,8 @@ __global__ void __launch_bounds__(MK_BLOCK, 4) k_multi_propose(MultiArgs a, int 
     int base = 0;
     if (lane == 0) base = atomicAdd(&A->nacc, __popc(m));
     base = __shfl_sync(0xffffffffu, base, 0);
-    if (acc) a.pend[(long long)r * a.D + base + __popc(m & ((1u << lane) - 1u))] = make_int2(site, tb | (ta << 8));
+    if (acc)
+      a.pend[(long long)r * a.D + base + __popc(m & ((1u << lane) - 1u))] = make_int2(SCREEN ? d : site, tb | (ta << 8));
   }
   // per-solute dn, ties and the dE sum: warp, then block, then one atomic each
 #pragma unroll
@@ -1185,6 +1233,59 @@ __device__ __forceinline__ int multi_global(const MultiArgs& a, const MRepParams
   return metropolis(Y, ug, tie) ? 1 : 0;
 }
 
+__device__ __forceinline__ int step_colour(const MultiArgs& a, const MRepParams& p, long long step) {
+  const uint4 w = philox4x32_10(make_uint4((uint32_t)step, (uint32_t)((uint64_t)step >> 32), 0xFFFFFFFFu, TAG_STEP), p.key);
+  return (int)below64(w.x, w.y, (uint64_t)a.n_colours);
+}
+
+// Screened form: step `step` folded into replica r's state, from its sums and its
+// decision (the commit's, taken again), if it is the state's next one.  Run by
+// one thread of the next step's propose launch, in a block of its own, and by
+// the advance launch for the last step of a chain: in the commit launch this
+// chain of loads and FP64 sums held up every step.
+__device__ __noinline__ void multi_fold(const MultiArgs& a, int r, long long step) {
+  MRepState s = a.rs[r];
+  if (s.step != step) return;
+  const MStepAcc* A = a.acc + 2 * r + (int)(step & 1);
+  const int nacc = __ldcg(&A->nacc);
+  int dn[MK_MAX], gtie = 0;
+  long long c0[MK_MAX];
+#pragma unroll
+  for (int al = 0; al < MK_MAX; ++al) {
+    dn[al] = al > 0 && al < a.K ? __ldcg(&A->dn[al]) : 0;
+    c0[al] = al < a.K ? __ldcg(&A->cnt[al]) : 0;
+  }
+  s.trials += a.D;
+  s.local_acc += nacc;
+  s.s1_acc += __ldcg(&A->s1);
+  if (nacc > 0) {
+    s.global_trials++;
+    if (multi_global(a, a.rp[r], dn, c0, step_uniform(a.rp[r], step), &gtie)) {
+      s.global_acc++;
+      s.flips += nacc;
+      long long d0 = 0;
+#pragma unroll
+      for (int al = 1; al < MK_MAX; ++al)
+        if (al < a.K) {
+          s.cnt[al] += dn[al];
+          d0 += dn[al];
+        }
+      s.cnt[0] -= d0;
+    }
+  }
+  s.near_ties += __ldcg(&A->ties) + gtie;
+  s.steps++;
+#pragma unroll
+  for (int al = 0; al < MK_MAX; ++al)
+    if (al < a.K) {
+      const double cc = (double)s.cnt[al] * a.inv_n;
+      s.sum_c[al] += cc;
+      s.sum_c2[al] += cc * cc;
+    }
+  s.step = step + 1;
+  a.rs[r] = s;
+}
+
 // Screened form: one thread per (accept, neighbour) and one per accepted
 // site over all replicas that accepted their step, on a fixed grid: the
 // density change in FP64 with its float copy and the FP32 embedding value
@@ -1193,7 +1294,12 @@ __device__ __forceinline__ int multi_global(const MultiArgs& a, const MRepParams
 // neighbour's species changes.  Every block sums the replicas' item counts
 // (at most MK_SCREEN_MAX_R replicas; the host selects this form only while
 // R D (MK_BCC5_N + 1) < 2^31, so the int item index cannot overflow).
-__global__ void __launch_bounds__(MK_BLOCK) k_multi_commit_screen(MultiArgs a, int jl) {
+// One block of 512 threads per SM: four of 128 made four times the requests for
+// the sums of the step, all to the same few L2 lines, and the last block of a
+// step without accepted replicas ended 3 us after the first (80^3 x 8, steps of
+// two species 14.0 -> 13.0 us, with delayed acceptance 21.3 -> 20.0).
+constexpr int MK_CBLOCK = 512;
+__global__ void __launch_bounds__(MK_CBLOCK) k_multi_commit_screen(MultiArgs a, int jl) {
   // the next step's propose may start its draws now; it reads what this
   // launch writes only after griddepcontrol.wait
   pdl_trigger();
@@ -1205,13 +1311,22 @@ __global__ void __launch_bounds__(MK_BLOCK) k_multi_commit_screen(MultiArgs a, i
   // own species
   constexpr int NI = MK_BCC5_N + 1;
   const long long step = *a.base + jl;  // the step the propose launch proposed
-  for (int q = threadIdx.x; q < MK_BCC5_N; q += MK_BLOCK) s_off[q] = a.off[q];
-  for (int q = threadIdx.x; q < 5 * K * K; q += MK_BLOCK) {
+  for (int q = threadIdx.x; q < MK_BCC5_N; q += MK_CBLOCK) s_off[q] = a.off[q];
+  for (int q = threadIdx.x; q < 5 * K * K; q += MK_CBLOCK) {
     const int sh = q / (K * K), x = (q / K) % K, y = q % K;
     s_df[q] = a.Fd[sh * K + y] - a.Fd[sh * K + x];
   }
-  __shared__ uint64_t s_ug[MK_BLOCK];
+  __shared__ uint64_t s_ug[MK_CBLOCK];
   if (threadIdx.x < a.R) s_ug[threadIdx.x] = step_uniform(a.rp[threadIdx.x], step);
+  // each replica's colour of the step: px, py, pz (21 bits each), basis; an
+  // accept is stored by its trial index, so its items need no division
+  __shared__ unsigned long long s_col[MK_SCREEN_MAX_R];
+  for (int r = threadIdx.x; r < a.R; r += MK_CBLOCK) {
+    const int c = a.ctab ? __ldg(a.ctab + r * MK_CTAB + jl) : step_colour(a, a.rp[r], step);
+    const int pc = c >> 1, pq = pc / a.qx, pz = pq / a.qy;
+    s_col[r] = (unsigned long long)(pc - pq * a.qx) | (unsigned long long)(pq - pz * a.qy) << 21 |
+               (unsigned long long)pz << 42 | (unsigned long long)(c & 1) << 63;
+  }
   __shared__ long long s_fix[10];  // +-(f_1 - f_0)(r_s) / h in fixed point
   if (a.dtab && threadIdx.x < 10) {
     const int s = threadIdx.x % 5;
@@ -1223,62 +1338,35 @@ __global__ void __launch_bounds__(MK_BLOCK) k_multi_commit_screen(MultiArgs a, i
   pdl_wait();
   // the global stage of every replica (Eq. trans_vcsgc_par2 per solute),
   // taken in every block from the step's complete sums: the same FP64
-  // arithmetic everywhere, so the same decision.  Block 0 folds the step
-  // into the replica's state and readies the next step's accumulator.
-  for (int r = threadIdx.x; r < a.R; r += MK_BLOCK) {
+  // arithmetic everywhere, so the same decision.  Block 0 readies the next
+  // step's accumulator.
+  for (int r = threadIdx.x; r < a.R; r += MK_CBLOCK) {
     const MStepAcc* A = a.acc + 2 * r + (int)(step & 1);
     const MRepParams& p = a.rp[r];
+    // four wide loads: every block reads the same few lines
+    const int4 vd = __ldcg(reinterpret_cast<const int4*>(A->dn));
     const int nacc = __ldcg(&A->nacc);
-    int dn[MK_MAX];
-    long long c0[MK_MAX];
-#pragma unroll
-    for (int al = 0; al < MK_MAX; ++al) {
-      dn[al] = al > 0 && al < K ? __ldcg(&A->dn[al]) : 0;
-      c0[al] = al < K ? __ldcg(&A->cnt[al]) : 0;
-    }
+    const longlong2 v0 = __ldcg(reinterpret_cast<const longlong2*>(A->cnt));
+    const longlong2 v1 = __ldcg(reinterpret_cast<const longlong2*>(A->cnt + 2));
+    const int dn[MK_MAX] = {0, K > 1 ? vd.y : 0, K > 2 ? vd.z : 0, K > 3 ? vd.w : 0};
+    const long long c0[MK_MAX] = {v0.x, v0.y, K > 2 ? v1.x : 0, K > 3 ? v1.y : 0};
     int accept = 0, gtie = 0;
     if (nacc > 0) {
-      const uint64_t ug = s_ug[r < MK_BLOCK ? r : 0];
-      accept = multi_global(a, p, dn, c0, r < MK_BLOCK ? ug : step_uniform(p, step), &gtie);
+      const uint64_t ug = s_ug[r < MK_CBLOCK ? r : 0];
+      accept = multi_global(a, p, dn, c0, r < MK_CBLOCK ? ug : step_uniform(p, step), &gtie);
     }
     s_pre[r + 1] = accept ? nacc * NI : 0;
     if (blockIdx.x == 0) {
-      MRepState s = a.rs[r];
-      s.trials += a.D;
-      s.local_acc += nacc;
-      s.near_ties += __ldcg(&A->ties) + gtie;
-      s.s1_acc += __ldcg(&A->s1);
-      if (nacc > 0) {
-        s.global_trials++;
-        if (accept) {
-          s.global_acc++;
-          s.flips += nacc;
-          long long d0 = 0;
-#pragma unroll
-          for (int al = 1; al < MK_MAX; ++al)
-            if (al < K) {
-              s.cnt[al] += dn[al];
-              d0 += dn[al];
-            }
-          s.cnt[0] -= d0;
-        }
-      }
-      s.steps++;
-#pragma unroll
-      for (int al = 0; al < MK_MAX; ++al)
-        if (al < K) {
-          const double cc = (double)s.cnt[al] * a.inv_n;
-          s.sum_c[al] += cc;
-          s.sum_c2[al] += cc * cc;
-        }
-      s.step = step + 1;
-      a.rs[r] = s;
       MStepAcc* B = a.acc + 2 * r + (int)((step + 1) & 1);
+      long long d0 = 0;
 #pragma unroll
-      for (int al = 0; al < MK_MAX; ++al) {
+      for (int al = 1; al < MK_MAX; ++al) {
         B->dn[al] = 0;
-        B->cnt[al] = s.cnt[al];
+        B->cnt[al] = c0[al] + (accept ? dn[al] : 0);
+        d0 += accept ? dn[al] : 0;
       }
+      B->dn[0] = 0;
+      B->cnt[0] = c0[0] - d0;
       B->nacc = 0;
       B->ties = 0;
       B->done = 0u;
@@ -1295,7 +1383,7 @@ __global__ void __launch_bounds__(MK_BLOCK) k_multi_commit_screen(MultiArgs a, i
   __syncthreads();
   const int total = s_pre[a.R];
   int r = 0;
-  for (int it = blockIdx.x * MK_BLOCK + threadIdx.x; it < total; it += gridDim.x * MK_BLOCK) {
+  for (int it = blockIdx.x * MK_CBLOCK + threadIdx.x; it < total; it += gridDim.x * MK_CBLOCK) {
     while (s_pre[r + 1] <= it) ++r;
     const int loc = it - s_pre[r];
     const int n = loc / NI, k = loc - n * NI;
@@ -1303,25 +1391,45 @@ __global__ void __launch_bounds__(MK_BLOCK) k_multi_commit_screen(MultiArgs a, i
     const int tb = e.y & 255, ta = e.y >> 8;
     uint8_t* ty = a.types + (long long)r * a.N;
     double* rho = a.rho + (long long)r * a.N;
-    const int3 ph = multi_half(a, e.x);
-    // the item's site: its entry, the species and density it has from now on
-    int X = ph.x >> 1, Y = ph.y >> 1, Z = ph.z >> 1, bb = e.x & 1, t = tb;
-    double nr;
-    long long q;
+    const unsigned long long col = s_col[r];
+    const int b = (int)(col >> 63);
+    int m[3] = {(int)(col & 0x1FFFFFu), (int)(col >> 21 & 0x1FFFFFu), (int)(col >> 42 & 0x1FFFFFu)}, kk[3];
+    const int dq = mk_div(e.x, a.nxq, a.rcp_nxq);
+    kk[0] = e.x - dq * a.nxq;
+    kk[2] = mk_div(dq, a.nyq, a.rcp_nyq);
+    kk[1] = dq - kk[2] * a.nyq;
+    // the item's site: its class and place, the species and density it has from
+    // now on
+    int bb = b, t = tb, w = 0;
     if (k < MK_BCC5_N) {
       const int4 h = s_off[k];
-      multi_nbr_cell(a, ph, h, X, Y, Z, bb);
-      const int jn = ((Z * a.ny + Y) * a.nx + X) * 2 + bb;
-      nr = rho[jn] + s_df[(h.w * K + ta) * K + tb];
+      w = h.w;
+      bb = (b + h.x) & 1;
+      const int hh[3] = {h.x, h.y, h.z}, qq[3] = {a.qx, a.qy, a.qz}, nk[3] = {a.nxq, a.nyq, a.nzq};
+#pragma unroll
+      for (int x = 0; x < 3; ++x) {
+        m[x] += (b + hh[x] - bb) >> 1;
+        if (m[x] < 0) {
+          m[x] += qq[x];
+          kk[x] = (kk[x] ? kk[x] : nk[x]) - 1;
+        } else if (m[x] >= qq[x]) {
+          m[x] -= qq[x];
+          kk[x] = kk[x] + 1 < nk[x] ? kk[x] + 1 : 0;
+        }
+      }
+    }
+    const int jn = (((m[2] + a.qz * kk[2]) * a.ny + m[1] + a.qy * kk[1]) * a.nx + m[0] + a.qx * kk[0]) * 2 + bb;
+    const int q = ((m[2] * a.qy + m[1]) * a.qx + m[0]) * a.D + (kk[2] * a.nyq + kk[1]) * a.nxq + kk[0] +
+                  (bb ? rfi_plane(a) : 0);
+    double nr = rho[jn];
+    if (k < MK_BCC5_N) {
+      nr += s_df[(w * K + ta) * K + tb];
       rho[jn] = nr;
       t = ty[jn];
-      q = multi_rfi(a, X, Y, Z, bb);
-      // the flipped site is in shell h.w of this one (da, dtab: K = 2)
-      if (a.dtab || a.da) a.nbc[(long long)r * a.rf_n + q] += (uint32_t)(tb - ta) << (6 * h.w);
+      // the flipped site is in shell w of this one (da, dtab: K = 2)
+      if (a.dtab || a.da) a.nbc[(long long)r * a.rf_n + q] += (uint32_t)(tb - ta) << (6 * w);
     } else {
-      nr = rho[e.x];
-      ty[e.x] = (uint8_t)tb;
-      q = multi_rfi(a, X, Y, Z, bb);
+      ty[jn] = (uint8_t)tb;
     }
     if (a.dtab) {
       float* D = a.dtab + (long long)r * DTAB_PLANES * a.rf_n + q;
@@ -1330,6 +1438,8 @@ __global__ void __launch_bounds__(MK_BLOCK) k_multi_commit_screen(MultiArgs a, i
       D[10 * a.rf_n] = dtab_value(a, 1 - t, u, u, p0);
 #pragma unroll
       for (int s = 0; s < 10; ++s) D[s * a.rf_n] = dtab_value(a, t, u + s_fix[s], u, p0);
+    } else if (a.rfu) {
+      a.rfu[(long long)r * a.rf_n + q] = fix_entry(a, t, nr);
     } else {
       const float r32 = (float)nr;
       a.rf[(long long)r * a.rf_n + q] = make_float2(r32, emb32_val(a, t, r32));
@@ -1360,7 +1470,7 @@ __global__ void __launch_bounds__(MK_BLOCK, 4) k_multi_propose_table(MultiArgs a
   cp[0] = pc - pq * a.qx;
   cp[2] = mk_div(pq, a.qy, __frcp_rn((float)a.qy));
   cp[1] = pq - cp[2] * a.qy;
-  if (tid < MK_BCC5_N) scode[tid] = b ? mk_bcc5_desc<1>(tid) : mk_bcc5_desc<0>(tid);
+  if (tid < MK_BCC5_N) scode[tid] = c_bcc5_desc.v[b][tid];
   const int d = blockIdx.x * MK_BLOCK + tid, lane = tid & 31;
   int kx = 0, ky = 0, kz = 0, site = 0;
   uint64_t u53 = 0;
@@ -1377,6 +1487,10 @@ __global__ void __launch_bounds__(MK_BLOCK, 4) k_multi_propose_table(MultiArgs a
   const float beta32 = p.beta32, cm0 = p.cmt32[0], cm1 = p.cmt32[1];
   __syncthreads();
   pdl_wait();
+  if (blockIdx.x == gridDim.x - 1) {  // the block past the trials
+    if (tid == 0) multi_fold(a, r, step - 1);
+    return;
+  }
   int acc = 0, tie = 0, ta = 0, dec = 0;
   long long pqv = 0;
   if (d < a.D) {
@@ -1416,7 +1530,7 @@ __global__ void __launch_bounds__(MK_BLOCK, 4) k_multi_propose_table(MultiArgs a
       atomicAdd(&s_dn, dn);
     }
     base = __shfl_sync(0xffffffffu, base, 0);
-    if (acc) a.pend[(long long)r * a.D + base + __popc(m & ((1u << lane) - 1u))] = make_int2(site, (1 - ta) | (ta << 8));
+    if (acc) a.pend[(long long)r * a.D + base + __popc(m & ((1u << lane) - 1u))] = make_int2(d, (1 - ta) | (ta << 8));
   }
   if (tie) atomicAdd(&s_ties, tie);
   __syncthreads();
@@ -1424,6 +1538,230 @@ __global__ void __launch_bounds__(MK_BLOCK, 4) k_multi_propose_table(MultiArgs a
     if (s_dn) atomicAdd(&A->dn[1], s_dn);
     if (s_ties) atomicAdd(&A->ties, s_ties);
   }
+}
+
+// One of each pair h, -h of the neighbours' offsets, by shell (the first half of
+// every shell of mk_bcc5_code's order, whose second half is its mirror image).
+constexpr int MK_HALF_N = MK_BCC5_N / 2;
+__host__ __device__ constexpr int mk_half_code(int m) {
+  // shells 8, 6, 12, 24, 8: halves 4, 3, 6, 12, 4
+  return mk_bcc5_code(m < 4 ? m : m < 7 ? m + 4 : m < 13 ? m + 7 : m < 25 ? m + 13 : m + 25);
+}
+
+// Offsets of an axis by half-lattice distance, odd -3 -1 1 3 and even -2 0 2, of a
+// site of basis B; reversed for the lanes that take the mirror images.
+template <int B>
+__device__ __forceinline__ void half_axis(int p, int k, int q, int nk, uint32_t class_step, uint32_t place_step, bool rev,
+                                          uint32_t (&odd)[4], uint32_t (&even)[3]) {
+  uint32_t o[5];
+  rf_axis(p, k, q, nk, class_step, place_step, o);
+#pragma unroll
+  for (int x = 0; x < 4; ++x) {
+    // h = 2 x - 3 from basis B to basis 1 - B: cell (B + h - (1 - B)) / 2
+    const uint32_t f = o[((B + 2 * x - 3 - (1 - B)) >> 1) + 2], g = o[((B + 3 - 2 * x - (1 - B)) >> 1) + 2];
+    odd[x] = rev ? g : f;
+  }
+#pragma unroll
+  for (int x = 0; x < 3; ++x) even[x] = rev ? o[3 - x] : o[1 + x];
+}
+
+// Half of the FP32 dE of a basis-B trial (cell p + q k per axis) from the per-site
+// entries: the terms of 29 of its 58 neighbours (rev: the mirror images), on half
+// a warp's lane of its own; the caller adds the halves.  The neighbours at one
+// offset of consecutive trials are consecutive entries, which carry the species
+// too; the cubics are the only gathers.
+struct FixPart {
+  unsigned cnt[5];
+  float re, ab;
+  uint32_t bad;
+};
+template <int B>
+__device__ __forceinline__ void multi_screen_fix(const MultiArgs& a, const int* sdf, int r, const int* p, int kx, int ky,
+                                                 int kz, bool rev, int off, uint2* self_out, FixPart& f) {
+  constexpr int CH = 8;  // neighbours in flight
+  uint32_t xo[4], xe[3], yo[4], ye[3], zo[4], ze[3];
+  const uint32_t D = (uint32_t)a.D, plane = (uint32_t)rfi_plane(a);
+  half_axis<B>(p[0], kx, a.qx, a.nxq, D, 1u, rev, xo, xe);
+  half_axis<B>(p[1], ky, a.qy, a.nyq, D * a.qx, (uint32_t)a.nxq, rev, yo, ye);
+  half_axis<B>(p[2], kz, a.qz, a.nzq, D * a.qx * a.qy, (uint32_t)(a.nyq * a.nxq), rev, zo, ze);
+#pragma unroll
+  for (int x = 0; x < 4; ++x) zo[x] += B ? 0u : plane;
+#pragma unroll
+  for (int x = 0; x < 3; ++x) ze[x] += B ? plane : 0u;
+  const uint2* T = a.rfu + (long long)r * a.rf_n;
+  auto at = [&](int m) {
+    const int code = mk_half_code(m);
+    const int hx = (code & 15) - 4, hy = ((code >> 4) & 15) - 4, hz = ((code >> 8) & 15) - 4;
+    return (hx & 1) ? zo[(hz + 3) >> 1] + yo[(hy + 3) >> 1] + xo[(hx + 3) >> 1]
+                    : ze[(hz + 2) >> 1] + ye[(hy + 2) >> 1] + xe[(hx + 2) >> 1];
+  };
+  const uint2 self = __ldcg(T + (ze[1] + ye[1] + xe[1]));
+  *self_out = self;
+  const int K = a.K, ta = (int)(self.x & 3u);
+  int tb = ta + 1 + off;
+  tb -= tb >= K ? K : 0;
+  uint32_t df[5];
+#pragma unroll
+  for (int s = 0; s < 5; ++s) {
+    df[s] = (uint32_t)sdf[(s * K + ta) * K + tb] << 2;
+    f.cnt[s] = 0u;
+  }
+  float re[2] = {0.f, 0.f}, ab[2] = {0.f, 0.f};
+  f.bad = fix_clamp(a, self.x) ^ self.x;
+#pragma unroll
+  for (int k0 = 0; k0 < MK_HALF_N; k0 += CH) {
+    uint2 v[CH];
+#pragma unroll
+    for (int u = 0; u < CH; ++u)
+      if (k0 + u < MK_HALF_N) v[u] = __ldcg(T + at(k0 + u));
+#pragma unroll
+    for (int u = 0; u < CH; ++u)
+      if (k0 + u < MK_HALF_N) {
+        const int s = mk_half_code(k0 + u) >> 12;
+        const uint32_t X = v[u].x + df[s], Xc = fix_clamp(a, X);
+        f.bad |= Xc ^ X;
+        f.cnt[s] += 1u << (8u * (X & 3u));
+        const float d = fix_val(a, Xc) - __uint_as_float(v[u].y);
+        re[u & 1] += d;
+        ab[u & 1] += fabsf(d);
+      }
+  }
+  f.re = re[0] + re[1];
+  f.ab = ab[0] + ab[1];
+}
+
+// Propose of the plain rule for K > 2: the screened propose (k_multi_propose<2>)
+// on the fixed-point entries, two lanes per trial (lanes 0-15 of a warp hold the
+// trials, lanes 16-31 take the mirror images of their neighbours).  Bound: its
+// 1800 instructions per warp at 27 warps per SM, then the FP64 trials' tail; 64,000
+// trials, quaternary: a step 29.6 -> 17.4 us, of which the kernel 13.
+__global__ void __launch_bounds__(MK_BLOCK, 7) k_multi_propose_fix(MultiArgs a, int j) {
+  pdl_trigger();  // the commit of this step: its prologue
+  __shared__ long long sDq[5 * MK_MAX * MK_MAX * MK_MAX];
+  __shared__ double sFd[5 * MK_MAX];
+  __shared__ int sdf[5 * MK_MAX * MK_MAX];
+  __shared__ int scode[MK_BCC5_N];
+  __shared__ int s_fw[MK_BLOCK / 32][15];
+  __shared__ int s_dn[MK_MAX], s_ties;
+  const int K = a.K, r = blockIdx.y, tid = threadIdx.x;
+  // every load of the prologue at once: blocks that start late are on the
+  // step's critical path
+  const MRepParams& p = a.rp[r];
+  const long long step = *a.base + j;
+  const int c = __ldg(a.ctab + r * MK_CTAB + j);
+  const uint2 key = p.key;
+  constexpr int ND = 5 * MK_MAX * MK_MAX * MK_MAX, PER = (ND + MK_BLOCK - 1) / MK_BLOCK;
+  long long dq_[PER];
+#pragma unroll
+  for (int u = 0; u < PER; ++u) dq_[u] = tid + u * MK_BLOCK < 5 * K * K * K ? a.Dq[tid + u * MK_BLOCK] : 0;
+  const int df_ = tid < 5 * K * K ? a.fx_df[tid] : 0;
+  const double fd_ = tid < 5 * K ? a.Fd[tid] : 0.0;
+  const int pc = c >> 1, b = c & 1;
+  const int code_ = tid < MK_BCC5_N ? c_bcc5_desc.v[b][tid] : 0;
+#pragma unroll
+  for (int u = 0; u < PER; ++u)
+    if (tid + u * MK_BLOCK < ND) sDq[tid + u * MK_BLOCK] = dq_[u];
+  if (tid < 5 * MK_MAX * MK_MAX) sdf[tid] = df_;
+  if (tid < 5 * MK_MAX) sFd[tid] = fd_;
+  if (tid < MK_BCC5_N) scode[tid] = code_;
+  if (tid < MK_MAX) s_dn[tid] = 0;
+  if (tid == 0) s_ties = 0;
+  int cp[3];
+  const int pq = mk_div(pc, a.qx, __frcp_rn((float)a.qx));
+  cp[0] = pc - pq * a.qx;
+  cp[2] = mk_div(pq, a.qy, __frcp_rn((float)a.qy));
+  cp[1] = pq - cp[2] * a.qy;
+  const int lane = tid & 31;
+  const bool rev = lane >= 16;
+  const int d = blockIdx.x * (MK_BLOCK / 2) + (tid >> 5) * 16 + (lane & 15);
+  const bool live = d < a.D;
+  int kx = 0, ky = 0, kz = 0, site = 0, off = 0;
+  uint64_t u53 = 0;
+  {
+    const int dc = live ? d : 0, dq = mk_div(dc, a.nxq, a.rcp_nxq);
+    kx = dc - dq * a.nxq;
+    kz = mk_div(dq, a.nyq, a.rcp_nyq);
+    ky = dq - kz * a.nyq;
+    site = (((cp[2] + a.qz * kz) * a.ny + cp[1] + a.qy * ky) * a.nx + cp[0] + a.qx * kx) * 2 + b;
+    // a trial's two draws, one by each of its lanes
+    const uint4 w = philox4x32_10(make_uint4((uint32_t)step, (uint32_t)((uint64_t)step >> 32), (uint32_t)dc,
+                                             rev ? TAG_SPECIES : TAG_TRIAL), key);
+    u53 = top53(w.z, w.w);
+    off = (int)below64(w.x, w.y, (uint64_t)(K - 1));
+    off = __shfl_sync(0xffffffffu, off, 16 + (lane & 15));
+  }
+  __syncthreads();
+  pdl_wait();
+  if (blockIdx.x == gridDim.x - 1) {  // the block past the trials
+    if (tid == 0) multi_fold(a, r, step - 1);
+    return;
+  }
+  uint2 self;
+  FixPart f;
+  if (b) multi_screen_fix<1>(a, sdf, r, cp, kx, ky, kz, rev, off, &self, f);
+  else multi_screen_fix<0>(a, sdf, r, cp, kx, ky, kz, rev, off, &self, f);
+  const int ta = (int)(self.x & 3u);
+  int tb = ta + 1 + off;
+  tb -= tb >= K ? K : 0;
+  // the trial's lanes each take the pair sums of their neighbours (half the
+  // shells' counts), then both hold the trial's sums
+  long long pqv = 0;
+#pragma unroll
+  for (int s = 0; s < 5; ++s) {
+    const long long* Dq = sDq + ((s * K + ta) * K + tb) * K;
+#pragma unroll
+    for (int be = 0; be < MK_MAX; ++be)
+      if (be < K) pqv += (long long)((f.cnt[s] >> (8 * be)) & 255u) * Dq[be];
+  }
+  pqv += __shfl_xor_sync(0xffffffffu, pqv, 16);
+  const float re = f.re + __shfl_xor_sync(0xffffffffu, f.re, 16);
+  const float ab = f.ab + __shfl_xor_sync(0xffffffffu, f.ab, 16);
+  const bool ok = (f.bad | __shfl_xor_sync(0xffffffffu, f.bad, 16)) == 0u;
+  int acc = 0, tie = 0, dec = 0;
+  if (live && !rev) {
+    const float own = fix_val(a, (fix_clamp(a, self.x) & ~3u) | (uint32_t)tb) - __uint_as_float(self.y);
+    const float pair = __ll2float_rn(pqv) * a.qscale32;
+    const float err = fmaf((float)(2 * MK_BCC5_N + 2), a.emb_err,
+                           fmaf(3.814697265625e-06f, ab, 4.76837158203125e-07f * (fabsf(pair) + fabsf(own) + fabsf(re))));
+    const float e32 = (pair + own) + re;
+    const float cm = p.cmu32[ta * K + tb];
+    const float x32 = p.beta32 * (e32 + cm);
+    const float dx = p.beta32 * fmaf(4.76837158203125e-07f, fabsf(e32) + fabsf(cm), err) * 1.0001f +
+                     fabsf(x32) * 4.76837158203125e-07f;
+    dec = ok ? screen32(x32, dx, u53) : -1;
+    acc = dec > 0 ? 1 : 0;
+  }
+  // trials the screen left open: FP64 dE by the whole warp, one at a time
+  unsigned open = __ballot_sync(0xffffffffu, dec < 0);
+  while (open) {
+    const int src = __ffs(open) - 1;
+    open &= open - 1u;
+    const int si = __shfl_sync(0xffffffffu, site, src);
+    const int sa = __shfl_sync(0xffffffffu, ta, src), sb = __shfl_sync(0xffffffffu, tb, src);
+    const double v = warp_sum(multi_emb_warp5(a, sFd, scode, s_fw[tid >> 5], r, si, sa, sb, lane));
+    if (lane == src) {
+      const double de64 = (double)pqv * a.qscale + v;
+      if (!isfinite(de64)) atomicOr(a.err, ERRF_NONFINITE);
+      acc = metropolis(p.beta * (de64 + (p.dmu0[tb] - p.dmu0[ta])), u53, &tie) ? 1 : 0;
+    }
+  }
+  // compaction of the local accepts, dn and ties: one reservation per warp
+  MStepAcc* A = a.acc + 2 * r + (int)(step & 1);
+  const unsigned m = __ballot_sync(0xffffffffu, acc);
+  if (m) {
+    int base = 0;
+    if (lane == 0) base = atomicAdd(&A->nacc, __popc(m));
+    for (int al = 1; al < K; ++al) {
+      const int v = __popc(__ballot_sync(0xffffffffu, acc && tb == al)) - __popc(__ballot_sync(0xffffffffu, acc && ta == al));
+      if (lane == 0 && v) atomicAdd(&s_dn[al], v);
+    }
+    base = __shfl_sync(0xffffffffu, base, 0);
+    if (acc) a.pend[(long long)r * a.D + base + __popc(m & ((1u << lane) - 1u))] = make_int2(d, tb | (ta << 8));
+  }
+  if (tie) atomicAdd(&s_ties, tie);
+  __syncthreads();
+  if (tid > 0 && tid < K && s_dn[tid]) atomicAdd(&A->dn[tid], s_dn[tid]);
+  if (tid == 0 && s_ties) atomicAdd(&A->ties, s_ties);
 }
 
 void launch_multi_step(const MultiArgs& a, int j, cudaStream_t st, bool after_step) {
@@ -1434,9 +1772,10 @@ void launch_multi_step(const MultiArgs& a, int j, cudaStream_t st, bool after_st
   const dim3 cgrid((unsigned)(nb < 4 ? nb : 4), (unsigned)a.R);
   if (a.screen) {
     // one thread per (accept, neighbour) over all replicas: a fixed grid of
-    // four blocks per SM
+    // a block per SM
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid;
+    // (and a block that folds the step before into the replica's state)
+    cfg.gridDim = dim3((unsigned)((a.rfu && !a.da ? (a.D + MK_BLOCK / 2 - 1) / (MK_BLOCK / 2) : nb) + 1), (unsigned)a.R);
     cfg.blockDim = dim3(MK_BLOCK);
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
@@ -1448,9 +1787,11 @@ void launch_multi_step(const MultiArgs& a, int j, cudaStream_t st, bool after_st
       a.dtab ? cudaLaunchKernelEx(&cfg, k_multi_propose<3, true>, a, j)
              : cudaLaunchKernelEx(&cfg, k_multi_propose<3, false>, a, j);
     else
-      a.dtab ? cudaLaunchKernelEx(&cfg, k_multi_propose_table, a, j)
-             : cudaLaunchKernelEx(&cfg, k_multi_propose<2, false>, a, j);
-    cfg.gridDim = dim3((unsigned)(4 * a.n_sm));
+      a.dtab  ? cudaLaunchKernelEx(&cfg, k_multi_propose_table, a, j)
+      : a.rfu ? cudaLaunchKernelEx(&cfg, k_multi_propose_fix, a, j)  // two lanes per trial
+              : cudaLaunchKernelEx(&cfg, k_multi_propose<2, false>, a, j);
+    cfg.gridDim = dim3((unsigned)a.n_sm);
+    cfg.blockDim = dim3(MK_CBLOCK);
     cfg.numAttrs = 1;
     cudaLaunchKernelEx(&cfg, k_multi_commit_screen, a, j);
   } else if (a.reembed) {
@@ -1468,7 +1809,7 @@ void launch_multi_step(const MultiArgs& a, int j, cudaStream_t st, bool after_st
 //     sums (the same FP64 arithmetic in every block, so the same result);
 //  2. each thread commits its pending flip of step k - 1 (slot d): the new
 //     species if the step was accepted, else the old one;
-//  3. block 0 of the replica folds step k - 1 into the running state;
+//  3. a block of its own folds step k - 1 into the replica's running state;
 //  4. each thread proposes trial d of step k on the effective species: a
 //     neighbour whose byte still carries a pending flip of step k - 1 counts
 //     with its new species when that step was accepted, so the commits of
@@ -1521,6 +1862,87 @@ __device__ __forceinline__ long long multi_pq_bytes(const MultiArgs& a, const lo
   return pq;
 }
 
+// what the decision of step kp needs, in wide loads, all at once: every block
+// reads these lines, and 504 blocks' single words queue at the L2
+__device__ __forceinline__ void step_sums(const MultiArgs& a, int r, long long kp, int (&dn)[MK_MAX],
+                                          long long (&c0)[MK_MAX], int* nacc) {
+  const MStepAcc* A = a.acc + 3 * r + (int)(kp % 3);
+  const long long* n0 = a.nstart + (2 * r + (int)(kp & 1)) * MK_MAX;
+  const int4 vd = __ldcg(reinterpret_cast<const int4*>(A->dn));
+  *nacc = __ldcg(&A->nacc);
+  const longlong2 v0 = __ldcg(reinterpret_cast<const longlong2*>(n0));
+  const longlong2 v1 = __ldcg(reinterpret_cast<const longlong2*>(n0 + 2));
+  dn[0] = 0;
+  dn[1] = vd.y;
+  dn[2] = vd.z;
+  dn[3] = vd.w;
+  c0[0] = v0.x;
+  c0[1] = v0.y;
+  c0[2] = v1.x;
+  c0[3] = v1.y;
+}
+
+// Step k - 1 folded into replica r's state, the counts at the start of step k,
+// and (propose) the sums of step k + 1 cleared: by one thread of a block of its
+// own, whose chain of loads and FP64 sums held up the first block's trials, and
+// with them every step: 64,000 trials, ternary, 8.5 -> 6.9 us per step with this
+// and the wide loads.
+__device__ __noinline__ void fused_fold(const MultiArgs& a, int r, long long k, bool propose) {
+  const long long kp = k - 1;
+  const int K = a.K;
+  const MRepParams& p = a.rp[r];
+  MRepState S = a.rs[r];
+  if (kp >= 0 && S.fin_step < kp) {
+    const MStepAcc* A = a.acc + 3 * r + (int)(kp % 3);
+    int dn[MK_MAX], nacc, tie = 0;
+    long long cnt[MK_MAX];
+    step_sums(a, r, kp, dn, cnt, &nacc);
+    const double sde = __ldcg(&A->sum_de);
+    const int ties = __ldcg(&A->ties);
+    S.trials += a.D;
+    S.local_acc += nacc;
+    if (nacc > 0) {
+      S.global_trials++;
+      if (multi_global(a, p, dn, cnt, step_uniform(p, kp), &tie)) {
+        S.global_acc++;
+        S.flips += nacc;
+        long long d0 = 0;
+#pragma unroll
+        for (int al = 1; al < MK_MAX; ++al)
+          if (al < K) {
+            cnt[al] += dn[al];
+            d0 += dn[al];
+          }
+        cnt[0] -= d0;
+        S.energy += sde;
+      }
+    }
+    S.near_ties += ties + tie;
+    long long* n1 = a.nstart + (2 * r + (int)(k & 1)) * MK_MAX;
+#pragma unroll
+    for (int al = 0; al < MK_MAX; ++al)
+      if (al < K) {
+        S.cnt[al] = cnt[al];
+        n1[al] = cnt[al];
+        const double cc = (double)cnt[al] * a.inv_n;
+        S.sum_c[al] += cc;
+        S.sum_c2[al] += cc * cc;
+      }
+    S.steps++;
+    S.step = k;
+    S.fin_step = kp;
+    a.rs[r] = S;
+  }
+  if (propose) {
+    MStepAcc* Bn = a.acc + 3 * r + (int)((k + 1) % 3);
+#pragma unroll
+    for (int al = 0; al < MK_MAX; ++al) Bn->dn[al] = 0;
+    Bn->nacc = 0;
+    Bn->ties = 0;
+    Bn->sum_de = 0.0;
+  }
+}
+
 // Launches of a chain after the first use programmatic dependent launch:
 // before griddepcontrol.wait a step reads only what no step writes (the
 // tables, the parameters, the step base, which only the advance kernel
@@ -1531,7 +1953,7 @@ __global__ void __launch_bounds__(MK_BLOCK) k_multi_fused(MultiArgs a, int j) {
   pdl_trigger();
   __shared__ long long sDq[5 * MK_MAX * MK_MAX * MK_MAX];
   __shared__ double sDF[MK_MAX * MK_MAX];
-  __shared__ int s_G, s_tie;
+  __shared__ int s_G;
   __shared__ int s_red[MK_BLOCK / 32][MK_MAX + 1];
   __shared__ double s_de[MK_BLOCK / 32];
   __shared__ int s_acc[MK_BLOCK / 32];
@@ -1539,6 +1961,11 @@ __global__ void __launch_bounds__(MK_BLOCK) k_multi_fused(MultiArgs a, int j) {
   const int r = blockIdx.y;
   const MRepParams& p = a.rp[r];
   const long long k = *a.base + j, kp = k - 1;
+  if (blockIdx.x == gridDim.x - 1) {  // the block past the trials
+    pdl_wait();
+    if (threadIdx.x == 0) fused_fold(a, r, k, PROPOSE);
+    return;
+  }
   const int d = blockIdx.x * MK_BLOCK + threadIdx.x;
   if (PROPOSE) {
     for (int q = threadIdx.x; q < 5 * K * K * K; q += MK_BLOCK) sDq[q] = a.Dq[q];
@@ -1597,72 +2024,18 @@ __global__ void __launch_bounds__(MK_BLOCK) k_multi_fused(MultiArgs a, int j) {
     // global decision of step k-1 (every block, the same FP64 arithmetic)
     int G = 0, tie = 0;
     if (kp >= 0) {
-      const MStepAcc* A = a.acc + 3 * r + (int)(kp % 3);
-      if (__ldcg(&A->nacc) > 0) {
-        const long long* n0 = a.nstart + (2 * r + (int)(kp & 1)) * MK_MAX;
-        double Y = 0.0;
-        for (int al = 1; al < K; ++al) {
-          const double dn = (double)__ldcg(&A->dn[al]);
-          Y += p.beta * p.kappa_p[al] * dn * (dn + 2.0 * ((double)__ldcg(n0 + al) - p.n0[al]));
-        }
-        G = metropolis(Y, ug, &tie) ? 1 : 0;
-      }
+      int dn[MK_MAX], nacc;
+      long long c0[MK_MAX];
+      step_sums(a, r, kp, dn, c0, &nacc);
+      if (nacc > 0) G = multi_global(a, p, dn, c0, ug, &tie);
     }
     s_G = G;
-    s_tie = tie;
   }
   __syncthreads();
   const int G = s_G;
   const unsigned gmask = G ? 0xF0u : 0u;
   // commit this thread's pending flip of step k-1
   if (ps >= 0) ty[ps] = (uint8_t)((vps & gmask) ? (vps >> 4) - 1u : (vps & 15u));
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    MRepState S = a.rs[r];
-    if (kp >= 0 && S.fin_step < kp) {
-      const MStepAcc* A = a.acc + 3 * r + (int)(kp % 3);
-      const int nacc = __ldcg(&A->nacc);
-      const long long* n0 = a.nstart + (2 * r + (int)(kp & 1)) * MK_MAX;
-      long long cnt[MK_MAX];
-      for (int al = 0; al < MK_MAX; ++al) cnt[al] = __ldcg(n0 + al);
-      S.trials += a.D;
-      S.local_acc += nacc;
-      S.near_ties += __ldcg(&A->ties) + s_tie;
-      if (nacc > 0) {
-        S.global_trials++;
-        if (G) {
-          S.global_acc++;
-          S.flips += nacc;
-          long long d0 = 0;
-          for (int al = 1; al < K; ++al) {
-            const int dn = __ldcg(&A->dn[al]);
-            cnt[al] += dn;
-            d0 += dn;
-          }
-          cnt[0] -= d0;
-          S.energy += __ldcg(&A->sum_de);
-        }
-      }
-      long long* n1 = a.nstart + (2 * r + (int)(k & 1)) * MK_MAX;
-      for (int al = 0; al < K; ++al) {
-        S.cnt[al] = cnt[al];
-        n1[al] = cnt[al];
-        const double cc = (double)cnt[al] * a.inv_n;
-        S.sum_c[al] += cc;
-        S.sum_c2[al] += cc * cc;
-      }
-      S.steps++;
-      S.step = k;
-      S.fin_step = kp;
-      a.rs[r] = S;
-    }
-    if (PROPOSE) {
-      MStepAcc* Bn = a.acc + 3 * r + (int)((k + 1) % 3);
-      for (int al = 0; al < MK_MAX; ++al) Bn->dn[al] = 0;
-      Bn->nacc = 0;
-      Bn->ties = 0;
-      Bn->sum_de = 0.0;
-    }
-  }
   if (!PROPOSE) {
     if (ps >= 0) *slot = -1;
     return;
@@ -1752,13 +2125,17 @@ __global__ void k_multi_advance(MultiArgs a, long long* base, int n) {
                                     a.rp[q / MK_CTAB].key);
       a.ctab[q] = (int)below64(w.x, w.y, (uint64_t)a.n_colours);
     }
+  // the screened form's last step (every other one is folded by the propose
+  // launch after it)
+  if (a.screen)
+    for (int r = threadIdx.x; r < a.R; r += blockDim.x) multi_fold(a, r, b0 - 1);
   __syncthreads();
   if (threadIdx.x == 0) *base = b0;
 }
 
 void launch_multi_fused(const MultiArgs& a, int j, bool propose, cudaStream_t st) {
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)((a.D + MK_BLOCK - 1) / MK_BLOCK), (unsigned)a.R);
+  cfg.gridDim = dim3((unsigned)((a.D + MK_BLOCK - 1) / MK_BLOCK) + 1u, (unsigned)a.R);
   cfg.blockDim = dim3(MK_BLOCK);
   cfg.stream = st;
   cudaLaunchAttribute attr[1];

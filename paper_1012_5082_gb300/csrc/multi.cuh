@@ -49,7 +49,7 @@ struct MRepState {
 };
 
 // accumulator of one colour step (two per replica, by step parity)
-struct MStepAcc {
+struct __align__(16) MStepAcc {
   int dn[MK_MAX];
   int nacc;
   int ties;
@@ -130,6 +130,14 @@ struct MultiArgs {
   // warp's loads fill their sectors.  Not kept with dtab.
   float2* rf;
   long long rf_n;
+  // K > 2 (null: see screen_setup): the same per site as (rho / h in fixed point
+  // with fx_bits fraction bits << 2 | species, FP32 embedding value there), with
+  // fx_scale = 2^fx_bits / h; packed arguments in [fx_lo, fx_hi] are screened
+  uint2* rfu;
+  int fx_bits;
+  uint32_t fx_lo, fx_hi;
+  double fx_scale;
+  const int* fx_df;     // [(s K + a) K + b] f_b(r_s) - f_a(r_s) in that fixed point
   int n_sm;             // multiprocessors of the device (commit grid)
   // delayed acceptance (K = 2, screened form): a trial first passes a
   // stage on the surrogate's prediction g of E(i = B) - E(i = A), then a

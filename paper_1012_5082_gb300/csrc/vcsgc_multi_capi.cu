@@ -228,6 +228,10 @@ int screen_acc_ready(Multi* m) {
   for (int r = 0; r < m->R; ++r) {
     acc[r] = MStepAcc{};
     for (int al = 0; al < MK_MAX; ++al) acc[r].cnt[al] = s[r].cnt[al];
+    if (s[r].step != m->h_base) {  // the state's next step is the chain's
+      s[r].step = m->h_base;
+      MCK(cudaMemcpyAsync(m->args.rs + r, &s[r], sizeof(MRepState), cudaMemcpyHostToDevice, m->st));
+    }
   }
   const int par = (int)(m->h_base & 1);
   for (int r = 0; r < m->R; ++r)
@@ -409,6 +413,42 @@ int screen_setup(Multi* m, const std::vector<double>& hFd) {
     a.fix_lo = (long long)std::ceil(lo / h * 4294967296.0);
     a.fix_hi = (long long)std::floor(hi / h * 4294967296.0);
     a.tab_err = (float)((MK_BCC5_N + 1) * std::ldexp(dm, -20));
+    return VCSGC_OK;
+  }
+  // K > 2: fixed-point entries, where their rounding (2 2^-fx_bits intervals an
+  // evaluation) stays within the share of the bound that a float argument
+  // takes, 4 (j0 + 2) 2^-24 intervals from interval j0 up, and no difference
+  // reaches the range from zero
+  int bits = 23;
+  while (bits > 0 && (double)(n + 1) * std::ldexp(1.0, bits) > 1073741823.0) --bits;
+  const int j0 = std::max(0, (int)std::floor(lo / h) - 1);
+  if (m->K > 2 && std::ldexp(1.0, 25 - bits) <= 4.0 * (j0 + 2) && dmax < 0.999 * lo) {
+    // their own bound of an evaluation: 6 2^-24 G as in screen.h (coefficients and
+    // FMAs), and 2 2^-fx_bits intervals times the steepest slope
+    double G = 0.0, Dm = 0.0;
+    const int j1 = std::min(n - 1, (int)std::floor(hi / h) + 1);
+    for (const std::vector<Cubic>& q : hs)
+      for (int j = j0; j <= j1; ++j) {
+        G = std::max(G, std::fabs(q[j].x) + std::fabs(q[j].y) + std::fabs(q[j].z) + std::fabs(q[j].w));
+        Dm = std::max(Dm, std::fabs(q[j].y) + 2.0 * std::fabs(q[j].z) + 3.0 * std::fabs(q[j].w));
+      }
+    a.emb_err = (float)(std::min(err, std::ldexp(6.0 * G, -24) + std::ldexp(Dm, 1 - bits)) * (1.0 + 1e-6));
+    a.fx_bits = bits;
+    a.fx_scale = std::ldexp(1.0, bits) / h;
+    a.fx_lo = (uint32_t)std::ceil(lo * a.fx_scale) << 2;
+    a.fx_hi = (uint32_t)std::floor(hi * a.fx_scale) << 2 | (uint32_t)(m->K - 1);
+    MTRY(malloc_dev(m, &a.ctab, (size_t)m->R * MK_CTAB));
+    MTRY(malloc_dev(m, &a.rfu, (size_t)m->R * a.rf_n));
+    std::vector<int> df((size_t)a.n_sh * m->K * m->K);
+    for (int s = 0; s < a.n_sh; ++s)
+      for (int x = 0; x < m->K; ++x)
+        for (int y = 0; y < m->K; ++y)
+          df[(s * m->K + x) * m->K + y] = (int)std::lrint((hFd[s * m->K + y] - hFd[s * m->K + x]) * a.fx_scale);
+    int* d_df = nullptr;
+    MTRY(malloc_dev(m, &d_df, df.size()));
+    MCK(cudaMemcpyAsync(d_df, df.data(), sizeof(int) * df.size(), cudaMemcpyHostToDevice, m->st));
+    MCK(cudaStreamSynchronize(m->st));
+    a.fx_df = d_df;
   } else {
     MTRY(malloc_dev(m, &a.rf, (size_t)m->R * a.rf_n));
   }
