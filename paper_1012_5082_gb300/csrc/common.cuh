@@ -178,6 +178,11 @@ __device__ __forceinline__ float narrow_pos(double d) {
 // their two conversions took eleven.  The term 3 e^2 / 8 < 2^-41 is formed in
 // FP32 (below 2^-63 of the result).
 __device__ __forceinline__ double sqrt3(double r2, double& ir) {
+  if ((uint32_t)__double2hiint(r2) < 0x38100000u) {  // below float's range: r2 = 0 gives NaN, as an error must
+    asm volatile("");  // keeps this a branch
+    ir = rsqrt_nr(r2);
+    return r2 * ir;
+  }
   const double y = widen(rsqrtf(narrow_pos(r2)));
   const double s = r2 * y, e = fma(-s, y, 1.0);
   const uint32_t eh = (uint32_t)__double2hiint(e) & 0x7FFFFFFFu;
@@ -243,6 +248,17 @@ __device__ __forceinline__ int locate_bits(double u, int n_int, double& t) {
   t = u - fl;
   return j;
 }
+
+// interval and offset of r on a table grid when 0 <= r < r_c <= the grid's
+// end is already known (no range test)
+__device__ __forceinline__ int locate_u(const Spline& s, double u, double& t) {
+  if (s.n_int < (1 << 19)) return locate_bits(u, s.n_int, t);
+  int j = (int)u;
+  j = j < s.n_int - 1 ? j : s.n_int - 1;
+  t = u - (double)j;
+  return j;
+}
+__device__ __forceinline__ int locate_in(const Spline& s, double r, double& t) { return locate_u(s, r * s.inv_h, t); }
 
 // ------------------------------------------------- FP32 tables (mixed form)
 // The mixed-precision form evaluates pair, density and embedding-table

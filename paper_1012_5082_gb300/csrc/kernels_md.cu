@@ -51,18 +51,6 @@ __global__ void k_md_rho(MdArgs m) {
   if (MIXED) m.dFp32[i] = (float)m.dFp[i];
   m.dF[i] = spline_val_at(m.tab.sp[6], q, t) - spline_val_at(m.tab.sp[5], q, t);
 }
-
-// interval and offset of r on a table grid when 0 <= r < r_c <= the grid's
-// end is already known (no range test)
-__device__ __forceinline__ int locate_u(const Spline& s, double u, double& t) {
-  if (s.n_int < (1 << 19)) return locate_bits(u, s.n_int, t);
-  int j = (int)u;
-  j = j < s.n_int - 1 ? j : s.n_int - 1;
-  t = u - (double)j;
-  return j;
-}
-__device__ __forceinline__ int locate_in(const Spline& s, double r, double& t) { return locate_u(s, r * s.inv_h, t); }
-
 // Position and species of every atom in one 32-byte record (FP64 passes) or
 // one 16-byte one (mixed): a neighbour is one sector instead of four.
 __global__ void k_md_records(MdArgs m) {

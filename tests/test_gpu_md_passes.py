@@ -99,3 +99,14 @@ def test_long_rows_take_several_lists(V):
     for a in range(3):
         assert np.max(np.abs(Fg[a] - Fo[a])) < 1e-10
     g.close()
+
+
+def test_coincident_atoms_are_an_error(V):
+    """Two atoms at one place have no force direction: refused, not finite."""
+    lat = I.bcc_lattice(6, 6, 6)
+    x, y, z = (np.array(a) for a in (lat.x, lat.y, lat.z))
+    x[101], y[101], z[101] = x[40], y[40], z[40]
+    bad = I.Lattice(x=x, y=y, z=z, box=lat.box.copy())
+    with pytest.raises(Exception):
+        V.Context(bad, np.zeros(lat.n, np.uint8), I.eam_tables(), -2.0, 10.0, 700.0, schedule=V.SCHED_SPATIAL,
+                  sched=(2, 2, 2, 2, 2, 2)).forces()
