@@ -172,6 +172,7 @@ struct Ctx {
   // resident form chosen by size (resident_shape)
   bool shape_set = false;
   int res_size = 0, res_block = 0;  // CTAs per cluster (0: none), trial threads
+  bool no_draws = false;            // no memory for the draws: not by default
   bool cl_offer[5] = {};            // sizes vcsgc_cluster_sizes lists (of cl_tiles)
   int pick_block = 0;               // BLOCKS, OVERLAP: trial threads of the one-CTA form (0: none)
   size_t pick_smem = 0;
@@ -983,9 +984,21 @@ int run_steps_resident(Ctx* c, long long n, int csize, int block) {
 // fewest steps of one call that pay for loading the lattice into shared memory
 constexpr long long RESIDENT_MIN_STEPS = 8;
 
+// whether a call of the default form can run resident: the draws' buffers are
+// there (without memory for them the context goes on with a launch per step)
+// and the caller is not capturing the stream, which takes no allocation
+bool resident_ready(Ctx* c, long long n) {
+  if (c->no_draws || !(c->res_size || c->pick_block)) return false;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(c->st, &cap) != cudaSuccess) cudaGetLastError();
+  if (cap != cudaStreamCaptureStatusNone) return false;
+  if (draw_buffers(c, n) != VCSGC_OK) c->no_draws = true;
+  return !c->no_draws;
+}
+
 int run_steps_fast(Ctx* c, long long n) {
   if (cluster_form_usable(c)) return run_steps_resident(c, n, c->cl_size, c->cl_block);
-  if (!c->shape_set && !c->lat.da && n >= RESIDENT_MIN_STEPS) {
+  if (!c->shape_set && !c->lat.da && n >= RESIDENT_MIN_STEPS && resident_ready(c, n)) {
     if (c->res_size) return run_steps_resident(c, n, c->res_size, c->res_block);
     if (c->pick_block) return run_steps_resident(c, n, 0, c->pick_block);
   }
