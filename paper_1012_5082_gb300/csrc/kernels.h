@@ -199,9 +199,11 @@ struct ChainDraws {
   int2* su;        // else: site, -ln u
   int2* cg;        // [step][R] colour or domains of the colour, -ln of the global uniform
   const int* off;  // [R]
+  long long* base; // first step of the chunk, as the control block had it
   int P, pmax;
 };
-cudaError_t launch_chain_draws(const LatArgs& a, const ChainDraws& cd, long long base, int m, cudaStream_t st);
+// draws of the next m steps of the chain
+cudaError_t launch_chain_draws(const LatArgs& a, const ChainDraws& cd, int m, cudaStream_t st);
 // the footprint by which a size is offered as launch form 1: 64-bit words (32
 // species and 32 pending bits) and 16 bytes per trial
 inline size_t cluster_offer_bytes(const ClTile& t, int W) {
@@ -209,21 +211,22 @@ inline size_t cluster_offer_bytes(const ClTile& t, int W) {
 }
 // largest dynamic shared memory a tile may use
 constexpr size_t CL_SMEM_MAX = 200 * 1024;
-// n colour steps from step `base` of every replica (R clusters of `csize`
+// the n colour steps of cd's chunk for every replica (R clusters of `csize`
 // CTAs of `block` trial threads, block 256 or 512); needs the five-shell or
 // (period 4 along x) two-shell table, the sublattice schedule, a uniform dF
-// and no pending commit.  Returns the launch status.
+// and no pending commit.  The control block's step base and colour table are
+// brought up to the step after.  Returns the launch status.
 cudaError_t launch_cluster_steps(const LatArgs& a, const ClTile* d_tiles, const ChainDraws& cd, size_t smem, int csize,
-                                 int block, long long base, int n, cudaStream_t st);
+                                 int block, int n, cudaStream_t st);
 // clusters of csize CTAs with `smem` bytes each that can be resident at once
 // (0: the shape cannot launch)
 int cluster_capacity(const LatArgs& a, int csize, int block, size_t smem);
-// n colour steps from step `base` of a BLOCKS or OVERLAP schedule, one CTA of
-// `block` threads (a multiple of 32, at most 512) per replica, at most 8
-// trials per thread.  Needs a uniform dF and no pending commit.
+// the same for a BLOCKS or OVERLAP schedule, one CTA of `block` threads (a
+// multiple of 32, at most 512) per replica, at most 8 trials per thread.
+// Needs a uniform dF and no pending commit.
 inline size_t pick_smem_bytes(long long words) { return sizeof(uint32_t) * ((size_t)words + 2); }
 constexpr size_t PICK_SMEM_MAX = 220 * 1024;
-cudaError_t launch_pick_steps(const LatArgs& a, const ChainDraws& cd, size_t smem, int block, long long base, int n,
+cudaError_t launch_pick_steps(const LatArgs& a, const ChainDraws& cd, size_t smem, int block, int n,
                               cudaStream_t st);
 // true when the rows and masks of a equal the compile-time five-shell table
 bool lattice_rows_bcc5(const LatArgs& a);

@@ -320,10 +320,14 @@ struct StepSums {
   }
 };
 
-// what the per-step launch expects after steps base .. base + n - 1: nothing
-// pending, step base + n - 1 finalised, zero accumulators
+// what the per-step launch expects before step kn: nothing pending, step kn - 1
+// finalised, zero accumulators, and (with the colour table, lat_colours_ahead)
+// the step base.  It is written here and not by a launch of its own, or by the
+// host when a per-step launch comes: the chain's position is then the device's
+// alone, whatever the caller captures and replays.
 __device__ __forceinline__ void hand_over(const LatArgs& a, int r, const RepState& S, long long kn) {
   a.rs[r] = S;
+  if (r == 0) a.ctl->base_step = kn;
   a.n_start[r * 2 + (int)(kn & 1)] = S.n;
   StepAcc* A = a.acc + r * 3;
   for (int q = 0; q < 3; ++q) {
@@ -422,20 +426,22 @@ __device__ __forceinline__ int decide(const LatArgs& a, const LatRep& lr, const 
 
 }  // namespace
 
-// Draws of steps base .. base + m - 1: step j's of replica r at lu + j P + off[r]
+// Draws of the next m steps from the control block's base: step j's of replica r at lu + j P + off[r]
 // (SUBLATTICE: -ln u of the trials, rows of the colour padded to whole groups
 // of GS) or su (else: site, -1 past the colour's domains, and -ln u of domain
 // d), and the step's colour (SUBLATTICE) or number of domains and -ln of its
 // global uniform at cg[j R + r].  blockIdx = (trials / 256, j, r).
 template <int GS>
-__global__ void __launch_bounds__(256) k_chain_draws(LatArgs a, ChainDraws cd, long long base) {
+__global__ void __launch_bounds__(256) k_chain_draws(LatArgs a, ChainDraws cd) {
   const int r = blockIdx.z, j = blockIdx.y;
+  const long long base = a.ctl->base_step;
   const LatGeom g = a.geom[r];
   const uint2 key = a.rp[r].key;
   const long long k = base + j;
   const int t = blockIdx.x * 256 + threadIdx.x;
   uint64_t ug;
   int c = 0;
+  if (r + j + t == 0) *cd.base = base;  // the chain moves the control block's while its last CTAs may not have started
   if (GS == 0 || t == 0) c = lat_colour(a, key, k, &ug);
   if (t == 0)
     cd.cg[(size_t)j * a.R + r] =
@@ -474,7 +480,7 @@ struct StepGeo {  // a step's colour on this tile
 
 template <int NSH, bool SWAR, int BS>
 __global__ void __launch_bounds__(BS + 32, 1)
-    k_cluster_steps(LatArgs a, const ClTile* tiles, ChainDraws cd, long long base, int n) {
+    k_cluster_steps(LatArgs a, const ClTile* tiles, ChainDraws cd, int n) {
   extern __shared__ __align__(16) uint32_t cl_smem[];
   __shared__ int s_part[2][16];               // every CTA's dn and nacc (16 bits each), by step parity
   __shared__ int s_acc[2];                    // this CTA's
@@ -486,6 +492,7 @@ __global__ void __launch_bounds__(BS + 32, 1)
 
   const int r = (int)cl_id();
   const uint32_t rank = cl_rank();
+  const long long base = *cd.base;
   const int nctas = (int)cl_nctas();
   const bool solo = nctas == 1;
   const ClTile T = tiles[r];
@@ -805,6 +812,7 @@ __global__ void __launch_bounds__(BS + 32, 1)
     sums.fold(S, a, sb, NSH, sb[NSH], n, n_prev, base + n);
     hand_over(a, r, S, base + n);
   }
+  if (rank == 0) lat_colours_ahead(a, r, p.key, base + n, threadIdx.x, BS + 32);
 }
 
 // ------------------------------------------------ one CTA per replica, picks
@@ -819,7 +827,7 @@ struct PickRow {
 };
 
 template <int NSH, int MAXB>
-__global__ void __launch_bounds__(MAXB, 1) k_pick_steps(LatArgs a, ChainDraws cd, long long base, int n) {
+__global__ void __launch_bounds__(MAXB, 1) k_pick_steps(LatArgs a, ChainDraws cd, int n) {
   extern __shared__ __align__(16) uint32_t cl_smem[];
   constexpr int NS = NSH > 0 ? NSH : LAT_MAX_SH;
   constexpr int NP = (NS + 1) / 2;  // words of two 16-bit per-shell sums
@@ -829,6 +837,7 @@ __global__ void __launch_bounds__(MAXB, 1) k_pick_steps(LatArgs a, ChainDraws cd
 
   const int r = blockIdx.x;
   const int BS = (int)blockDim.x;
+  const long long base = *cd.base;
   const bool one = BS == 32;
   const LatGeom g = a.geom[r];
   const RepParams p = a.rp[r];
@@ -1012,11 +1021,12 @@ __global__ void __launch_bounds__(MAXB, 1) k_pick_steps(LatArgs a, ChainDraws cd
     sums.fold(S, a, sb_sum, NS, s_sb[NS], n, n_prev, base + n);
     hand_over(a, r, S, base + n);
   }
+  lat_colours_ahead(a, r, p.key, base + n, threadIdx.x, BS);
 }
 
 namespace {
 
-using ClusterKernel = void (*)(LatArgs, const ClTile*, ChainDraws, long long, int);
+using ClusterKernel = void (*)(LatArgs, const ClTile*, ChainDraws, int);
 
 template <int BS>
 ClusterKernel cluster_kernel_bs(const LatArgs& a) {
@@ -1046,16 +1056,16 @@ void cluster_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute& attr, int bloc
 
 }  // namespace
 
-cudaError_t launch_chain_draws(const LatArgs& a, const ChainDraws& cd, long long base, int m, cudaStream_t st) {
+cudaError_t launch_chain_draws(const LatArgs& a, const ChainDraws& cd, int m, cudaStream_t st) {
   const dim3 grid((unsigned)((cd.pmax + 255) / 256), (unsigned)m, (unsigned)a.R);
-  if (!a.sublattice) k_chain_draws<0><<<grid, 256, 0, st>>>(a, cd, base);
-  else if (a.qx == 4) k_chain_draws<4><<<grid, 256, 0, st>>>(a, cd, base);
-  else k_chain_draws<1><<<grid, 256, 0, st>>>(a, cd, base);
+  if (!a.sublattice) k_chain_draws<0><<<grid, 256, 0, st>>>(a, cd);
+  else if (a.qx == 4) k_chain_draws<4><<<grid, 256, 0, st>>>(a, cd);
+  else k_chain_draws<1><<<grid, 256, 0, st>>>(a, cd);
   return cudaGetLastError();
 }
 
 cudaError_t launch_cluster_steps(const LatArgs& a, const ClTile* d_tiles, const ChainDraws& cd, size_t smem, int csize,
-                                 int block, long long base, int n, cudaStream_t st) {
+                                 int block, int n, cudaStream_t st) {
   const ClusterKernel k = cluster_kernel(a, block);
   const cudaError_t e = cluster_attributes(k, smem);
   if (e != cudaSuccess) return e;
@@ -1063,7 +1073,7 @@ cudaError_t launch_cluster_steps(const LatArgs& a, const ClTile* d_tiles, const 
   cudaLaunchAttribute attr[1];
   cluster_config(cfg, attr[0], a.R * csize, csize, block, smem);
   cfg.stream = st;
-  return cudaLaunchKernelEx(&cfg, k, a, d_tiles, cd, base, n);
+  return cudaLaunchKernelEx(&cfg, k, a, d_tiles, cd, n);
 }
 
 int cluster_capacity(const LatArgs& a, int csize, int block, size_t smem) {
@@ -1079,13 +1089,12 @@ int cluster_capacity(const LatArgs& a, int csize, int block, size_t smem) {
   return n;
 }
 
-cudaError_t launch_pick_steps(const LatArgs& a, const ChainDraws& cd, size_t smem, int block, long long base, int n,
-                              cudaStream_t st) {
+cudaError_t launch_pick_steps(const LatArgs& a, const ChainDraws& cd, size_t smem, int block, int n, cudaStream_t st) {
   auto k = block <= 64 ? (a.bcc5 ? k_pick_steps<5, 64> : (a.bcc2 ? k_pick_steps<2, 64> : k_pick_steps<0, 64>))
                        : (a.bcc5 ? k_pick_steps<5, 512> : (a.bcc2 ? k_pick_steps<2, 512> : k_pick_steps<0, 512>));
   const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  k<<<a.R, block, smem, st>>>(a, cd, base, n);
+  k<<<a.R, block, smem, st>>>(a, cd, n);
   return cudaGetLastError();
 }
 

@@ -564,14 +564,8 @@ __global__ void k_lattice_advance(LatCtl* ctl, int n) { ctl->base_step += n; }
 // colours and global uniforms of steps base - 1 .. base + LAT_CTAB - 2 of
 // every replica (one block per replica); entries for steps < 0 are zero
 __global__ void k_colour_table(LatArgs a) {
-  const int r = blockIdx.x, t = threadIdx.x;
-  if (t >= LAT_CTAB) return;
-  const long long k = a.ctl->base_step + t - 1;
-  int c = 0;
-  uint64_t ug = 0;
-  if (k >= 0) c = lat_colour(a, a.rp[r].key, k, &ug);
-  a.ctab[r * LAT_CTAB + t] = c;
-  a.ugtab[r * LAT_CTAB + t] = ug;
+  const int r = blockIdx.x;
+  lat_colours_ahead(a, r, a.rp[r].key, a.ctl->base_step, threadIdx.x, blockDim.x);
 }
 
 void launch_colour_table(const LatArgs& a, cudaStream_t st) {

@@ -136,4 +136,19 @@ __device__ __forceinline__ int lat_colour(const LatArgs& a, uint2 key, long long
   return (int)below64(w.x, w.y, (uint64_t)a.n_colours);
 }
 
+// replica r's entries first, first + stride, ... of the table of a chain's
+// next steps from `next` on (LAT_CTAB; entry t: step next + t - 1, zero before
+// the chain's first)
+__device__ __forceinline__ void lat_colours_ahead(const LatArgs& a, int r, uint2 key, long long next, int first,
+                                                  int stride) {
+  for (int t = first; t < LAT_CTAB; t += stride) {
+    const long long k = next + t - 1;
+    int c = 0;
+    uint64_t ug = 0;
+    if (k >= 0) c = lat_colour(a, key, k, &ug);
+    a.ctab[r * LAT_CTAB + t] = c;
+    a.ugtab[r * LAT_CTAB + t] = ug;
+  }
+}
+
 }  // namespace vcsgc

@@ -167,7 +167,6 @@ struct Ctx {
   ClTile* cl_tiles[5] = {};
   size_t cl_smem[5] = {};
   int cl_lcap[5] = {};             // most trials of one CTA in one step
-  long long base_lag = 0;          // steps run in a resident form not yet added to lat.ctl->base_step
   // until a launch shape is set (vcsgc_set_launch, vcsgc_autotune): the
   // resident form chosen by size (resident_shape)
   bool shape_set = false;
@@ -894,16 +893,6 @@ int sync_state_from_types(Ctx* c, int r, const uint8_t* host_types) {
   return VCSGC_OK;
 }
 
-// bring the device step base (and the colour table of the per-step launch)
-// up to the host's after steps run in the cluster-resident form
-int sync_base(Ctx* c) {
-  if (c->base_lag == 0) return VCSGC_OK;
-  launch_lattice_advance(c->lat, (int)c->base_lag, c->st);
-  CK(cudaGetLastError());
-  c->base_lag = 0;
-  return VCSGC_OK;
-}
-
 bool cluster_form_usable(const Ctx* c) {
   const int q = cl_index(c->cl_size);
   return c->form == 1 && q >= 0 && c->cl_offer[q] && !c->lat.da;
@@ -937,6 +926,7 @@ int draw_buffers(Ctx* c, long long n) {
     CK(cudaMemcpyAsync(doff, off.data(), sizeof(int) * c->R, cudaMemcpyHostToDevice, c->st));
     CK(cudaStreamSynchronize(c->st));
     d.off = doff;
+    TRY(dalloc(c, &d.base, 1));
     d.P = (int)P;
     d.pmax = pmax;
     c->draw_steps = 0;
@@ -968,13 +958,12 @@ int run_steps_resident(Ctx* c, long long n, int csize, int block) {
   TRY(draw_buffers(c, n));
   while (n > 0) {
     const int m = (int)std::min(n, c->draw_steps);
-    CK(launch_chain_draws(c->lat, c->draws, c->h_base, m, c->st));
+    CK(launch_chain_draws(c->lat, c->draws, m, c->st));
     if (csize > 0)
-      CK(launch_cluster_steps(c->lat, c->cl_tiles[q], c->draws, c->cl_smem[q], csize, block, c->h_base, m, c->st));
+      CK(launch_cluster_steps(c->lat, c->cl_tiles[q], c->draws, c->cl_smem[q], csize, block, m, c->st));
     else
-      CK(launch_pick_steps(c->lat, c->draws, c->pick_smem, block, c->h_base, m, c->st));
+      CK(launch_pick_steps(c->lat, c->draws, c->pick_smem, block, m, c->st));
     c->h_base += m;
-    c->base_lag += m;
     n -= m;
   }
   c->pending = false;
@@ -1002,7 +991,6 @@ int run_steps_fast(Ctx* c, long long n) {
     if (c->res_size) return run_steps_resident(c, n, c->res_size, c->res_block);
     if (c->pick_block) return run_steps_resident(c, n, 0, c->pick_block);
   }
-  TRY(sync_base(c));
   const int G = 64;
   if (n >= G && !c->graph) {
     cudaGraph_t g;
@@ -2349,7 +2337,6 @@ static int reschedule(Ctx* c, int kind, const int32_t sched[6]) {
   select_blk(c);
   fill_args(c);
   // the colour table of the chain's next steps under the new colour count
-  TRY(sync_base(c));
   launch_colour_table(l, c->st);
   CK(cudaGetLastError());
   TRY(drop_draws(c, true));
@@ -2398,7 +2385,6 @@ static int snap_take(Ctx* c, Snap& s) {
 static int snap_restore(Ctx* c, const Snap& s) {
   TRY(flush(c));
   c->h_base = s.h_base;
-  c->base_lag = 0;
   if (c->fast) {
     LatCtl ctl{s.h_base};
     CK(cudaMemcpyAsync(c->lat.ctl, &ctl, sizeof(LatCtl), cudaMemcpyHostToDevice, c->st));
@@ -3213,7 +3199,6 @@ int vcsgc_load(void* ctx, const char* path) {
   CK(cudaStreamSynchronize(c->st));
   // step base (fused form) first: the species upload writes n at its parity
   c->h_base = h_base;
-  c->base_lag = 0;
   if (c->fast) {
     LatCtl ctl{h_base};
     CK(cudaMemcpyAsync(c->lat.ctl, &ctl, sizeof(LatCtl), cudaMemcpyHostToDevice, c->st));
@@ -3278,7 +3263,6 @@ int vcsgc_profile_steps(void* ctx, int64_t n, double* ms_propose, double* ms_com
     *ms_commit = 0.0;
     return check_device_error(c);
   }
-  if (c->fast) TRY(sync_base(c));
   std::vector<cudaEvent_t> ev(2 * n + 1);
   for (auto& e : ev) CK(cudaEventCreate(&e));
   CK(cudaEventRecord(ev[0], c->st));
