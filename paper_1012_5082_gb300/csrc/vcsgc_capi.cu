@@ -3202,6 +3202,8 @@ int vcsgc_load(void* ctx, const char* path) {
   if (c->fast) {
     LatCtl ctl{h_base};
     CK(cudaMemcpyAsync(c->lat.ctl, &ctl, sizeof(LatCtl), cudaMemcpyHostToDevice, c->st));
+    // no dn or accepts left of the steps this context ran before
+    CK(cudaMemsetAsync(c->lat.acc, 0, sizeof(StepAcc) * c->R * 3, c->st));
     launch_colour_table(c->lat, c->st);
     CK(cudaGetLastError());
   }

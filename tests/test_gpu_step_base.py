@@ -119,3 +119,23 @@ def test_bases_beyond_32_bits(V, tmp_path, kind, base):
         for k in ("n_b", "steps", "trials", "local_accepts", "global_accepts", "flips", "near_ties"):
             assert oa[k] == ob[k], k
         assert oa["flips"] > 0
+
+
+@pytest.mark.parametrize("ran", [1, 2, 4])
+def test_load_into_a_context_that_has_run(V, tmp_path, ran):
+    """A checkpoint continues the same chain whether the context it is loaded
+    into is fresh or has run per-step calls of its own."""
+    path = str(tmp_path / "chain")
+    lat, tab, types, g = _context(V, "sublattice")
+    g.steps(20)
+    g.save(path)
+    g.close()
+    orcs = _oracles("sublattice", lat, tab, types)
+    for o in orcs:
+        o.parallel_steps(20 + 5)
+    _, _, _, g = _context(V, "sublattice")
+    g.steps(ran)
+    g.load(path)
+    g.steps(5)
+    _agree(g, orcs)
+    g.close()
