@@ -143,6 +143,7 @@ struct Ctx {
   LatArgs lat{};
   long long h_base = 0;            // host mirror of lat.ctl->base_step
   bool pending = false;            // steps launched since the last flush
+  bool captured = false;           // the caller has captured steps (see flush)
   void* h_pin = nullptr;           // pinned staging: RepState[R] then the error word
   size_t h_pin_bytes = 0;
   std::vector<int3> offsets;       // half-lattice neighbour offsets (kind 0)
@@ -949,6 +950,13 @@ int draw_buffers(Ctx* c, long long n) {
   return VCSGC_OK;
 }
 
+// whether the caller is capturing the context's stream
+bool caller_captures(Ctx* c) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(c->st, &cap) != cudaSuccess) cudaGetLastError();
+  return cap != cudaStreamCaptureStatusNone;
+}
+
 // n colour steps in a resident form (csize 0: one CTA per replica with site
 // picks): any pending commit of the per-step form first, then one persistent
 // launch per chunk of steps
@@ -978,9 +986,7 @@ constexpr long long RESIDENT_MIN_STEPS = 8;
 // and the caller is not capturing the stream, which takes no allocation
 bool resident_ready(Ctx* c, long long n) {
   if (c->no_draws || !(c->res_size || c->pick_block)) return false;
-  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(c->st, &cap) != cudaSuccess) cudaGetLastError();
-  if (cap != cudaStreamCaptureStatusNone) return false;
+  if (caller_captures(c)) return false;
   if (draw_buffers(c, n) != VCSGC_OK) c->no_draws = true;
   return !c->no_draws;
 }
@@ -991,6 +997,7 @@ int run_steps_fast(Ctx* c, long long n) {
     if (c->res_size) return run_steps_resident(c, n, c->res_size, c->res_block);
     if (c->pick_block) return run_steps_resident(c, n, 0, c->pick_block);
   }
+  c->captured |= caller_captures(c);
   const int G = 64;
   if (n >= G && !c->graph) {
     cudaGraph_t g;
@@ -1024,9 +1031,10 @@ int run_steps_fast(Ctx* c, long long n) {
 }
 
 // apply the pending commit of the last proposed step (fused form); a no-op
-// when no step ran since the last flush
+// when no step ran since the last flush.  Once the caller has captured steps a
+// replay may have left one at any time.
 int flush(Ctx* c) {
-  if (!c->fast || !c->pending) return VCSGC_OK;
+  if (!c->fast || !(c->pending || c->captured)) return VCSGC_OK;
   launch_lattice_step(c->lat, 0, false, c->st);
   CK(cudaGetLastError());
   c->pending = false;

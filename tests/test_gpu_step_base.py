@@ -80,6 +80,35 @@ def test_captured_steps_replay_after_resident_ones(V, kind):
     g.close()
 
 
+@pytest.mark.parametrize("kind", SCHED)
+def test_resident_steps_follow_a_replay(V, kind):
+    """A replay leaves a commit pending that the host has not seen: the next
+    call, resident or a read, applies it."""
+    import torch
+    s = torch.cuda.Stream()
+    lat, tab, types, g = _context(V, kind, stream=s)
+    orcs = _oracles(kind, lat, tab, types)
+    graph = torch.cuda.CUDAGraph()
+    s.synchronize()
+    with torch.cuda.graph(graph, stream=s, capture_error_mode="thread_local"):
+        g.steps(5)
+    g.types(0)  # nothing has run: no pending commit for the host
+    with torch.cuda.stream(s):
+        graph.replay()
+        graph.replay()
+    g.steps(30)  # resident
+    for o in orcs:
+        o.parallel_steps(2 * 5 + 30)
+    _agree(g, orcs)
+    with torch.cuda.stream(s):
+        graph.replay()
+    for o in orcs:
+        o.parallel_steps(5)
+    _agree(g, orcs)
+    del graph
+    g.close()
+
+
 # ------------------------------------------------------------ 64-bit steps
 def _move_base(path, base, n_replicas):
     """The checkpoint's chain moved to step `base`: the running states' next
