@@ -211,6 +211,9 @@ inline size_t cluster_offer_bytes(const ClTile& t, int W) {
 }
 // largest dynamic shared memory a tile may use
 constexpr size_t CL_SMEM_MAX = 200 * 1024;
+// lets the resident kernels of these lattices use the largest shared memory on
+// the current device; before their first launch or occupancy query there
+cudaError_t resident_attributes(const LatArgs& a);
 // the n colour steps of cd's chunk for every replica (R clusters of `csize`
 // CTAs of `block` trial threads, block 256 or 512); needs the five-shell or
 // (period 4 along x) two-shell table, the sublattice schedule, a uniform dF

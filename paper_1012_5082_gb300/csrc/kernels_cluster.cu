@@ -1037,9 +1037,11 @@ ClusterKernel cluster_kernel(const LatArgs& a, int block) {
   return block == 256 ? cluster_kernel_bs<256>(a) : cluster_kernel_bs<512>(a);
 }
 
-cudaError_t cluster_attributes(ClusterKernel k, size_t smem) {
-  const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-  return e != cudaSuccess ? e : cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+using PickKernel = void (*)(LatArgs, ChainDraws, int);
+
+PickKernel pick_kernel(const LatArgs& a, int block) {
+  if (block <= 64) return a.bcc5 ? k_pick_steps<5, 64> : (a.bcc2 ? k_pick_steps<2, 64> : k_pick_steps<0, 64>);
+  return a.bcc5 ? k_pick_steps<5, 512> : (a.bcc2 ? k_pick_steps<2, 512> : k_pick_steps<0, 512>);
 }
 
 void cluster_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute& attr, int blocks, int csize, int block, size_t smem) {
@@ -1064,11 +1066,26 @@ cudaError_t launch_chain_draws(const LatArgs& a, const ChainDraws& cd, int m, cu
   return cudaGetLastError();
 }
 
+// Attributes belong to a kernel, not to a context: every context sets the same
+// largest size, so that none lowers it under another thread's launch.
+cudaError_t resident_attributes(const LatArgs& a) {
+  for (int block : {256, 512}) {
+    const ClusterKernel k = cluster_kernel(a, block);
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CL_SMEM_MAX);
+    if (e != cudaSuccess) return e;
+  }
+  for (int block : {64, 512}) {
+    const cudaError_t e = cudaFuncSetAttribute(pick_kernel(a, block), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               (int)PICK_SMEM_MAX);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
 cudaError_t launch_cluster_steps(const LatArgs& a, const ClTile* d_tiles, const ChainDraws& cd, size_t smem, int csize,
                                  int block, int n, cudaStream_t st) {
   const ClusterKernel k = cluster_kernel(a, block);
-  const cudaError_t e = cluster_attributes(k, smem);
-  if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[1];
   cluster_config(cfg, attr[0], a.R * csize, csize, block, smem);
@@ -1082,7 +1099,7 @@ int cluster_capacity(const LatArgs& a, int csize, int block, size_t smem) {
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[1];
   cluster_config(cfg, attr[0], csize, csize, block, smem);
-  if (cluster_attributes(k, smem) != cudaSuccess || cudaOccupancyMaxActiveClusters(&n, k, &cfg) != cudaSuccess) {
+  if (cudaOccupancyMaxActiveClusters(&n, k, &cfg) != cudaSuccess) {
     cudaGetLastError();
     return 0;
   }
@@ -1090,11 +1107,7 @@ int cluster_capacity(const LatArgs& a, int csize, int block, size_t smem) {
 }
 
 cudaError_t launch_pick_steps(const LatArgs& a, const ChainDraws& cd, size_t smem, int block, int n, cudaStream_t st) {
-  auto k = block <= 64 ? (a.bcc5 ? k_pick_steps<5, 64> : (a.bcc2 ? k_pick_steps<2, 64> : k_pick_steps<0, 64>))
-                       : (a.bcc5 ? k_pick_steps<5, 512> : (a.bcc2 ? k_pick_steps<2, 512> : k_pick_steps<0, 512>));
-  const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  k<<<a.R, block, smem, st>>>(a, cd, n);
+  pick_kernel(a, block)<<<a.R, block, smem, st>>>(a, cd, n);
   return cudaGetLastError();
 }
 

@@ -1974,6 +1974,7 @@ static void resident_shape(Ctx* c, const int* capacity) {
 // dropped.
 static int cluster_setup(Ctx* c) {
   const LatArgs& l = c->lat;
+  CK(resident_attributes(l));
   int capacity[5] = {0, 0, 0, 0, 0};
   if (!l.sublattice || !(l.bcc5 || (l.bcc2 && l.qx == 4)) || !l.df_uniform) {
     resident_shape(c, capacity);
