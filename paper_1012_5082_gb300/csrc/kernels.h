@@ -185,7 +185,9 @@ void launch_lattice_step(const LatArgs& a, int j, bool propose, cudaStream_t st)
 struct ClTile {
   int TY, TZ, Ty, Tz, lcap;
 };
-constexpr int CL_TRIALS_PER_THREAD = 8;
+// most trials of a CTA in a step: 16 a thread of 256, whose warp's per-shell
+// sums (512 trials of up to 24 neighbours) stay within 16 bits
+constexpr int CL_TRIALS_MAX = 4096;
 // dynamic shared memory of a tile: rows with halo, two pad words (a window's
 // second word may lie one past the last row; its bits are never used), two
 // bytes per trial group (lcap rounded to 16 each)
@@ -204,11 +206,6 @@ struct ChainDraws {
 };
 // draws of the next m steps of the chain
 cudaError_t launch_chain_draws(const LatArgs& a, const ChainDraws& cd, int m, cudaStream_t st);
-// the footprint by which a size is offered as launch form 1: 64-bit words (32
-// species and 32 pending bits) and 16 bytes per trial
-inline size_t cluster_offer_bytes(const ClTile& t, int W) {
-  return 8 * ((size_t)(t.Ty + 4) * (t.Tz + 4) * W + 1 + t.lcap) + 8 * (size_t)t.lcap;
-}
 // largest dynamic shared memory a tile may use
 constexpr size_t CL_SMEM_MAX = 200 * 1024;
 // lets the resident kernels of these lattices use the largest shared memory on

@@ -173,7 +173,7 @@ struct Ctx {
   bool shape_set = false;
   int res_size = 0, res_block = 0;  // CTAs per cluster (0: none), trial threads
   bool no_draws = false;            // no memory for the draws: not by default
-  bool cl_offer[5] = {};            // sizes vcsgc_cluster_sizes lists (of cl_tiles)
+  bool cl_offer[5] = {};            // sizes vcsgc_cluster_sizes lists: cl_tiles of the five-shell table
   int pick_block = 0;               // BLOCKS, OVERLAP: trial threads of the one-CTA form (0: none)
   size_t pick_smem = 0;
   ChainDraws draws{};               // draws of a chunk of steps of a resident form
@@ -1968,7 +1968,7 @@ static void resident_shape(Ctx* c, const int* capacity) {
 // 4, 8, 16 every replica needs a TY x TZ = s grid of tiles dividing its
 // ny x nz rows with Ty, Tz >= 2, whose rows with halo, (Ty + 4)(Tz + 4) W
 // words, and accept lists fit in shared memory, and whose trials per step
-// fit the threads; among such grids the one with whole sublattice periods
+// fit a CTA (CL_TRIALS_MAX); among such grids the one with whole sublattice periods
 // per tile (equal trials per CTA) and the squarest tile is taken.  Sizes
 // the GPU cannot co-schedule (cudaOccupancyMaxActiveClusters = 0) are
 // dropped.
@@ -1984,7 +1984,7 @@ static int cluster_setup(Ctx* c) {
   for (int qi = 0; qi < 5; ++qi) {
     const int s = sizes[qi];
     std::vector<ClTile> tiles;
-    size_t smem = 0, offer = 0;
+    size_t smem = 0;
     bool ok = true;
     for (int r = 0; r < c->R && ok; ++r) {
       const LatGeom& g = c->h_geom[r];
@@ -1998,7 +1998,7 @@ static int cluster_setup(Ctx* c) {
         if (Ty < 2 || Tz < 2) continue;
         ClTile t{TY, TZ, Ty, Tz, 0};
         t.lcap = ((Ty + l.qy - 1) / l.qy) * ((Tz + l.qz - 1) / l.qz) * g.nxq;
-        if (t.lcap > 512 * CL_TRIALS_PER_THREAD) continue;
+        if (t.lcap > CL_TRIALS_MAX) continue;
         const size_t sm = cluster_smem_bytes(t, g.W);
         if (sm > CL_SMEM_MAX) continue;
         const bool whole = Ty % l.qy == 0 && Tz % l.qz == 0;
@@ -2012,7 +2012,6 @@ static int cluster_setup(Ctx* c) {
       if (!found) ok = false;
       tiles.push_back(best);
       smem = std::max(smem, cluster_smem_bytes(best, g.W));
-      offer = std::max(offer, cluster_offer_bytes(best, g.W));
       c->cl_lcap[qi] = std::max(c->cl_lcap[qi], best.lcap);
     }
     if (!ok || cluster_capacity(l, s, 512, smem) < 1) continue;
@@ -2020,7 +2019,7 @@ static int cluster_setup(Ctx* c) {
     TRY(dalloc(c, &c->cl_tiles[qi], tiles.size()));
     CK(cudaMemcpyAsync(c->cl_tiles[qi], tiles.data(), sizeof(ClTile) * tiles.size(), cudaMemcpyHostToDevice, c->st));
     c->cl_smem[qi] = smem;
-    c->cl_offer[qi] = l.bcc5 && offer <= CL_SMEM_MAX;
+    c->cl_offer[qi] = l.bcc5;
   }
   resident_shape(c, capacity);
   return VCSGC_OK;
@@ -2467,8 +2466,7 @@ int vcsgc_set_launch(void* ctx, int32_t form, int32_t block, int32_t variant) {
   if (!c->fast) return fail(c, VCSGC_ERR_STATE, "launch shape: the context is not in the fused form");
   if (f1) {
     const int q = cl_index(variant);
-    if (!c->cl_offer[q] || c->cl_lcap[q] > block * CL_TRIALS_PER_THREAD ||
-        (block == 256 && cluster_capacity(c->lat, variant, 256, c->cl_smem[q]) < 1))
+    if (!c->cl_offer[q] || (block == 256 && cluster_capacity(c->lat, variant, 256, c->cl_smem[q]) < 1))
       return fail(c, VCSGC_ERR_STATE, "launch shape: no cluster-resident form of this size for these lattices");
     if (c->lat.da) return fail(c, VCSGC_ERR_STATE, "launch shape: the cluster-resident form has no delayed acceptance");
     c->form = 1;
