@@ -1024,7 +1024,8 @@ def main():
            "clock": "host wall clock over all steps"}
 
     ctx.close()
-    launches = (spw * args.steps + 2 * ((spw * args.steps) // 64)) if launch[0] == 0 else args.steps
+    # resident forms: a sweep is a launch of the draws and one of the chain
+    launches = (spw * args.steps + 2 * ((spw * args.steps) // 64)) if launch[0] == 0 else 2 * args.steps
     line = {"metric": METRIC, "value": value, "unit": "trial moves/s", "n_gpus": world,
             "steps": args.steps, "warmup": args.warmup, "ms_per_step": ms_max / args.steps,
             "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "f64",

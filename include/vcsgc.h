@@ -222,9 +222,10 @@ int vcsgc_batch_init(void** ctx, int32_t n_rep, const int32_t* cells, double a, 
  * steps with each candidate (these are real steps of the chain): form 0
  * with thread-block size 64, 128 or 256, each with and without loading the
  * trial's neighbour rows ahead of the block barrier (shorter dependent
- * chain, more registers), and form 1 with every cluster size the lattices
- * allow at 256 and 512 threads (see vcsgc_set_launch).  The fastest is kept
- * for later launches (vcsgc_get_launch reports it); *best_block receives its
+ * chain, more registers), form 2 where it has a resident form, and form 1
+ * with every cluster size the lattices allow at 256 and 512 threads (see
+ * vcsgc_set_launch).  The fastest is kept for later launches, form 2 unless
+ * form 1 is 3 % faster (vcsgc_get_launch reports it); *best_block receives its
  * block size.  A context outside the fused form reports its fixed block
  * size. */
 int vcsgc_autotune(void* ctx, int64_t steps, int32_t* best_block);
@@ -328,13 +329,17 @@ int vcsgc_profile_steps(void* ctx, int64_t n, double* ms_propose, double* ms_com
  *           the period-q sublattice schedule, the five-shell BCC table, one
  *           density function and no surrogate; vcsgc_cluster_sizes lists
  *           the sizes these lattices allow.
- * Until a shape is set, calls of 8 steps or more run a resident form chosen by
- * size where one applies (form 1, or for the BLOCKS and OVERLAP schedules one
- * block per replica with the whole lattice in shared memory); vcsgc_get_launch
- * then reports the shape of the per-step launch that shorter calls use.
+ *   form 2: calls of 8 steps or more run a resident form chosen by size where
+ *           one applies (form 1, also for the two-shell BCC table, or for the
+ *           BLOCKS and OVERLAP schedules one block per replica with the whole
+ *           lattice in shared memory); shorter calls, and calls where none
+ *           applies, run form 0 with this `block` and `variant`.
+ * Until a shape is set a context runs as in form 2, and vcsgc_get_launch reports
+ * the shape of the per-step launch (form 0) that its shorter calls use.
  * vcsgc_autotune picks a shape by timing; this call sets one explicitly.
  * Errors: INVALID_ARG (unknown form or shape), STATE (not the fused form,
- * or a form-1 size these lattices or this GPU do not allow). */
+ * or a form-1 size these lattices or this GPU do not allow).  A schedule change
+ * that leaves no such size ends form 1: the context is as before any was set. */
 int vcsgc_set_launch(void* ctx, int32_t form, int32_t block, int32_t variant);
 /* The current launch shape (HOST outputs; any may be NULL). */
 int vcsgc_get_launch(void* ctx, int32_t* form, int32_t* block, int32_t* variant);

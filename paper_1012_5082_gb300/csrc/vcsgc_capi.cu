@@ -171,6 +171,7 @@ struct Ctx {
   // until a launch shape is set (vcsgc_set_launch, vcsgc_autotune): the
   // resident form chosen by size (resident_shape)
   bool shape_set = false;
+  bool by_size = false;             // form 2 was set: the same as before any was, and reported
   int res_size = 0, res_block = 0;  // CTAs per cluster (0: none), trial threads
   bool no_draws = false;            // no memory for the draws: not by default
   bool cl_offer[5] = {};            // sizes vcsgc_cluster_sizes lists: cl_tiles of the five-shell table
@@ -985,15 +986,17 @@ constexpr long long RESIDENT_MIN_STEPS = 8;
 // there (without memory for them the context goes on with a launch per step)
 // and the caller is not capturing the stream, which takes no allocation
 bool resident_ready(Ctx* c, long long n) {
-  if (c->no_draws || !(c->res_size || c->pick_block)) return false;
-  if (caller_captures(c)) return false;
+  if (c->no_draws || caller_captures(c)) return false;
   if (draw_buffers(c, n) != VCSGC_OK) c->no_draws = true;
   return !c->no_draws;
 }
 
+// whether the default form has a resident form for calls that are long enough
+bool resident_by_size(const Ctx* c) { return (c->res_size || c->pick_block) && !c->lat.da; }
+
 int run_steps_fast(Ctx* c, long long n) {
   if (cluster_form_usable(c)) return run_steps_resident(c, n, c->cl_size, c->cl_block);
-  if (!c->shape_set && !c->lat.da && n >= RESIDENT_MIN_STEPS && resident_ready(c, n)) {
+  if (!c->shape_set && resident_by_size(c) && n >= RESIDENT_MIN_STEPS && resident_ready(c, n)) {
     if (c->res_size) return run_steps_resident(c, n, c->res_size, c->res_block);
     if (c->pick_block) return run_steps_resident(c, n, 0, c->pick_block);
   }
@@ -1967,10 +1970,10 @@ static void resident_shape(Ctx* c, const int* capacity) {
 // Tilings of the cluster-resident form.  For each cluster size s in 1, 2,
 // 4, 8, 16 every replica needs a TY x TZ = s grid of tiles dividing its
 // ny x nz rows with Ty, Tz >= 2, whose rows with halo, (Ty + 4)(Tz + 4) W
-// words, and accept lists fit in shared memory, and whose trials per step
-// fit a CTA (CL_TRIALS_MAX); among such grids the one with whole sublattice periods
-// per tile (equal trials per CTA) and the squarest tile is taken.  Sizes
-// the GPU cannot co-schedule (cudaOccupancyMaxActiveClusters = 0) are
+// words, and trial bytes fit in shared memory, and whose trials per step
+// fit a CTA (CL_TRIALS_MAX); among such grids the one with whole sublattice
+// periods per tile (equal trials per CTA) and the squarest tile is taken.
+// Sizes the GPU cannot co-schedule (cudaOccupancyMaxActiveClusters = 0) are
 // dropped.
 static int cluster_setup(Ctx* c) {
   const LatArgs& l = c->lat;
@@ -2243,19 +2246,25 @@ int vcsgc_autotune(void* ctx, int64_t steps, int32_t* best_block) {
   }
   // candidates (form, block, variant): one launch per colour step with block
   // size x row prefetch (prefetching shortens the dependent chain of a step
-  // but costs registers, i.e. resident blocks), then the cluster-resident
+  // but costs registers, i.e. resident blocks), then the form chosen by size,
+  // with the fastest of these for its short calls, then the cluster-resident
   // form with each cluster size that serves these lattices x block size
   std::vector<std::array<int, 3>> cand = {{0, 64, 1}, {0, 128, 1}, {0, 256, 1}, {0, 64, 0}, {0, 128, 0}, {0, 256, 0}};
+  if (resident_by_size(c)) cand.push_back({2, 0, 0});
   if (!c->lat.da)
     for (int s : {1, 2, 4, 8, 16})
       if (c->cl_offer[cl_index(s)])
         for (int b : {256, 512}) cand.push_back({1, b, s});
   float best = 0.0f;
   std::array<int, 3> bc = {0, 128, 1};
+  // a later candidate has to be clearly faster than the form chosen by size:
+  // among its own cluster sizes the timings differ by a percent or two
+  float lead = 1.0f;
   cudaEvent_t e0, e1;
   CK(cudaEventCreate(&e0));
   CK(cudaEventCreate(&e1));
-  for (const auto& cb : cand) {
+  for (auto cb : cand) {
+    if (cb[0] == 2) cb = {2, bc[1], bc[2]};
     if (vcsgc_set_launch(c, cb[0], cb[1], cb[2]) != VCSGC_OK) continue;
     // one untimed step with the candidate, then the timed ones
     TRY(run_steps_fast(c, 1));
@@ -2265,9 +2274,12 @@ int vcsgc_autotune(void* ctx, int64_t steps, int32_t* best_block) {
     CK(cudaEventSynchronize(e1));
     float ms = 0.0f;
     CK(cudaEventElapsedTime(&ms, e0, e1));
-    if (best == 0.0f || ms < best) {
-      best = ms;
+    // (timed over fewer steps than run resident, it is the fastest of form 0)
+    const bool tie = cb[0] == 2 && steps < RESIDENT_MIN_STEPS;
+    if (best == 0.0f || ms < lead * best || tie) {
+      best = tie ? std::min(best, ms) : ms;
       bc = cb;
+      lead = cb[0] == 2 ? 0.97f : 1.0f;
     }
   }
   cudaEventDestroy(e0);
@@ -2356,7 +2368,10 @@ static int reschedule(Ctx* c, int kind, const int32_t sched[6]) {
     c->cl_lcap[k] = 0;
   }
   TRY(cluster_setup(c));
-  if (c->form == 1 && !cluster_form_usable(c)) c->form = 0;
+  if (c->form == 1 && !cluster_form_usable(c)) {
+    c->form = 0;
+    c->shape_set = false;
+  }
   CK(cudaStreamSynchronize(c->st));
   return check_device_error(c);
 }
@@ -2459,9 +2474,10 @@ int vcsgc_set_launch(void* ctx, int32_t form, int32_t block, int32_t variant) {
   if (!c) return VCSGC_ERR_INVALID_ARG;
   const bool f0 = form == 0 && (block == 64 || block == 128 || block == 256) && (variant == 0 || variant == 1);
   const bool f1 = form == 1 && (block == 256 || block == 512) && cl_index(variant) >= 0;
-  if (!f0 && !f1)
+  const bool f2 = form == 2 && (block == 64 || block == 128 || block == 256) && (variant == 0 || variant == 1);
+  if (!f0 && !f1 && !f2)
     return fail(c, VCSGC_ERR_INVALID_ARG,
-                "launch shape: form 0 with block 64, 128 or 256 and prefetch 0 or 1, or form 1 with block 256 or "
+                "launch shape: form 0 or 2 with block 64, 128 or 256 and prefetch 0 or 1, or form 1 with block 256 or "
                 "512 and 1, 2, 4, 8 or 16 CTAs per cluster");
   if (!c->fast) return fail(c, VCSGC_ERR_STATE, "launch shape: the context is not in the fused form");
   if (f1) {
@@ -2473,10 +2489,12 @@ int vcsgc_set_launch(void* ctx, int32_t form, int32_t block, int32_t variant) {
     c->cl_size = variant;
     c->cl_block = block;
     c->shape_set = true;
+    c->by_size = false;
     return VCSGC_OK;
   }
   c->form = 0;
-  c->shape_set = true;
+  c->shape_set = !f2;
+  c->by_size = f2;
   c->lat.block = block;
   c->lat.prefetch = variant;
   select_blk(c);
@@ -2488,7 +2506,7 @@ int vcsgc_get_launch(void* ctx, int32_t* form, int32_t* block, int32_t* variant)
   Ctx* c = static_cast<Ctx*>(ctx);
   if (!c) return VCSGC_ERR_INVALID_ARG;
   const bool f1 = c->fast && cluster_form_usable(c);
-  if (form) *form = f1 ? 1 : 0;
+  if (form) *form = f1 ? 1 : (c->fast && c->by_size ? 2 : 0);
   if (block) *block = f1 ? c->cl_block : (c->fast ? c->lat.block : MC_BLOCK);
   if (variant) *variant = f1 ? c->cl_size : (c->fast ? c->lat.prefetch : 0);
   return VCSGC_OK;

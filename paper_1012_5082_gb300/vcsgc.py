@@ -561,7 +561,9 @@ class Context:
 
     def set_launch(self, form=0, block=128, variant=1):
         """Launch shape of the fused colour step (vcsgc_set_launch): form 0
-        with variant = row prefetch, form 1 with variant = CTAs per cluster."""
+        with variant = row prefetch, form 1 with variant = CTAs per cluster,
+        form 2 (as before any shape is set) resident by size for calls of 8
+        steps and more, with block and variant as form 0 for shorter ones."""
         _check(lib().vcsgc_set_launch(self.h, int(form), int(block), int(variant)), self.h)
 
     def set_schedule(self, kind, sched):
@@ -593,7 +595,8 @@ class Context:
         return f.value, b.value, p.value
 
     def autotune(self, steps=64):
-        """Pick the fused colour step's block size by timing (real steps)."""
+        """Pick the fused colour step's launch shape by timing (real steps);
+        returns its block size (get_launch: the whole shape)."""
         b = C.c_int32()
         _check(lib().vcsgc_autotune(self.h, int(steps), C.byref(b)), self.h)
         return b.value
