@@ -311,7 +311,9 @@ int vcsgc_kinetic_energy(void* ctx, double* out);
 
 /* Run n colour steps with a CUDA event after each launch on the context's
  * stream and return the summed device time (ms) of the propose kernels and
- * of the commit kernels.  Same work as vcsgc_steps(n); for profiling. */
+ * of the commit kernels.  Same work as vcsgc_steps(n), in the form in which
+ * that runs them: where it is a resident one, the whole time is reported as
+ * propose.  For profiling. */
 int vcsgc_profile_steps(void* ctx, int64_t n, double* ms_propose, double* ms_commit);
 
 /* Launch shape of the fused colour step.  Any shape advances the same chain

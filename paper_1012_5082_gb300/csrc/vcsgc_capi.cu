@@ -994,30 +994,51 @@ bool resident_ready(Ctx* c, long long n) {
 // whether the default form has a resident form for calls that are long enough
 bool resident_by_size(const Ctx* c) { return (c->res_size || c->pick_block) && !c->lat.da; }
 
+// whether a call of n steps runs resident, with the draws' buffers made
+bool runs_resident(Ctx* c, long long n) {
+  if (cluster_form_usable(c)) return true;
+  return !c->shape_set && resident_by_size(c) && n >= RESIDENT_MIN_STEPS && resident_ready(c, n);
+}
+
+// the graph of the per-step launch
+constexpr int STEP_GRAPH = 64;
+
+int step_graph(Ctx* c) {
+  constexpr int G = STEP_GRAPH;
+  if (c->graph) return VCSGC_OK;
+  cudaGraph_t g;
+  CK(cudaStreamBeginCapture(c->st, cudaStreamCaptureModeThreadLocal));
+  for (int q = 0; q < G; ++q) launch_lattice_step(c->lat, q, true, c->st);
+  launch_lattice_advance(c->lat, G, c->st);
+  cudaError_t e1 = cudaGetLastError();
+  CK(cudaStreamEndCapture(c->st, &g));
+  if (e1 != cudaSuccess) {
+    cudaGraphDestroy(g);
+    return fail(c, VCSGC_ERR_CUDA, std::string("capture: ") + cudaGetErrorString(e1));
+  }
+  cudaError_t e2 = cudaGraphInstantiate(&c->graph, g, 0);
+  cudaGraphDestroy(g);
+  if (e2 != cudaSuccess) return fail(c, VCSGC_ERR_CUDA, std::string("graph: ") + cudaGetErrorString(e2));
+  c->graph_steps = G;
+  return VCSGC_OK;
+}
+
+// what a call of n steps allocates or instantiates, before it is timed
+int prepare_steps(Ctx* c, long long n) {
+  if (cluster_form_usable(c)) return draw_buffers(c, n);
+  if (!runs_resident(c, n) && n >= STEP_GRAPH) return step_graph(c);
+  return VCSGC_OK;
+}
+
 int run_steps_fast(Ctx* c, long long n) {
-  if (cluster_form_usable(c)) return run_steps_resident(c, n, c->cl_size, c->cl_block);
-  if (!c->shape_set && resident_by_size(c) && n >= RESIDENT_MIN_STEPS && resident_ready(c, n)) {
+  if (runs_resident(c, n)) {
+    if (cluster_form_usable(c)) return run_steps_resident(c, n, c->cl_size, c->cl_block);
     if (c->res_size) return run_steps_resident(c, n, c->res_size, c->res_block);
-    if (c->pick_block) return run_steps_resident(c, n, 0, c->pick_block);
+    return run_steps_resident(c, n, 0, c->pick_block);
   }
   c->captured |= caller_captures(c);
-  const int G = 64;
-  if (n >= G && !c->graph) {
-    cudaGraph_t g;
-    CK(cudaStreamBeginCapture(c->st, cudaStreamCaptureModeThreadLocal));
-    for (int q = 0; q < G; ++q) launch_lattice_step(c->lat, q, true, c->st);
-    launch_lattice_advance(c->lat, G, c->st);
-    cudaError_t e1 = cudaGetLastError();
-    CK(cudaStreamEndCapture(c->st, &g));
-    if (e1 != cudaSuccess) {
-      cudaGraphDestroy(g);
-      return fail(c, VCSGC_ERR_CUDA, std::string("capture: ") + cudaGetErrorString(e1));
-    }
-    cudaError_t e2 = cudaGraphInstantiate(&c->graph, g, 0);
-    cudaGraphDestroy(g);
-    if (e2 != cudaSuccess) return fail(c, VCSGC_ERR_CUDA, std::string("graph: ") + cudaGetErrorString(e2));
-    c->graph_steps = G;
-  }
+  constexpr int G = STEP_GRAPH;
+  if (n >= G) TRY(step_graph(c));
   while (n >= G) {
     CK(cudaGraphLaunch(c->graph, c->st));
     c->h_base += G;
@@ -2266,8 +2287,10 @@ int vcsgc_autotune(void* ctx, int64_t steps, int32_t* best_block) {
   for (auto cb : cand) {
     if (cb[0] == 2) cb = {2, bc[1], bc[2]};
     if (vcsgc_set_launch(c, cb[0], cb[1], cb[2]) != VCSGC_OK) continue;
-    // one untimed step with the candidate, then the timed ones
+    // one untimed step with the candidate, then the timed ones, whose buffers
+    // and graph are made before
     TRY(run_steps_fast(c, 1));
+    TRY(prepare_steps(c, steps));
     CK(cudaEventRecord(e0, c->st));
     TRY(run_steps_fast(c, steps));
     CK(cudaEventRecord(e1, c->st));
@@ -3272,14 +3295,15 @@ int vcsgc_load(void* ctx, const char* path) {
 int vcsgc_profile_steps(void* ctx, int64_t n, double* ms_propose, double* ms_commit) {
   Ctx* c = static_cast<Ctx*>(ctx);
   if (!c || n < 1 || !ms_propose || !ms_commit) return VCSGC_ERR_INVALID_ARG;
-  if (c->multi || (c->fast && cluster_form_usable(c))) {
-    // one persistent launch of n steps: its whole time is reported as propose
+  if (c->multi || (c->fast && runs_resident(c, n))) {
+    // persistent launches of many steps: their whole time is reported as propose
     cudaEvent_t e0, e1;
     CK(cudaEventCreate(&e0));
     CK(cudaEventCreate(&e1));
     TRY(flush(c));
+    if (!c->multi) TRY(prepare_steps(c, n));
     CK(cudaEventRecord(e0, c->st));
-    TRY(c->multi ? run_steps(c, n) : run_steps_resident(c, n, c->cl_size, c->cl_block));
+    TRY(run_steps(c, n));
     CK(cudaEventRecord(e1, c->st));
     CK(cudaEventSynchronize(e1));
     float ms = 0.f;

@@ -80,3 +80,21 @@ def test_form_2_takes_a_shape_back(V):
         assert e.value.code == -1
     g.close()
     h.close()
+
+
+@pytest.mark.parametrize("shape", [None, (1, 256, 8)])
+def test_profiled_steps_hold_no_allocation(V, shape):
+    """The first profiled run of a length, whose draws need larger buffers than
+    the calls before, takes what later ones take, not the allocation's time
+    (which is more than the steps' own); and a context without a shape is
+    profiled in the form its calls run."""
+    g = _context(V, "sublattice", (80, 80, 80), (4, 4, 4), "eam", R=8)
+    if shape:
+        g.set_launch(*shape)
+    for _ in range(3):
+        g.steps(8)
+    first = g.profile_steps(64)
+    later = [g.profile_steps(64) for _ in range(5)]
+    assert first[1] == 0.0 and all(q[1] == 0.0 for q in later)  # one launch of many steps: no commits
+    assert first[0] < 1.6 * np.median([q[0] for q in later]), (first, later)
+    g.close()
