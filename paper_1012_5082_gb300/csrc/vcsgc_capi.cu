@@ -15,6 +15,7 @@
 #include "common.cuh"
 #include "kernels.h"
 #include "multi_host.h"
+#include "optional.h"
 #include "readout.h"
 #include "screen.h"
 #include "trace.h"
@@ -267,6 +268,22 @@ void dfree(Ctx* c, T** p) {
   *p = nullptr;
 }
 
+// buffers of an optional path: all of them, or none and no error
+bool dalloc_optional(Ctx* c, std::initializer_list<Wanted> list) {
+  return get_all(
+      list,
+      [&](size_t bytes) -> void* {
+        void* q = nullptr;
+        if (cudaMalloc(&q, bytes) != cudaSuccess) {
+          cudaGetLastError();
+          return nullptr;
+        }
+        c->allocs.push_back(q);
+        return q;
+      },
+      [&](void* q) { dfree(c, &q); });
+}
+
 // the device error bits e (already copied to the host) as a status
 int device_error_status(Ctx* c, unsigned e) {
   if (!e) return VCSGC_OK;
@@ -441,26 +458,25 @@ int ensure_pairs(Ctx* c) {
     const size_t want = c->pair_need + c->pair_need / 8;
     size_t free_b = 0, total_b = 0;
     CK(cudaMemGetInfo(&free_b, &total_b));
-    if (want * (sizeof(uint32_t) + sizeof(double2)) <= free_b / 4 && dalloc(c, &c->pair_j, want) == VCSGC_OK) {
-      if (dalloc(c, &c->pair_ui, want) == VCSGC_OK) c->pair_cap = want;
-      else dfree(c, &c->pair_j);
-    }
+    if (want * (sizeof(uint32_t) + sizeof(double2)) <= free_b / 4 &&
+        dalloc_optional(c, {wanted(&c->pair_j, want), wanted(&c->pair_ui, want)}))
+      c->pair_cap = want;
   }
   fill_args(c);
   return VCSGC_OK;
 }
 
 // pair blocks from now on (MD and minimisation, whose list serves many passes)
+// where there is memory for them
 int enable_pairs(Ctx* c) {
   if (c->md_pairs || !c->p4 || !c->nbr_h || c->N > (1ll << 28)) return VCSGC_OK;
   size_t free_b = 0, total_b = 0;
   CK(cudaMemGetInfo(&free_b, &total_b));
   if ((size_t)c->N * (sizeof(float4) + 2 * sizeof(int)) > free_b / 4) return VCSGC_OK;
   const long long groups = (c->N + md_pair_group(c->N) - 1) / md_pair_group(c->N);
-  TRY(dalloc(c, &c->f4, c->N));
-  TRY(dalloc(c, &c->pair_off, groups));
-  TRY(dalloc(c, &c->pair_rows, groups));
-  TRY(dalloc(c, &c->pair_total, 1));
+  if (!dalloc_optional(c, {wanted(&c->f4, c->N), wanted(&c->pair_off, groups), wanted(&c->pair_rows, groups),
+                           wanted(&c->pair_total, 1)}))
+    return VCSGC_OK;
   c->md_pairs = true;
   return ensure_pairs(c);
 }
