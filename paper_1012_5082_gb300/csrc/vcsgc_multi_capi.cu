@@ -10,6 +10,7 @@
 
 #include "kernels.h"
 #include "multi.cuh"
+#include "optional.h"
 #include "readout.h"
 #include "screen.h"
 #include "trace.h"
@@ -84,6 +85,25 @@ int malloc_dev(Multi* m, T** p, size_t count) {
   m->allocs.push_back(q);
   *p = static_cast<T*>(q);
   return VCSGC_OK;
+}
+
+// buffers of an optional path: all of them, or none and no error
+bool malloc_optional(Multi* m, std::initializer_list<Wanted> list) {
+  return get_all(
+      list,
+      [&](size_t bytes) -> void* {
+        void* q = nullptr;
+        if (cudaMalloc(&q, bytes) != cudaSuccess) {
+          cudaGetLastError();
+          return nullptr;
+        }
+        m->allocs.push_back(q);
+        return q;
+      },
+      [&](void* q) {
+        m->allocs.erase(std::find(m->allocs.begin(), m->allocs.end(), q));
+        cudaFree(q);
+      });
 }
 
 int device_error(Multi* m) {
@@ -384,11 +404,13 @@ int screen_setup(Multi* m, const std::vector<double>& hFd) {
   const size_t counts = sizeof(uint32_t) * (size_t)m->R * a.rf_n;
   size_t free_b = 0, total_b = 0;
   MCK(cudaMemGetInfo(&free_b, &total_b));
+  float4* s4 = nullptr;
+  float* lo0 = nullptr;
   // (offsets within a replica's planes are 32-bit byte offsets)
-  if (m->K == 2 && table + counts <= free_b / 4 && sizeof(float) * (size_t)DTAB_PLANES * a.rf_n < (1ull << 32)) {
-    MTRY(malloc_dev(m, &a.ctab, (size_t)m->R * MK_CTAB));
-    MTRY(malloc_dev(m, &a.nbc, counts / sizeof(uint32_t)));
-    MTRY(malloc_dev(m, &a.dtab, table / sizeof(float)));
+  if (m->K == 2 && table + counts <= free_b / 4 && sizeof(float) * (size_t)DTAB_PLANES * a.rf_n < (1ull << 32) &&
+      malloc_optional(m, {wanted(&a.ctab, (size_t)m->R * MK_CTAB), wanted(&a.nbc, counts / sizeof(uint32_t)),
+                          wanted(&a.dtab, table / sizeof(float)), wanted(&s4, (size_t)2 * n),
+                          wanted(&lo0, (size_t)2 * n)})) {
     std::vector<float4> hs4((size_t)2 * n);
     std::vector<float> hlo((size_t)2 * n);
     const int j0 = std::max(0, (int)std::floor(lo / h) - 1), j1 = std::min(n - 1, (int)std::floor(hi / h) + 1);
@@ -401,10 +423,6 @@ int screen_setup(Multi* m, const std::vector<double>& hFd) {
         hlo[(size_t)al * n + j] = (float)(q.x - (double)c0);
         if (j >= j0 && j <= j1) dm = std::max(dm, std::fabs(q.y) + 2.0 * std::fabs(q.z) + 3.0 * std::fabs(q.w));
       }
-    float4* s4 = nullptr;
-    float* lo0 = nullptr;
-    MTRY(malloc_dev(m, &s4, hs4.size()));
-    MTRY(malloc_dev(m, &lo0, hlo.size()));
     MCK(cudaMemcpyAsync(s4, hs4.data(), sizeof(float4) * hs4.size(), cudaMemcpyHostToDevice, m->st));
     MCK(cudaMemcpyAsync(lo0, hlo.data(), sizeof(float) * hlo.size(), cudaMemcpyHostToDevice, m->st));
     MCK(cudaStreamSynchronize(m->st));
