@@ -174,7 +174,7 @@ struct Ctx {
   bool shape_set = false;
   bool by_size = false;             // form 2 was set: the same as before any was, and reported
   int res_size = 0, res_block = 0;  // CTAs per cluster (0: none), trial threads
-  bool no_draws = false;            // no memory for the draws: not by default
+  bool no_draws = false;            // no memory for the draws
   bool cl_offer[5] = {};            // sizes vcsgc_cluster_sizes lists: cl_tiles of the five-shell table
   int pick_block = 0;               // BLOCKS, OVERLAP: trial threads of the one-CTA form (0: none)
   size_t pick_smem = 0;
@@ -998,12 +998,15 @@ int run_steps_resident(Ctx* c, long long n, int csize, int block) {
 // fewest steps of one call that pay for loading the lattice into shared memory
 constexpr long long RESIDENT_MIN_STEPS = 8;
 
-// whether a call of the default form can run resident: the draws' buffers are
-// there (without memory for them the context goes on with a launch per step)
-// and the caller is not capturing the stream, which takes no allocation
+// whether a call can run resident: the draws' buffers are there (without memory
+// for them the context goes on with a launch per step until a shape is set
+// again) and the caller is not capturing the stream, which takes no allocation
 bool resident_ready(Ctx* c, long long n) {
   if (c->no_draws || caller_captures(c)) return false;
-  if (draw_buffers(c, n) != VCSGC_OK) c->no_draws = true;
+  if (draw_buffers(c, n) != VCSGC_OK) {
+    c->no_draws = true;
+    c->err.clear();
+  }
   return !c->no_draws;
 }
 
@@ -1012,7 +1015,7 @@ bool resident_by_size(const Ctx* c) { return (c->res_size || c->pick_block) && !
 
 // whether a call of n steps runs resident, with the draws' buffers made
 bool runs_resident(Ctx* c, long long n) {
-  if (cluster_form_usable(c)) return true;
+  if (cluster_form_usable(c)) return resident_ready(c, n);
   return !c->shape_set && resident_by_size(c) && n >= RESIDENT_MIN_STEPS && resident_ready(c, n);
 }
 
@@ -1041,7 +1044,6 @@ int step_graph(Ctx* c) {
 
 // what a call of n steps allocates or instantiates, before it is timed
 int prepare_steps(Ctx* c, long long n) {
-  if (cluster_form_usable(c)) return draw_buffers(c, n);
   if (!runs_resident(c, n) && n >= STEP_GRAPH) return step_graph(c);
   return VCSGC_OK;
 }
@@ -2529,8 +2531,10 @@ int vcsgc_set_launch(void* ctx, int32_t form, int32_t block, int32_t variant) {
     c->cl_block = block;
     c->shape_set = true;
     c->by_size = false;
+    c->no_draws = false;
     return VCSGC_OK;
   }
+  if (f2) c->no_draws = false;
   c->form = 0;
   c->shape_set = !f2;
   c->by_size = f2;

@@ -53,11 +53,15 @@ def _agree(g, orcs):
             assert oo[k] == og[k], (r, k, oo[k], og[k])
 
 
-@pytest.mark.parametrize("kind", SCHED)
-def test_captured_steps_replay_after_resident_ones(V, kind):
+@pytest.mark.parametrize("kind,shape", [("sublattice", None), ("blocks", None), ("sublattice", (1, 256, 2))])
+def test_captured_steps_replay_after_resident_ones(V, kind, shape):
+    """In the default form, and in form 1 asked for: a capture takes the
+    per-step launch."""
     import torch
     s = torch.cuda.Stream()
     lat, tab, types, g = _context(V, kind, stream=s)
+    if shape:
+        g.set_launch(*shape)
     orcs = _oracles(kind, lat, tab, types)
     g.steps(23)  # resident
     graph = torch.cuda.CUDAGraph()
