@@ -64,7 +64,6 @@ void launch_multi_fixed(const double* V, int n_sh, int K, int qbits, long long* 
   k_multi_fixed<<<1, 256, 0, st>>>(V, n_sh, K, qbits, Dq);
 }
 
-// rho_i = sum_j f_{t_j}(r_ij)
 // A packed argument X = x << 2 | t: x = rho / h in fixed point (fx_bits fraction
 // bits) of species t's FP32 cubics, in range.  The argument of a density and a
 // shell's difference is within 2 2^-fx_bits intervals (two roundings, and the
@@ -79,7 +78,8 @@ __device__ __forceinline__ uint32_t fix_clamp(const MultiArgs& a, uint32_t X) {
   return X < a.fx_lo ? a.fx_lo : (X > a.fx_hi ? a.fx_hi : X);
 }
 // a site's entry; an argument out of range is stored as 0, which no shell's
-// difference brings into range
+// difference, added or taken (around the word's end), brings into range
+// (fixed_point.h)
 __device__ __forceinline__ uint2 fix_entry(const MultiArgs& a, int t, double rho) {
   const double v = rho * a.fx_scale;
   const uint32_t X = v > 0.0 && v < 1073741823.0 ? __double2uint_rn(v) << 2 | (uint32_t)t : 0u;
@@ -87,6 +87,7 @@ __device__ __forceinline__ uint2 fix_entry(const MultiArgs& a, int t, double rho
   return make_uint2(in ? X : (uint32_t)t, in ? __float_as_uint(fix_val(a, X)) : 0u);
 }
 
+// rho_i = sum_j f_{t_j}(r_ij)
 __global__ void k_multi_rho(MultiArgs a, int r0) {
   const int r = r0 + blockIdx.y;
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;

@@ -8,6 +8,7 @@
 #include <string>
 #include <vector>
 
+#include "fixed_point.h"
 #include "kernels.h"
 #include "multi.cuh"
 #include "optional.h"
@@ -433,14 +434,10 @@ int screen_setup(Multi* m, const std::vector<double>& hFd) {
     a.tab_err = (float)((MK_BCC5_N + 1) * std::ldexp(dm, -20));
     return VCSGC_OK;
   }
-  // K > 2: fixed-point entries, where their rounding (2 2^-fx_bits intervals an
-  // evaluation) stays within the share of the bound that a float argument
-  // takes, 4 (j0 + 2) 2^-24 intervals from interval j0 up, and no difference
-  // reaches the range from zero
-  int bits = 23;
-  while (bits > 0 && (double)(n + 1) * std::ldexp(1.0, bits) > 1073741823.0) --bits;
-  const int j0 = std::max(0, (int)std::floor(lo / h) - 1);
-  if (m->K > 2 && std::ldexp(1.0, 25 - bits) <= 4.0 * (j0 + 2) && dmax < 0.999 * lo) {
+  // K > 2: fixed-point entries where a format fits these tables
+  const FixedFormat fx = m->K > 2 ? fixed_format(m->K, n, h, lo, hi, dmax) : FixedFormat{0, 0u, 0u};
+  if (fx.bits > 0) {
+    const int bits = fx.bits, j0 = std::max(0, (int)std::floor(lo / h) - 1);
     // their own bound of an evaluation: 6 2^-24 G as in screen.h (coefficients and
     // FMAs), and 2 2^-fx_bits intervals times the steepest slope
     double G = 0.0, Dm = 0.0;
@@ -453,8 +450,8 @@ int screen_setup(Multi* m, const std::vector<double>& hFd) {
     a.emb_err = (float)(std::min(err, std::ldexp(6.0 * G, -24) + std::ldexp(Dm, 1 - bits)) * (1.0 + 1e-6));
     a.fx_bits = bits;
     a.fx_scale = std::ldexp(1.0, bits) / h;
-    a.fx_lo = (uint32_t)std::ceil(lo * a.fx_scale) << 2;
-    a.fx_hi = (uint32_t)std::floor(hi * a.fx_scale) << 2 | (uint32_t)(m->K - 1);
+    a.fx_lo = fx.lo;
+    a.fx_hi = fx.hi;
     MTRY(malloc_dev(m, &a.ctab, (size_t)m->R * MK_CTAB));
     MTRY(malloc_dev(m, &a.rfu, (size_t)m->R * a.rf_n));
     std::vector<int> df((size_t)a.n_sh * m->K * m->K);
