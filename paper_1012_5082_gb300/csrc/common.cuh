@@ -250,10 +250,11 @@ __device__ __forceinline__ int locate_bits(double u, int n_int, double& t) {
 }
 
 // interval and offset of r on a table grid when 0 <= r < r_c <= the grid's
-// end is already known (no range test)
+// end is already known (no range test), or r is NaN (interval 0, t = NaN: the
+// conversion alone would give the most negative integer)
 __device__ __forceinline__ int locate_u(const Spline& s, double u, double& t) {
   if (s.n_int < (1 << 19)) return locate_bits(u, s.n_int, t);
-  int j = (int)u;
+  int j = not_finite(u) ? 0 : (int)u;
   j = j < s.n_int - 1 ? j : s.n_int - 1;
   t = u - (double)j;
   return j;
