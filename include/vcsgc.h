@@ -331,7 +331,8 @@ int vcsgc_profile_steps(void* ctx, int64_t n, double* ms_propose, double* ms_com
  *           the period-q sublattice schedule, the five-shell BCC table, one
  *           density function and no surrogate; vcsgc_cluster_sizes lists
  *           the sizes these lattices allow.
- *   form 2: calls of 8 steps or more run a resident form chosen by size where
+ *   form 2: calls of 8 steps or more (more where loading the lattice takes
+ *           longer than that pays) run a resident form chosen by size where
  *           one applies (form 1, also for the two-shell BCC table, or for the
  *           BLOCKS and OVERLAP schedules one block per replica with the whole
  *           lattice in shared memory); shorter calls, and calls where none

@@ -226,6 +226,8 @@ int cluster_capacity(const LatArgs& a, int csize, int block, size_t smem);
 // Needs a uniform dF and no pending commit.
 inline size_t pick_smem_bytes(long long words) { return sizeof(uint32_t) * ((size_t)words + 2); }
 constexpr size_t PICK_SMEM_MAX = 220 * 1024;
+// CTAs of that size an SM holds
+int pick_capacity(const LatArgs& a, int block, size_t smem);
 cudaError_t launch_pick_steps(const LatArgs& a, const ChainDraws& cd, size_t smem, int block, int n,
                               cudaStream_t st);
 // true when the rows and masks of a equal the compile-time five-shell table

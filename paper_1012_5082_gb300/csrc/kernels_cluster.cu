@@ -1106,6 +1106,15 @@ int cluster_capacity(const LatArgs& a, int csize, int block, size_t smem) {
   return n;
 }
 
+int pick_capacity(const LatArgs& a, int block, size_t smem) {
+  int n = 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, pick_kernel(a, block), block, smem) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  return n;
+}
+
 cudaError_t launch_pick_steps(const LatArgs& a, const ChainDraws& cd, size_t smem, int block, int n, cudaStream_t st) {
   pick_kernel(a, block)<<<a.R, block, smem, st>>>(a, cd, n);
   return cudaGetLastError();

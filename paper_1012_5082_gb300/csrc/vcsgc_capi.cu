@@ -26,6 +26,9 @@ namespace {
 
 std::string g_init_error;
 
+// no resident call is shorter (resident_shape)
+constexpr long long RESIDENT_MIN_STEPS = 8;
+
 struct Ctx {
   std::string err;
   cudaStream_t st = nullptr;
@@ -174,6 +177,7 @@ struct Ctx {
   bool shape_set = false;
   bool by_size = false;             // form 2 was set: the same as before any was, and reported
   int res_size = 0, res_block = 0;  // CTAs per cluster (0: none), trial threads
+  long long res_min = 0;            // fewest steps of a call that runs so
   bool no_draws = false;            // no memory for the draws
   bool cl_offer[5] = {};            // sizes vcsgc_cluster_sizes lists: cl_tiles of the five-shell table
   int pick_block = 0;               // BLOCKS, OVERLAP: trial threads of the one-CTA form (0: none)
@@ -995,9 +999,6 @@ int run_steps_resident(Ctx* c, long long n, int csize, int block) {
   return VCSGC_OK;
 }
 
-// fewest steps of one call that pay for loading the lattice into shared memory
-constexpr long long RESIDENT_MIN_STEPS = 8;
-
 // whether a call can run resident: the draws' buffers are there (without memory
 // for them the context goes on with a launch per step until a shape is set
 // again) and the caller is not capturing the stream, which takes no allocation
@@ -1016,7 +1017,7 @@ bool resident_by_size(const Ctx* c) { return (c->res_size || c->pick_block) && !
 // whether a call of n steps runs resident, with the draws' buffers made
 bool runs_resident(Ctx* c, long long n) {
   if (cluster_form_usable(c)) return resident_ready(c, n);
-  return !c->shape_set && resident_by_size(c) && n >= RESIDENT_MIN_STEPS && resident_ready(c, n);
+  return !c->shape_set && resident_by_size(c) && n >= c->res_min && resident_ready(c, n);
 }
 
 // the graph of the per-step launch
@@ -1970,7 +1971,9 @@ static int lattice_state(Ctx* c, const std::vector<long long>& n0, const std::ve
   return check_device_error(c);
 }
 
-// The resident form a context runs until a launch shape is set, by size.
+// The resident form a context runs until a launch shape is set, by size, and the
+// fewest steps of a call that it pays for.
+//
 // SUBLATTICE: the largest cluster size that gives every CTA an SM of its own
 // with all R clusters resident, down to 32 groups of trials per CTA.  A step
 // costs about 1.3 us of fixed work (two barriers, the decision, the chain of
@@ -1981,29 +1984,84 @@ static int lattice_state(Ctx* c, const std::vector<long long>& n0, const std::ve
 // BLOCKS and OVERLAP: one CTA per replica while its step holds at most 1024
 // trials and the lattice fits in shared memory (10^3 cells, 1 trial per step:
 // 0.9 us against 2.8 per launch; 40^3, 64 trials: 1.4 against 6.5).
+//
+// More replicas than CTAs the GPU holds run in waves, each with the fixed work
+// of a step, while the per-step launch fills its blocks' warps: us per step of
+// both (resident / per-step, calls of 128 steps) 8^3 x 304 2.8 / 3.1, x 608 5.3 /
+// 3.2; 16^3 x 304 2.9 / 3.7, x 456 4.3 / 3.9; 24^3 x 456 5.2 / 5.1; 48^3 x 608 23 /
+// 37.  So a form in waves is taken where the costs below say it is faster.
+// A call also loads the lattice into shared memory and stores it back: 0.4 to 0.6
+// us per round of words of a tile (k_cluster_steps), 0.06 us (k_pick_steps, whose
+// rounds are many when few threads hold a large lattice).  us per step in calls
+// of 8: 128^3 x 1 5.5 / 5.0 (16 steps: 4.1 / 4.3), 80^3 in blocks of 20^3 11.3 / 4.0 (48
+// steps: 2.7 / 3.0).  Calls too short for that gain take the per-step launch.
 static void resident_shape(Ctx* c, const int* capacity) {
   const LatArgs& l = c->lat;
   c->res_size = c->res_block = c->pick_block = 0;
+  c->res_min = RESIDENT_MIN_STEPS;
   if (!l.df_uniform) return;
+  int n_sm = 0;
+  if (cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, c->device) != cudaSuccess) cudaGetLastError();
+  long long trials = 0, blocks = 0;  // of the per-step launch (128 threads a block)
+  for (const LatGeom& g : c->h_geom) {
+    trials += g.dmax;
+    blocks += (g.dmax + 127) / 128;
+  }
+  const auto min_steps = [](double call, double gain, long long most) {
+    const double n = gain > 0.0 ? std::ceil(call / gain) : (double)most;
+    return std::max(RESIDENT_MIN_STEPS, n < (double)most ? (long long)n : most);
+  };
+  constexpr long long LONG_CALL = 4096;
   if (l.sublattice) {
-    int n_sm = 0;
-    if (cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, c->device) != cudaSuccess) cudaGetLastError();
     const int gs = l.qx == 4 ? 4 : 1;
+    int groups = 0, q = -1;
     for (int qi = 0; qi < 5; ++qi) {
       if (!c->cl_tiles[qi]) continue;
-      const int s = 1 << qi, groups = c->cl_lcap[qi] / gs;
-      if (s > 1 && (capacity[qi] < c->R || (long long)c->R * s > n_sm || groups < 32)) continue;
-      c->res_size = s;
-      c->res_block = groups > 256 ? 512 : 256;
+      const int s = 1 << qi, gq = c->cl_lcap[qi] / gs;
+      if (s > 1 && (capacity[qi] < c->R || (long long)c->R * s > n_sm || gq < 32)) continue;
+      q = qi;
+      groups = gq;
     }
+    if (q < 0) return;
+    const int block = groups > 256 ? 512 : 256;
+    const int held = std::max(1, capacity[0]), waves = q == 0 ? (c->R + held - 1) / held : 1;
+    const double rounds = (double)(c->cl_smem[q] / sizeof(uint32_t)) / (block + 32);
+    // us per step of the per-step launch, six blocks to an SM and more, and of
+    // this one
+    const bool full = blocks > 6LL * n_sm;
+    double per_step = full ? 3.5 + 3.9e-3 * (double)blocks : 3.1 + 1.5e-3 * (double)blocks;
+    if (!l.bcc5) per_step += 1.3;
+    double step = groups <= 256 ? 1.2 + 2.9e-3 * groups : 2.75 + 5.5e-3 * std::max(0, groups - 512);
+    double call = 3.0 + 0.4 * rounds;
+    if (waves > 1) {
+      if (!full) per_step = std::max(per_step, 3.1 + 2.4e-5 * (double)trials);
+      step = 1.3 * waves + (gs == 4 ? 6e-3 : 2.5e-3) * groups * c->R / held;
+      if (step > 0.95 * per_step) return;
+      call = waves * (4.0 + 0.6 * rounds);
+    }
+    c->res_size = 1 << q;
+    c->res_block = block;
+    // (32 steps pay for a single wave whatever its size)
+    c->res_min = min_steps(call, per_step - step, waves > 1 ? LONG_CALL : 32);
     return;
   }
   // site picks: the whole replica in one CTA
   const size_t smem = pick_smem_bytes(c->max_words);
-  if (c->R >= 1 && c->subs.empty() && l.dmax <= 1024 && smem <= PICK_SMEM_MAX) {
-    c->pick_smem = smem;
-    c->pick_block = std::min(512, (l.dmax + 31) / 32 * 32);
+  if (c->R < 1 || !c->subs.empty() || l.dmax > 1024 || smem > PICK_SMEM_MAX) return;
+  const int block = std::min(512, (l.dmax + 31) / 32 * 32);
+  const int held = std::max(1, pick_capacity(l, block, smem)) * std::max(1, n_sm);
+  const int waves = (c->R + held - 1) / held;
+  double gain = (l.dmax <= 8 ? 1.4 : (l.dmax <= 32 ? 2.0 : 2.8)) + (l.bcc5 ? 0.0 : 2.5);
+  if (waves > 1) {
+    const double per_step = 2.4 + std::max(3.3e-3 * (double)blocks, 1e-4 * (double)trials);
+    const double step = waves * (1.3 + 2.7e-3 * l.dmax);
+    if (step > 0.9 * per_step) return;
+    gain = per_step - step;
   }
+  c->pick_smem = smem;
+  c->pick_block = block;
+  // (loads of every SM at once take twice as long)
+  c->res_min = min_steps(waves * (2.0 + 0.06 * (double)c->max_words / block) * (c->R >= n_sm ? 2.0 : 1.0), gain, LONG_CALL);
 }
 
 // Tilings of the cluster-resident form.  For each cluster size s in 1, 2,
@@ -2316,7 +2374,7 @@ int vcsgc_autotune(void* ctx, int64_t steps, int32_t* best_block) {
     float ms = 0.0f;
     CK(cudaEventElapsedTime(&ms, e0, e1));
     // (timed over fewer steps than run resident, it is the fastest of form 0)
-    const bool tie = cb[0] == 2 && steps < RESIDENT_MIN_STEPS;
+    const bool tie = cb[0] == 2 && steps < c->res_min;
     if (best == 0.0f || ms < lead * best || tie) {
       best = tie ? std::min(best, ms) : ms;
       bc = cb;

@@ -563,7 +563,8 @@ class Context:
         """Launch shape of the fused colour step (vcsgc_set_launch): form 0
         with variant = row prefetch, form 1 with variant = CTAs per cluster,
         form 2 (as before any shape is set) resident by size for calls of 8
-        steps and more, with block and variant as form 0 for shorter ones."""
+        steps and more (more on some lattices), with block and variant as form
+        0 for shorter ones."""
         _check(lib().vcsgc_set_launch(self.h, int(form), int(block), int(variant)), self.h)
 
     def set_schedule(self, kind, sched):

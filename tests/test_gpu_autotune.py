@@ -98,3 +98,25 @@ def test_profiled_steps_hold_no_allocation(V, shape):
     assert first[1] == 0.0 and all(q[1] == 0.0 for q in later)  # one launch of many steps: no commits
     assert first[0] < 1.6 * np.median([q[0] for q in later]), (first, later)
     g.close()
+
+
+@pytest.mark.parametrize("kind,cells,sched,R", [
+    ("blocks", (80, 80, 40), (20, 20, 20, 2, 2, 2), 2),   # a large lattice on few threads: pays from some 30 steps up
+    ("sublattice", (8, 8, 8), (4, 4, 4), 200),            # two waves of CTAs: from about 10
+    ("sublattice", (8, 8, 8), (4, 4, 4), 500),            # four: never
+    ("sublattice", (24, 24, 24), (4, 4, 4), 700),         # five full ones: again
+    ("blocks", (10, 10, 10), (5, 5, 5, 2, 2, 2), 5000),   # more CTAs than the GPU holds
+])
+def test_calls_of_any_length_are_one_chain(V, kind, cells, sched, R):
+    """Lengths on both sides of the shortest call that runs resident, by size."""
+    g, h = (_context(V, kind, cells, sched, "eam", R=R) for _ in range(2))
+    h.set_launch(0, 128, 1)
+    lengths = (8, 9, 11, 13, 20, 27, 31, 40, 64, 8)
+    for n in lengths:
+        g.steps(n)
+    h.steps(sum(lengths))
+    assert np.array_equal(g.types_all(), h.types_all())
+    for og, oh in zip(g.observables_all(), h.observables_all()):
+        assert [og[k] for k in COUNTERS] == [oh[k] for k in COUNTERS]
+    g.close()
+    h.close()

@@ -27,7 +27,7 @@ def _run(V, k, out):
     try:
         g = _context(V, *SIZES[k], seed=k + 1)
         for _ in range(1500):
-            g.steps(9)
+            g.steps(64)
         out[k] = (g.types(), g.observables()["flips"])
         g.close()
     except Exception as e:  # reported by the test
