@@ -87,6 +87,25 @@ __device__ __forceinline__ uint2 fix_entry(const MultiArgs& a, int t, double rho
   return make_uint2(in ? X : (uint32_t)t, in ? __float_as_uint(fix_val(a, X)) : 0u);
 }
 
+// entry i of a.rf from site i's density and species
+__device__ __forceinline__ void rf_entry(const MultiArgs& a, int r, long long i, int t, double rho) {
+  const float r32 = (float)rho;
+  const int3 h = multi_half(a, (int)i);
+  const int b = (int)(i & 1);
+  a.rf[(long long)r * a.rf_n + multi_rfi(a, (h.x - b) >> 1, (h.y - b) >> 1, (h.z - b) >> 1, b)] =
+      make_float2(r32, emb32_val(a, t, r32));
+}
+
+__global__ void k_multi_rf(MultiArgs a) {
+  const int r = blockIdx.y;
+  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < a.N) rf_entry(a, r, i, a.types[(long long)r * a.N + i], a.rho[(long long)r * a.N + i]);
+}
+
+void launch_multi_rf(const MultiArgs& a, cudaStream_t st) {
+  k_multi_rf<<<dim3((unsigned)((a.N + 255) / 256), (unsigned)a.R), 256, 0, st>>>(a);
+}
+
 // rho_i = sum_j f_{t_j}(r_ij)
 __global__ void k_multi_rho(MultiArgs a, int r0) {
   const int r = r0 + blockIdx.y;
@@ -104,13 +123,7 @@ __global__ void k_multi_rho(MultiArgs a, int r0) {
     const int b = (int)(i & 1);
     a.rfu[(long long)r * a.rf_n + multi_rfi(a, (h.x - b) >> 1, (h.y - b) >> 1, (h.z - b) >> 1, b)] = fix_entry(a, ty[i], rho);
   }
-  if (a.rf) {
-    const float r32 = (float)rho;
-    const int3 h = multi_half(a, (int)i);
-    const int b = (int)(i & 1);
-    a.rf[(long long)r * a.rf_n + multi_rfi(a, (h.x - b) >> 1, (h.y - b) >> 1, (h.z - b) >> 1, b)] =
-        make_float2(r32, emb32_val(a, ty[i], r32));
-  }
+  if (a.rf) rf_entry(a, r, i, ty[i], rho);
 }
 
 void launch_multi_rho(const MultiArgs& a, int r0, int nrep, cudaStream_t st) {

@@ -272,6 +272,8 @@ void launch_multi_delta_e(const MultiArgs& a, int r, const long long* sites, con
 void launch_multi_nbc(const MultiArgs& a, int r0, int nrep, cudaStream_t st);
 // re-embedding table of replicas r0 ... from their rf and species
 void launch_multi_table(const MultiArgs& a, int r0, int nrep, cudaStream_t st);
+// float entries (rf) of every replica from its densities and species
+void launch_multi_rf(const MultiArgs& a, cudaStream_t st);
 void launch_multi_features(const MultiArgs& a, float* X, float* Y, cudaStream_t st);
 // one colour step (propose and commit); after_step: the previous launch on
 // the stream is this context's commit (the screened form then overlaps).

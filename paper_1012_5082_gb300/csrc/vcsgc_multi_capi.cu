@@ -54,6 +54,10 @@ struct Multi {
   // screened form: F_t at the middle of the reachable densities, the
   // offset of species t's FP32 embedding table
   std::vector<double> fref;
+  // K = 2, the re-embedding table (null: none) and the float entries, of which
+  // args holds the ones in use (use_table)
+  float* dtab = nullptr;
+  float2* rf = nullptr;
 };
 
 #define MCK(call)                                                                      \
@@ -307,6 +311,28 @@ void drop_graph(Multi* m) {
   m->graph = nullptr;
 }
 
+// K = 2: the colour steps read the re-embedding table, or the float entries
+// and the embedding cubics, from here on; the entries are filled from the
+// densities and species.  Without memory for the float entries the table stays.
+int use_table(Multi* m, bool on) {
+  MultiArgs& a = m->args;
+  if (!m->dtab || on == (a.dtab != nullptr)) return VCSGC_OK;
+  if (!on && !m->rf && !malloc_optional(m, {wanted(&m->rf, (size_t)m->R * a.rf_n)})) return VCSGC_OK;
+  a.dtab = on ? m->dtab : nullptr;
+  a.rf = on ? nullptr : m->rf;
+  if (on) {
+    launch_multi_nbc(a, 0, m->R, m->st);
+    launch_multi_table(a, 0, m->R, m->st);
+  } else {
+    launch_multi_rf(a, m->st);
+  }
+  m->nbc_stale = false;  // the table's commits have kept the counts
+  MCK(cudaGetLastError());
+  if (m->graph) MCK(cudaStreamSynchronize(m->st));
+  drop_graph(m);  // the captured steps hold the arguments by value
+  return VCSGC_OK;
+}
+
 void destroy(Multi* m) {
   if (!m) return;
   if (m->st) cudaStreamSynchronize(m->st);
@@ -427,6 +453,7 @@ int screen_setup(Multi* m, const std::vector<double>& hFd) {
     MCK(cudaMemcpyAsync(s4, hs4.data(), sizeof(float4) * hs4.size(), cudaMemcpyHostToDevice, m->st));
     MCK(cudaMemcpyAsync(lo0, hlo.data(), sizeof(float) * hlo.size(), cudaMemcpyHostToDevice, m->st));
     MCK(cudaStreamSynchronize(m->st));
+    m->dtab = a.dtab;
     a.emb_s = s4;
     a.emb_lo0 = lo0;
     a.fix_lo = (long long)std::ceil(lo / h * 4294967296.0);
@@ -874,6 +901,16 @@ int vcsgc_multi_set_surrogate(void* h, void* mlp) {
   a.mlp = mlp_view(m->sur);
   a.da = 1;
   drop_graph(m);  // the captured steps hold the arguments by value
+  return VCSGC_OK;
+}
+
+int vcsgc_multi_set_table(void* h, int32_t table) {
+  Multi* m = as_multi(h);
+  if (!m || table < 0 || table > 1) return VCSGC_ERR_INVALID_ARG;
+  MCK(cudaSetDevice(m->device));
+  if (!m->dtab) return mfail(m, VCSGC_ERR_STATE, "no re-embedding table (K = 2, species-dependent densities, memory)");
+  MTRY(use_table(m, table != 0));
+  if ((m->args.dtab != nullptr) != (table != 0)) return mfail(m, VCSGC_ERR_NOMEM, "no memory for the float entries");
   return VCSGC_OK;
 }
 

@@ -77,7 +77,7 @@ EXPORTS = ["vcsgc_default_options", "vcsgc_init", "vcsgc_steps", "vcsgc_sweep", 
            "vcsgc_multi_last_error", "vcsgc_multi_free", "vcsgc_set_ensemble", "vcsgc_md_state",
            "vcsgc_minimize", "vcsgc_save", "vcsgc_load", "vcsgc_set_launch", "vcsgc_get_launch",
            "vcsgc_philox", "vcsgc_cluster_sizes", "vcsgc_set_schedule", "vcsgc_autotune_schedule",
-           "vcsgc_multi_set_surrogate", "vcsgc_multi_features"]
+           "vcsgc_multi_set_surrogate", "vcsgc_multi_features", "vcsgc_multi_set_table"]
 
 
 def lib():
@@ -143,6 +143,7 @@ def lib():
             "vcsgc_multi_energy": (I32, [P, I32, P]),
             "vcsgc_multi_set_surrogate": (I32, [P, P]),
             "vcsgc_multi_features": (I32, [P, P, P]),
+            "vcsgc_multi_set_table": (I32, [P, I32]),
             "vcsgc_multi_last_error": (C.c_char_p, [P]),
             "vcsgc_multi_free": (None, [P]),
             "vcsgc_set_launch": (I32, [P, I32, I32, I32]),
@@ -800,6 +801,11 @@ class Multi:
         """Delayed acceptance (K = 2, species-dependent densities) with a copy
         of surrogate's weights (None: off); vcsgc_multi_set_surrogate."""
         self._chk(lib().vcsgc_multi_set_surrogate(self.h, None if surrogate is None else surrogate.h))
+
+    def set_table(self, table):
+        """Whether the steps of K = 2 with species-dependent densities read the
+        re-embedding table or the embedding cubics (vcsgc_multi_set_table)."""
+        self._chk(lib().vcsgc_multi_set_table(self.h, int(table)))
 
     def features(self):
         """(X [R N, 10], Y [R N]) CUDA float32 tensors of every site of every
