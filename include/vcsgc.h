@@ -624,10 +624,12 @@ int vcsgc_multi_set_surrogate(void* m, void* mlp);
 int vcsgc_multi_features(void* m, float* d_X, float* d_Y);
 /* K = 2 with species-dependent densities on the five-shell table: whether the
  * colour steps get the neighbours' re-embedding changes from a table of 44
- * bytes per site that the commits keep up to date (1; the default where it
- * takes at most a quarter of the free memory at creation) or from the
- * embedding cubics and 8 bytes per site (0).  The chain is the same.  Errors:
- * INVALID_ARG, STATE (a context without a table), NOMEM (for the 8 bytes). */
+ * bytes per site that the commits keep up to date (1; made where it takes at
+ * most a quarter of the free memory at creation) or from the embedding cubics
+ * and 8 bytes per site (0).  -1, the default: from the table while the calls
+ * before flipped less than about a thousand sites a step, over all replicas,
+ * else from the cubics.  The chain is the same.  Errors: INVALID_ARG, STATE (a
+ * context without a table), NOMEM (for the 8 bytes). */
 int vcsgc_multi_set_table(void* m, int32_t table);
 const char* vcsgc_multi_last_error(void* m);
 void vcsgc_multi_free(void* m);

@@ -58,6 +58,14 @@ struct Multi {
   // args holds the ones in use (use_table)
   float* dtab = nullptr;
   float2* rf = nullptr;
+  // which of them is in use follows the flips per step (table_policy) unless the
+  // caller has said: the replicas' flip counters, copied behind a stretch of
+  // steps and read once the copy is done
+  bool table_auto = true;
+  long long* flips = nullptr;   // pinned, [R]
+  cudaEvent_t flips_done = nullptr;
+  bool flips_asked = false;     // a copy is under way, of step flips_step
+  long long flips_step = 0, seen_step = 0, seen_flips = 0;
 };
 
 #define MCK(call)                                                                      \
@@ -249,6 +257,11 @@ int screen_acc_ready(Multi* m) {
   std::vector<MRepState> s(m->R);
   MCK(cudaMemcpyAsync(s.data(), m->args.rs, sizeof(MRepState) * m->R, cudaMemcpyDeviceToHost, m->st));
   MCK(cudaStreamSynchronize(m->st));
+  // the flips per step are counted from here (table_policy)
+  m->flips_asked = false;
+  m->seen_step = m->h_base;
+  m->seen_flips = 0;
+  for (const MRepState& q : s) m->seen_flips += q.flips;
   std::vector<MStepAcc> acc(m->R);
   for (int r = 0; r < m->R; ++r) {
     acc[r] = MStepAcc{};
@@ -269,8 +282,69 @@ int screen_acc_ready(Multi* m) {
   return VCSGC_OK;
 }
 
+// The re-embedding table saves a trial its 58 cubics and costs a flip the refresh
+// of 59 sites' eleven entries (scattered over 44 bytes per site), so it loses
+// where many trials flip: us per step, table / cubics, 80^3 x 8 with 550, 890, 1650,
+// 3000, 13,800 flips a step 7 / 20, 21 / 25, 28 / 26, 51 / 29, 233 / 58; 48^3 x 8 with 360,
+// 650, 1640 19 / 21, 20 / 22, 30 / 25; 24^3 x 16 with 750, 2850 19 / 22, 44 / 30.  The
+// break-even is 900 to 1500 flips a step whatever the lattice.  The form changes
+// between calls, by the flips per step since the last look, beyond either side.
+constexpr double TABLE_MOST_FLIPS = 1400.0, TABLE_FEW_FLIPS = 700.0;
+constexpr long long TABLE_LOOK_STEPS = 256;  // fewest steps between two looks
+
+int use_table(Multi* m, bool on);
+
+bool caller_captures(Multi* m) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(m->st, &cap) != cudaSuccess) cudaGetLastError();
+  return cap != cudaStreamCaptureStatusNone;
+}
+
+// takes in the counters asked for, if they have come, and changes the form
+int table_policy(Multi* m) {
+  if (!m->flips_asked || caller_captures(m)) return VCSGC_OK;
+  const cudaError_t e = cudaEventQuery(m->flips_done);
+  if (e == cudaErrorNotReady) {
+    cudaGetLastError();
+    return VCSGC_OK;
+  }
+  MCK(e);
+  m->flips_asked = false;
+  long long now = 0;
+  for (int r = 0; r < m->R; ++r) now += m->flips[r];
+  const long long steps = m->flips_step - m->seen_step, flips = now - m->seen_flips;
+  m->seen_step = m->flips_step;
+  m->seen_flips = now;
+  if (steps <= 0 || flips < 0) return VCSGC_OK;
+  const double rate = (double)flips / (double)steps;
+  if (m->args.dtab && rate > TABLE_MOST_FLIPS) return use_table(m, false);
+  if (!m->args.dtab && rate < TABLE_FEW_FLIPS) return use_table(m, true);
+  return VCSGC_OK;
+}
+
+// asks for the counters behind the steps launched so far
+int ask_flips(Multi* m) {
+  if (m->flips_asked || m->h_base - m->seen_step < TABLE_LOOK_STEPS || caller_captures(m)) return VCSGC_OK;
+  if (!m->flips) {
+    if (cudaMallocHost(&m->flips, sizeof(long long) * m->R) != cudaSuccess ||
+        cudaEventCreateWithFlags(&m->flips_done, cudaEventDisableTiming) != cudaSuccess) {
+      cudaGetLastError();
+      m->table_auto = false;  // the form stays
+      return VCSGC_OK;
+    }
+  }
+  MCK(cudaMemcpy2DAsync(m->flips, sizeof(long long), &m->args.rs->flips, sizeof(MRepState), sizeof(long long), m->R,
+                        cudaMemcpyDeviceToHost, m->st));
+  MCK(cudaEventRecord(m->flips_done, m->st));
+  m->flips_asked = true;
+  m->flips_step = m->h_base;
+  return VCSGC_OK;
+}
+
 int run_steps(Multi* m, long long n) {
   if (m->args.fused) return run_steps_fused(m, n);
+  const bool look = m->dtab && m->table_auto && n > 0;
+  if (look) MTRY(table_policy(m));
   MTRY(screen_acc_ready(m));
   if (m->args.da) MTRY(nbc_fresh(m));
   // steps without delayed acceptance do not keep the counts
@@ -303,6 +377,7 @@ int run_steps(Multi* m, long long n) {
     m->h_base += n;
   }
   MCK(cudaGetLastError());
+  if (look) MTRY(ask_flips(m));
   return VCSGC_OK;
 }
 
@@ -337,6 +412,8 @@ void destroy(Multi* m) {
   if (!m) return;
   if (m->st) cudaStreamSynchronize(m->st);
   if (m->graph) cudaGraphExecDestroy(m->graph);
+  if (m->flips) cudaFreeHost(m->flips);
+  if (m->flips_done) cudaEventDestroy(m->flips_done);
   for (void* p : m->allocs) cudaFree(p);
   if (m->own_stream && m->st) cudaStreamDestroy(m->st);
   delete m;
@@ -906,9 +983,11 @@ int vcsgc_multi_set_surrogate(void* h, void* mlp) {
 
 int vcsgc_multi_set_table(void* h, int32_t table) {
   Multi* m = as_multi(h);
-  if (!m || table < 0 || table > 1) return VCSGC_ERR_INVALID_ARG;
+  if (!m || table < -1 || table > 1) return VCSGC_ERR_INVALID_ARG;
   MCK(cudaSetDevice(m->device));
   if (!m->dtab) return mfail(m, VCSGC_ERR_STATE, "no re-embedding table (K = 2, species-dependent densities, memory)");
+  m->table_auto = table < 0;
+  if (table < 0) return VCSGC_OK;
   MTRY(use_table(m, table != 0));
   if ((m->args.dtab != nullptr) != (table != 0)) return mfail(m, VCSGC_ERR_NOMEM, "no memory for the float entries");
   return VCSGC_OK;

@@ -804,7 +804,8 @@ class Multi:
 
     def set_table(self, table):
         """Whether the steps of K = 2 with species-dependent densities read the
-        re-embedding table or the embedding cubics (vcsgc_multi_set_table)."""
+        re-embedding table (1), the embedding cubics (0) or what the flips per
+        step call for (-1, the default); vcsgc_multi_set_table."""
         self._chk(lib().vcsgc_multi_set_table(self.h, int(table)))
 
     def features(self):

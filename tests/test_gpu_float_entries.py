@@ -140,3 +140,37 @@ def test_more_species_without_a_fixed_point_format(V, K, ds, phi, cells, period,
         _agree(g, orcs)
     assert sum(g.observables(r)["flips"] for r in range(R)) > 0
     g.close()
+
+
+def test_the_form_follows_the_flips(V):
+    """A hot chain flips thousands of sites a step and runs from the cubics after
+    its first calls.  It is the chain of the table alone, and the time per step
+    says which form ran: with 48^3 x 8 hot the table takes more than twice the
+    cubics' time."""
+    import time
+
+    import torch
+    tab = I.eam_tables(I.multi_eam_params(2, dens_scale=(1.0, 1.25)))
+    lat = I.bcc_lattice(48, 48, 48)
+    R = 8
+    types = np.stack([I.multi_random_types(lat.n, [lat.n // 3], seed=r) for r in range(R)])
+
+    def chain(table):
+        g = V.Multi(lat, types, tab, [-1.5], 0.0, 20000.0, c0=0.3, seed_r=np.arange(R, dtype=np.uint64))
+        if table is not None:
+            g.set_table(table)
+        us = []
+        for _ in range(6):
+            torch.cuda.synchronize()
+            t0 = time.perf_counter()
+            g.steps(256)
+            o = g.observables(0)
+            us.append((time.perf_counter() - t0) / 256 * 1e6)
+        out = [g.types(r) for r in range(R)], o["flips"], o["local_accepts"]
+        g.close()
+        return out, us
+
+    (ta, fa, la), hot = chain(None)
+    (tb, fb, lb), fixed = chain(1)
+    assert fa == fb > 256 * 6 * 1000 and la == lb and all(np.array_equal(x, y) for x, y in zip(ta, tb))
+    assert min(hot[2:]) < 0.7 * min(fixed[2:]), (hot, fixed)
