@@ -285,11 +285,13 @@ int screen_acc_ready(Multi* m) {
 // The re-embedding table saves a trial its 58 cubics and costs a flip the refresh
 // of 59 sites' eleven entries (scattered over 44 bytes per site), so it loses
 // where many trials flip: us per step, table / cubics, 80^3 x 8 with 550, 890, 1650,
-// 3000, 13,800 flips a step 7 / 20, 21 / 25, 28 / 26, 51 / 29, 233 / 58; 48^3 x 8 with 360,
-// 650, 1640 19 / 21, 20 / 22, 30 / 25; 24^3 x 16 with 750, 2850 19 / 22, 44 / 30.  The
-// break-even is 900 to 1500 flips a step whatever the lattice.  The form changes
-// between calls, by the flips per step since the last look, beyond either side.
-constexpr double TABLE_MOST_FLIPS = 1400.0, TABLE_FEW_FLIPS = 700.0;
+// 3000, 13,800 flips a step 7 / 20, 22 / 25, 30 / 26, 47 / 30, 93 / 54; 64^3 x 8 with 840,
+// 1550, 3900 22 / 23, 27 / 24, 41 / 31; and with tables that the L2 holds, 64^3 x 4
+// with 1900, 3500, 13,500 23 / 26, 28 / 29, 64 / 43, 80^3 x 1 with 1700, 6600 20 / 25, 35 /
+// 32.  The form changes between calls, by the flips per step since the last look,
+// beyond the break-even and below half of it.
+constexpr double TABLE_MOST_FLIPS = 1200.0, TABLE_MOST_FLIPS_L2 = 4000.0;
+constexpr size_t TABLE_L2_BYTES = 100u << 20;
 constexpr long long TABLE_LOOK_STEPS = 256;  // fewest steps between two looks
 
 int use_table(Multi* m, bool on);
@@ -317,8 +319,10 @@ int table_policy(Multi* m) {
   m->seen_flips = now;
   if (steps <= 0 || flips < 0) return VCSGC_OK;
   const double rate = (double)flips / (double)steps;
-  if (m->args.dtab && rate > TABLE_MOST_FLIPS) return use_table(m, false);
-  if (!m->args.dtab && rate < TABLE_FEW_FLIPS) return use_table(m, true);
+  const size_t bytes = sizeof(float) * (size_t)m->R * DTAB_PLANES * m->args.rf_n;
+  const double most = bytes <= TABLE_L2_BYTES ? TABLE_MOST_FLIPS_L2 : TABLE_MOST_FLIPS;
+  if (m->args.dtab && rate > most) return use_table(m, false);
+  if (!m->args.dtab && rate < 0.5 * most) return use_table(m, true);
   return VCSGC_OK;
 }
 

@@ -143,15 +143,15 @@ def test_more_species_without_a_fixed_point_format(V, K, ds, phi, cells, period,
 
 
 def test_the_form_follows_the_flips(V):
-    """A hot chain flips thousands of sites a step and runs from the cubics after
-    its first calls.  It is the chain of the table alone, and the time per step
-    says which form ran: with 48^3 x 8 hot the table takes more than twice the
-    cubics' time."""
+    """A hot chain flips tens of thousands of sites a step and runs from the cubics
+    after its first calls.  It is the chain of the table alone, and the time per
+    step says which form ran: hot, 64^3 x 8 takes 119 us with the table and 65
+    from the cubics."""
     import time
 
     import torch
     tab = I.eam_tables(I.multi_eam_params(2, dens_scale=(1.0, 1.25)))
-    lat = I.bcc_lattice(48, 48, 48)
+    lat = I.bcc_lattice(64, 64, 64)
     R = 8
     types = np.stack([I.multi_random_types(lat.n, [lat.n // 3], seed=r) for r in range(R)])
 
@@ -173,4 +173,4 @@ def test_the_form_follows_the_flips(V):
     (ta, fa, la), hot = chain(None)
     (tb, fb, lb), fixed = chain(1)
     assert fa == fb > 256 * 6 * 1000 and la == lb and all(np.array_equal(x, y) for x, y in zip(ta, tb))
-    assert min(hot[2:]) < 0.7 * min(fixed[2:]), (hot, fixed)
+    assert min(hot[2:]) < 0.75 * min(fixed[2:]), (hot, fixed)
