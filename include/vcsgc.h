@@ -335,8 +335,10 @@ int vcsgc_profile_steps(void* ctx, int64_t n, double* ms_propose, double* ms_com
  *           longer than that pays) run a resident form chosen by size where
  *           one applies (form 1, also for the two-shell BCC table, or for the
  *           BLOCKS and OVERLAP schedules one block per replica with the whole
- *           lattice in shared memory); shorter calls, and calls where none
- *           applies, run form 0 with this `block` and `variant`.
+ *           lattice in shared memory); shorter calls, calls where none
+ *           applies, and later calls of chains that accept so many steps
+ *           that it is the slower one, run form 0 with this `block` and
+ *           `variant`.
  * Until a shape is set a context runs as in form 2, and vcsgc_get_launch reports
  * the shape of the per-step launch (form 0) that its shorter calls use.
  * vcsgc_autotune picks a shape by timing; this call sets one explicitly.

@@ -178,6 +178,16 @@ struct Ctx {
   bool by_size = false;             // form 2 was set: the same as before any was, and reported
   int res_size = 0, res_block = 0;  // CTAs per cluster (0: none), trial threads
   long long res_min = 0;            // fewest steps of a call that runs so
+  // An accepted step is proposed twice there: above this share of accepted steps
+  // the per-step launch is the faster one (1 and more: never), and calls take it
+  // (res_off).  The replicas' states are copied behind a stretch of steps and
+  // read once the copy is done (accept_policy).
+  double res_accept = 1.0;
+  bool res_off = false;
+  RepState* look = nullptr;         // pinned, [R]
+  cudaEvent_t look_done = nullptr;
+  bool look_asked = false;
+  long long look_base = 0, seen_steps = 0, seen_accepts = 0;  // seen_steps < 0: not known
   bool no_draws = false;            // no memory for the draws
   bool cl_offer[5] = {};            // sizes vcsgc_cluster_sizes lists: cl_tiles of the five-shell table
   int pick_block = 0;               // BLOCKS, OVERLAP: trial threads of the one-CTA form (0: none)
@@ -1017,7 +1027,52 @@ bool resident_by_size(const Ctx* c) { return (c->res_size || c->pick_block) && !
 // whether a call of n steps runs resident, with the draws' buffers made
 bool runs_resident(Ctx* c, long long n) {
   if (cluster_form_usable(c)) return resident_ready(c, n);
-  return !c->shape_set && resident_by_size(c) && n >= c->res_min && resident_ready(c, n);
+  return !c->shape_set && resident_by_size(c) && !c->res_off && n >= c->res_min && resident_ready(c, n);
+}
+
+constexpr long long LOOK_STEPS = 256;  // fewest steps between two looks
+
+// takes in the states asked for, if they have come, and changes the form
+int accept_policy(Ctx* c) {
+  if (!c->look_asked || caller_captures(c)) return VCSGC_OK;
+  const cudaError_t e = cudaEventQuery(c->look_done);
+  if (e == cudaErrorNotReady) {
+    cudaGetLastError();
+    return VCSGC_OK;
+  }
+  CK(e);
+  c->look_asked = false;
+  long long steps = 0, accepts = 0;
+  for (int r = 0; r < c->R; ++r) {
+    steps += c->look[r].steps;
+    accepts += c->look[r].global_acc;
+  }
+  const long long ds = steps - c->seen_steps, da = accepts - c->seen_accepts;
+  const bool known = c->seen_steps >= 0 && ds > 0 && da >= 0;
+  c->seen_steps = steps;
+  c->seen_accepts = accepts;
+  if (!known) return VCSGC_OK;
+  const double share = (double)da / (double)ds;
+  if (share > c->res_accept) c->res_off = true;
+  else if (share < 0.85 * c->res_accept) c->res_off = false;
+  return VCSGC_OK;
+}
+
+// asks for the states behind the steps launched so far
+int ask_states(Ctx* c) {
+  if (c->look_asked || (c->seen_steps >= 0 && c->h_base - c->look_base < LOOK_STEPS) || caller_captures(c))
+    return VCSGC_OK;
+  if (!c->look && (cudaMallocHost(&c->look, sizeof(RepState) * c->R) != cudaSuccess ||
+                   cudaEventCreateWithFlags(&c->look_done, cudaEventDisableTiming) != cudaSuccess)) {
+    cudaGetLastError();
+    c->res_accept = 1.0;  // the form stays
+    return VCSGC_OK;
+  }
+  CK(cudaMemcpyAsync(c->look, c->rs, sizeof(RepState) * c->R, cudaMemcpyDeviceToHost, c->st));
+  CK(cudaEventRecord(c->look_done, c->st));
+  c->look_asked = true;
+  c->look_base = c->h_base;
+  return VCSGC_OK;
 }
 
 // the graph of the per-step launch
@@ -1049,7 +1104,17 @@ int prepare_steps(Ctx* c, long long n) {
   return VCSGC_OK;
 }
 
+int launch_steps_fast(Ctx* c, long long n);
+
 int run_steps_fast(Ctx* c, long long n) {
+  if (c->shape_set || !c->res_size || c->res_accept >= 1.0) return launch_steps_fast(c, n);
+  TRY(accept_policy(c));
+  if (c->seen_steps < 0) TRY(ask_states(c));  // where a loaded chain starts
+  TRY(launch_steps_fast(c, n));
+  return ask_states(c);
+}
+
+int launch_steps_fast(Ctx* c, long long n) {
   if (runs_resident(c, n)) {
     if (cluster_form_usable(c)) return run_steps_resident(c, n, c->cl_size, c->cl_block);
     if (c->res_size) return run_steps_resident(c, n, c->res_size, c->res_block);
@@ -1999,6 +2064,8 @@ static void resident_shape(Ctx* c, const int* capacity) {
   const LatArgs& l = c->lat;
   c->res_size = c->res_block = c->pick_block = 0;
   c->res_min = RESIDENT_MIN_STEPS;
+  c->res_accept = 1.0;
+  c->res_off = false;
   if (!l.df_uniform) return;
   int n_sm = 0;
   if (cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, c->device) != cudaSuccess) cudaGetLastError();
@@ -2031,7 +2098,8 @@ static void resident_shape(Ctx* c, const int* capacity) {
     const bool full = blocks > 6LL * n_sm;
     double per_step = full ? 3.5 + 3.9e-3 * (double)blocks : 3.1 + 1.5e-3 * (double)blocks;
     if (!l.bcc5) per_step += 1.3;
-    double step = groups <= 256 ? 1.2 + 2.9e-3 * groups : 2.75 + 5.5e-3 * std::max(0, groups - 512);
+    double step = gs == 1 ? 1.0 + 2.3e-3 * groups
+                          : (groups <= 256 ? 1.2 + 2.9e-3 * groups : 2.75 + 5.5e-3 * std::max(0, groups - 512));
     double call = 3.0 + 0.4 * rounds;
     if (waves > 1) {
       if (!full) per_step = std::max(per_step, 3.1 + 2.4e-5 * (double)trials);
@@ -2041,6 +2109,12 @@ static void resident_shape(Ctx* c, const int* capacity) {
     }
     c->res_size = 1 << q;
     c->res_block = block;
+    // all steps accepted: 2.15 of a rejected one's time, the per-step launch 0.6
+    // us more (128^3, 1 replica: 2.6 / 3.5 -> 5.7 / 4.2; 100^3 x 8, period 5: 3.4 / 4.0 -> 7.4 /
+    // 4.7; 80^3 x 8: 1.9 / 3.9 -> 3.9 / 4.8); a fifth over the crossing, where both
+    // are within a few percent (128^3, 1 replica, 0.27 accepted: 3.1 / 3.3)
+    const double more = 1.15 * step - 0.6, lead = 1.2 * (per_step + (l.bcc5 ? 0.0 : 1.2) - step);
+    c->res_accept = more > 0.0 && lead < more ? std::max(0.1, lead / more) : 1.0;
     // (32 steps pay for a single wave whatever its size)
     c->res_min = min_steps(call, per_step - step, waves > 1 ? LONG_CALL : 32);
     return;
@@ -2164,6 +2238,8 @@ static void destroy(Ctx* c) {
   drop_graph(c);
   if (c->st) cudaStreamSynchronize(c->st);
   drop_draws(c, true);
+  if (c->look) cudaFreeHost(c->look);
+  if (c->look_done) cudaEventDestroy(c->look_done);
   if (c->h_pin) cudaFreeHost(c->h_pin);
   for (void* p : c->allocs) cudaFree(p);
   if (c->own_stream && c->st) cudaStreamDestroy(c->st);
@@ -2507,6 +2583,8 @@ static int snap_take(Ctx* c, Snap& s) {
 static int snap_restore(Ctx* c, const Snap& s) {
   TRY(flush(c));
   c->h_base = s.h_base;
+  c->look_asked = false;
+  c->seen_steps = -1;
   if (c->fast) {
     LatCtl ctl{s.h_base};
     CK(cudaMemcpyAsync(c->lat.ctl, &ctl, sizeof(LatCtl), cudaMemcpyHostToDevice, c->st));
@@ -3325,6 +3403,8 @@ int vcsgc_load(void* ctx, const char* path) {
   CK(cudaStreamSynchronize(c->st));
   // step base (fused form) first: the species upload writes n at its parity
   c->h_base = h_base;
+  c->look_asked = false;
+  c->seen_steps = -1;
   if (c->fast) {
     LatCtl ctl{h_base};
     CK(cudaMemcpyAsync(c->lat.ctl, &ctl, sizeof(LatCtl), cudaMemcpyHostToDevice, c->st));

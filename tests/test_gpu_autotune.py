@@ -120,3 +120,34 @@ def test_calls_of_any_length_are_one_chain(V, kind, cells, sched, R):
         assert [og[k] for k in COUNTERS] == [oh[k] for k in COUNTERS]
     g.close()
     h.close()
+
+
+def test_the_form_follows_the_accepts(V):
+    """One large lattice without the variance constraint, hot: every step is
+    accepted and takes 5.6 us resident, 4.1 by the per-step launch, which the
+    default form takes after its first calls.  One chain."""
+    import time
+
+    import torch
+    lat = I.bcc_lattice(112, 112, 112)
+    types = I.random_types(lat.n, lat.n // 3, seed=1)
+
+    def chain(shape):
+        g = V.Context(lat, types, I.eam_tables(), -2.1, 0.0, 5000.0, c0=0.3, seed=3)
+        if shape:
+            g.set_launch(*shape)
+        us = []
+        for _ in range(6):
+            torch.cuda.synchronize()
+            t0 = time.perf_counter()
+            g.steps(1000)
+            o = g.observables()
+            us.append((time.perf_counter() - t0) * 1e3)
+        out = g.types(), [o[k] for k in COUNTERS]
+        g.close()
+        return out, us
+
+    (ta, oa), follows = chain(None)
+    (tb, ob), resident = chain((1, 512, 16))
+    assert np.array_equal(ta, tb) and oa == ob and oa[3] > 0.9 * oa[0]
+    assert min(follows[2:]) < 0.85 * min(resident[2:]), (follows, resident)
