@@ -1069,18 +1069,18 @@ cudaError_t launch_chain_draws(const LatArgs& a, const ChainDraws& cd, int m, cu
 // Attributes belong to a kernel, not to a context: every context sets the same
 // largest size, so that none lowers it under another thread's launch.
 cudaError_t resident_attributes(const LatArgs& a) {
+  cudaError_t e = cudaSuccess;
   for (int block : {256, 512}) {
-    const ClusterKernel k = cluster_kernel(a, block);
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CL_SMEM_MAX);
-    if (e != cudaSuccess) return e;
+    if (a.sublattice) {
+      const ClusterKernel k = cluster_kernel(a, block);
+      if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+      if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CL_SMEM_MAX);
+    } else if (e == cudaSuccess) {
+      e = cudaFuncSetAttribute(pick_kernel(a, block == 256 ? 64 : 512), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               (int)PICK_SMEM_MAX);
+    }
   }
-  for (int block : {64, 512}) {
-    const cudaError_t e = cudaFuncSetAttribute(pick_kernel(a, block), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               (int)PICK_SMEM_MAX);
-    if (e != cudaSuccess) return e;
-  }
-  return cudaSuccess;
+  return e;
 }
 
 cudaError_t launch_cluster_steps(const LatArgs& a, const ClTile* d_tiles, const ChainDraws& cd, size_t smem, int csize,
