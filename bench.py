@@ -456,10 +456,9 @@ def timed_sweeps(torch, stream, b, sweeps, flush=None):
 def batch_bench(V, torch, stream, local, dmu0, sweeps=30, warmup=3, surrogate=True):
     """64 replicas of rigid BCC of uneven sizes (L = 24 + 4 (r mod 7) cells,
     27,648 to 221,184 sites) at 8 temperatures in 500-900 K x 8 phi values,
-    kappa = 1000, advanced together by one fused launch per colour step
-    (CUDA graphs of 64 steps); block size picked by the autotuner.  With
-    surrogate: the same run with delayed acceptance by a network trained on
-    the sampler's own dE."""
+    kappa = 1000, advanced together in the launch shape that the autotuner
+    keeps.  With surrogate: the same run with delayed acceptance by a network
+    trained on the sampler's own dE."""
     tab = I.eam_tables()
     b = c4_batch(V, stream, local, tab, dmu0)
     best = b.autotune(steps=64)
@@ -949,9 +948,10 @@ def main():
     reps = sampling(o_start, o_end, ms * 1e-3)
 
     # roofline of the dominant kernel: the fused colour step.  Its average time
-    # per colour step is the timed region over its steps (the graph's other
-    # nodes of the per-step form, the step-base advance and the colour table
-    # of the next 64 steps, add ~3 us per 64 launches, ~1 %).
+    # per colour step is the timed region over its steps (the per-step form's
+    # other graph nodes, the step-base advance and the colour table of the next
+    # 64 steps, add ~3 us per 64 launches, ~1 %; the resident form's draws are a
+    # launch of 45 us per 128 steps).
     avg_ms = ms_max / (args.steps * spw)
     trials_per_colour_step = N_PHI * (lat.n // 128)
     achieved = OPS_PER_TRIAL * trials_per_colour_step / (avg_ms * 1e-3) / 1e12
@@ -960,21 +960,29 @@ def main():
     hbm_ach = HBM_BYTES_PER_TRIAL * trials_per_colour_step / (avg_ms * 1e-3) / 1e9
     kname = ("k_lattice_step (one launch per colour step: commit of step k-1, site pick, dE from bit-packed "
              "shell counts, local test, dn reduction)" if launch[0] == 0 else
-             "k_cluster_steps (one thread-block cluster per replica, 128 colour steps per launch)")
+             "k_cluster_steps (one thread-block cluster per replica, 128 colour steps per launch; draws by "
+             "k_chain_draws)")
     roof = {"kernel": kname, "bound": "alu", "achieved": achieved, "peak": peak, "unit": "Tops/s",
             "frac": achieved / peak,
             "peak_source": (f"derived from measured per-SM rates (INT32 120, popc 20.7, multiply pairs 31, FP32 122, "
                             f"expf 11.3 per clock): the ALU pipe needs {SM_CYCLES_PER_TRIAL:.2f} SM cycles per trial "
                             f"({OPS_PER_TRIAL} algorithmic ops), x 152 SMs x 2.07 GHz"),
-            # DRAM bytes per launch from an ncu capture of the per-step kernel
-            # (256-thread blocks, warm L2, three launches of the timed loop);
-            # the cluster form is another kernel, not captured
-            "traffic": 255061 if launch[0] == 0 else None,
+            # DRAM bytes per launch from ncu captures of the timed loop (warm L2,
+            # three launches each)
+            "traffic": 255061 if launch[0] == 0 else 7543381,
             "traffic_source": ("ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum --cache-control none, "
                                "k_lattice_step<...,256,...> x 3 (launches 600-602): read 47,360 / 256 / 256 B, "
                                "write 252,672 / 250,368 / 214,272 B; the kernel's own reads are L2-resident, the "
                                "writes are write-backs of lines dirtied before it (the L2 flush between sweeps)"
-                               if launch[0] == 0 else None),
+                               if launch[0] == 0 else
+                               "ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum --cache-control none, "
+                               "k_cluster_steps x 3, 128 steps each: read 2,541,568 / 2,460,160 / 2,473,984 B (the "
+                               "bit rows), write 4,905,728 / 5,070,592 / 5,178,112 B (the rows back, and write-backs "
+                               "of the draws, which the launch before leaves in L2)"),
+            # thread instructions of the resident form's two kernels per trial (ncu,
+            # smsp__inst_executed.sum of 128 steps): byte sums count four trials at
+            # once, so it executes fewer than the algorithmic operations
+            "executed_per_trial": None if launch[0] == 0 else {"k_cluster_steps": 185, "k_chain_draws": 149},
             "ops_per_trial": {"simple_int": OPS_SIMPLE, "popc": OPS_POPC, "mul_pairs": OPS_MULPAIR,
                               "fp32": OPS_FP32, "mufu": OPS_MUFU},
             "trials_per_colour_step": trials_per_colour_step, "avg_colour_step_us": avg_ms * 1e3,

@@ -45,7 +45,7 @@
 // Measured, 80^3 x 8 replicas (64,000 trials per step): 2.3 us per step against
 // 4.2 for the per-step launch; what sizes it serves, and both sides there:
 // resident_shape in vcsgc_capi.cu.  Bound: the latency of one step's chain of
-// about 700 instructions per warp at two warps per scheduler (issue 35 %
+// about 700 instructions per warp at two warps per scheduler (issue 40 %
 // active), not a pipe.
 //
 // Every CTA of a cluster runs the same number of cluster barriers (the
@@ -263,7 +263,7 @@ __device__ __forceinline__ int sum_hi(int w) { return (w - sum_lo(w)) >> 16; }
 // replica's state once at the end: integers, but for the sums of c and c^2,
 // which grow a step at a time as in the per-step launch (an FP64 addition
 // each; c changes only with an accepted step, and its quotient is taken by the
-// reciprocal and one correction instead of a division).
+// reciprocal and one residual correction, q + (x - q N) / N, instead of a division).
 struct StepSums {
   long long trials = 0, local_acc = 0, flips = 0, dn = 0;
   int near_ties = 0, global_trials = 0, global_acc = 0;

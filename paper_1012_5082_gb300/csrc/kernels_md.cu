@@ -115,6 +115,8 @@ __global__ void __launch_bounds__(128) k_md_rho_half(MdArgs m) {
   if (live && sub == 0) atomicAdd(m.rho + i, rho);
 }
 
+// warp sum of the per-thread virial terms, one atomic per warp (every lane
+// of the warp reaches this point)
 __device__ __forceinline__ void add_virial(const MdArgs& m, double vir) {
   if (!m.vir) return;
 #pragma unroll
@@ -423,8 +425,6 @@ __global__ void k_md_embed(MdArgs m) {
   if (m.mixed) m.dFp32[i] = (float)m.dFp[i];
 }
 
-// warp sum of the per-thread virial terms, one atomic per warp (every lane
-// of the warp reaches this point)
 // FP64 forces on the half list: F_i += g (x_j - x_i) / r, F_j -= the same,
 // g = phi'_{ti tj} + F'_i f'_{tj} + F'_j f'_{ti} (one density derivative
 // when same_dens); force arrays zeroed before.  The virial term of the

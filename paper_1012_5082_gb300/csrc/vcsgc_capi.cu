@@ -2440,9 +2440,11 @@ int vcsgc_autotune(void* ctx, int64_t steps, int32_t* best_block) {
     if (cb[0] == 2) cb = {2, bc[1], bc[2]};
     if (vcsgc_set_launch(c, cb[0], cb[1], cb[2]) != VCSGC_OK) continue;
     // one untimed step with the candidate, then the timed ones, whose buffers
-    // and graph are made before
+    // and graph are made before; a resident run does not pay for the commit that
+    // a per-step one left
     TRY(run_steps_fast(c, 1));
     TRY(prepare_steps(c, steps));
+    TRY(flush(c));
     CK(cudaEventRecord(e0, c->st));
     TRY(run_steps_fast(c, steps));
     CK(cudaEventRecord(e1, c->st));
