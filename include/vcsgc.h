@@ -630,8 +630,10 @@ int vcsgc_multi_features(void* m, float* d_X, float* d_Y);
  * most a quarter of the free memory at creation) or from the embedding cubics
  * and 8 bytes per site (0).  -1, the default: from the table while the calls
  * before flipped less than about a thousand sites a step, over all replicas,
- * else from the cubics.  The chain is the same.  Errors: INVALID_ARG, STATE (a
- * context without a table), NOMEM (for the 8 bytes). */
+ * else from the cubics.  The chain is the same.  Steps captured into a CUDA
+ * graph hold the form of their capture: from then on it no longer follows the
+ * flips, and after a change by this call they must not be replayed.  Errors:
+ * INVALID_ARG, STATE (a context without a table), NOMEM (for the 8 bytes). */
 int vcsgc_multi_set_table(void* m, int32_t table);
 const char* vcsgc_multi_last_error(void* m);
 void vcsgc_multi_free(void* m);

@@ -304,7 +304,7 @@ bool caller_captures(Multi* m) {
 
 // takes in the counters asked for, if they have come, and changes the form
 int table_policy(Multi* m) {
-  if (!m->flips_asked || caller_captures(m)) return VCSGC_OK;
+  if (!m->flips_asked) return VCSGC_OK;
   const cudaError_t e = cudaEventQuery(m->flips_done);
   if (e == cudaErrorNotReady) {
     cudaGetLastError();
@@ -328,7 +328,7 @@ int table_policy(Multi* m) {
 
 // asks for the counters behind the steps launched so far
 int ask_flips(Multi* m) {
-  if (m->flips_asked || m->h_base - m->seen_step < TABLE_LOOK_STEPS || caller_captures(m)) return VCSGC_OK;
+  if (m->flips_asked || m->h_base - m->seen_step < TABLE_LOOK_STEPS) return VCSGC_OK;
   if (!m->flips) {
     if (cudaMallocHost(&m->flips, sizeof(long long) * m->R) != cudaSuccess ||
         cudaEventCreateWithFlags(&m->flips_done, cudaEventDisableTiming) != cudaSuccess) {
@@ -347,6 +347,9 @@ int ask_flips(Multi* m) {
 
 int run_steps(Multi* m, long long n) {
   if (m->args.fused) return run_steps_fused(m, n);
+  // captured steps hold the form they were captured in, which must stay: each
+  // form's commits keep its own entries only
+  if (m->dtab && m->table_auto && caller_captures(m)) m->table_auto = false;
   const bool look = m->dtab && m->table_auto && n > 0;
   if (look) MTRY(table_policy(m));
   MTRY(screen_acc_ready(m));

@@ -174,3 +174,40 @@ def test_the_form_follows_the_flips(V):
     (tb, fb, lb), fixed = chain(1)
     assert fa == fb > 256 * 6 * 1000 and la == lb and all(np.array_equal(x, y) for x, y in zip(ta, tb))
     assert min(hot[2:]) < 0.75 * min(fixed[2:]), (hot, fixed)
+
+
+def test_captured_steps_keep_their_form(V):
+    """Steps captured with the table and replayed among hot calls that would
+    change the form: the table's chain."""
+    import torch
+    tab = I.eam_tables(I.multi_eam_params(2, dens_scale=(1.0, 1.25)))
+    lat = I.bcc_lattice(48, 48, 48)
+    R = 8
+    types = np.stack([I.multi_random_types(lat.n, [lat.n // 3], seed=r) for r in range(R)])
+    s = torch.cuda.Stream()
+    args = (lat, types, tab, [-1.5], 0.0, 20000.0)
+    g = V.Multi(*args, c0=0.3, seed_r=np.arange(R, dtype=np.uint64), stream=s)
+    h = V.Multi(*args, c0=0.3, seed_r=np.arange(R, dtype=np.uint64))
+    h.set_table(1)
+    g.steps(2)
+    graph = torch.cuda.CUDAGraph()
+    s.synchronize()
+    with torch.cuda.graph(graph, stream=s, capture_error_mode="thread_local"):
+        g.steps(6)
+    n = 2
+    for _ in range(4):
+        with torch.cuda.stream(s):
+            graph.replay()
+        g.observables(0)
+        g.steps(256)
+        g.observables(0)
+        n += 6 + 256
+    with torch.cuda.stream(s):
+        graph.replay()
+    h.steps(n + 6)
+    for r in range(R):
+        assert np.array_equal(g.types(r), h.types(r))
+        assert g.observables(r)["flips"] == h.observables(r)["flips"] > n * 500
+    del graph
+    g.close()
+    h.close()
